@@ -84,9 +84,11 @@ typedef struct pa_opts {
                                 kernel with per-site threshold tables; 512 is their default); a
                                 lattice class that does not support the size takes its default;
                                 0 = library default */
-  int32_t threads_per_replica; /* threads sweeping one replica: cubic lattices 1, 2, 4 or 8 for
+  int32_t threads_per_replica; /* threads sharing a replica's sweep: cubic lattices 1, 2, 4 or 8 for
                                   +-1 couplings, 1, 2 or 4 for Gaussian ones (ranges of whole rows;
-                                  PA_ERR_INVALID where the rows do not split so); +-1 chains 1, 2,
+                                  PA_ERR_INVALID where the rows do not split so; the library
+                                  itself also takes 3, 5, 6, 7 or 12, and lets a thread sweep two
+                                  replicas side by side in large populations); +-1 chains 1, 2,
                                   4 or 8 (ranges of ceil(words / P) words); Gaussian chains and
                                   general boxes 1; 0 = library default */
 } pa_opts;

@@ -292,32 +292,23 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
   PA_CUDA(cudaEventCreate(&t1));
   int count = 0;
   for (auto& c : E.cls) {
-    // candidates: (block size, threads per replica); several threads per
-    // replica only for +-1 cubic lattices whose rows split evenly
-    std::vector<std::pair<int, int>> cands;
-    for (int split : {1, 2, 4, 8}) {
-      if (!split_supported(c, split)) continue;
-      for (int tpb : {32, 64, 128, 256, 512, 1024}) {
-        if (!tpb_supported(c, tpb)) continue;
-        if (split == 1 && tpb == 256) continue;
-        if (split > 1 && (tpb < 64 || tpb / split < 4)) continue;
-        cands.push_back({tpb, split});
-      }
-    }
     float best = 1e30f;
-    std::pair<int, int> pick = {c.tpb, c.split};
+    LaunchShape pick = {c.tpb, c.split, c.rp};
     LatticeClass trial = c;
-    for (const auto& cand : cands) {
-      trial.tpb = cand.first;
-      trial.split = cand.second;
+    for (const LaunchShape& cand : launch_shapes(c)) {
+      if (cand.split == 1 && cand.tpb == 256) continue;
+      trial.tpb = cand.tpb;
+      trial.split = cand.split;
+      trial.rp = cand.rp;
       trial.d_table = nullptr;
-      int st = build_class_table(E, trial);
+      int st = prepare_class_launch(E.d_runs, E.st, trial);
+      if (st == PA_OK) st = build_class_table(E, trial);
       if (st != PA_OK) return st;
-      st = launch_class(E, trial, trial.d_table, trial.nwork, false, trial.tpb);  // warm-up
+      st = launch_class(E, trial, trial.d_table, trial.nwork, false);  // warm-up
       if (st != PA_OK) return st;
       PA_CUDA(cudaEventRecord(t0, E.st));
       for (int rep = 0; rep < 2; ++rep) {
-        st = launch_class(E, trial, trial.d_table, trial.nwork, false, trial.tpb);
+        st = launch_class(E, trial, trial.d_table, trial.nwork, false);
         if (st != PA_OK) return st;
       }
       PA_CUDA(cudaEventRecord(t1, E.st));
@@ -330,10 +321,11 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
         pick = cand;
       }
     }
-    if (pick.first != c.tpb || pick.second != c.split) {
+    if (pick.tpb != c.tpb || pick.split != c.split || pick.rp != c.rp) {
       E.dfree(c.d_table, sizeof(Work) * std::max(c.nwork, 1));
-      c.tpb = pick.first;
-      c.split = pick.second;
+      c.tpb = pick.tpb;
+      c.split = pick.split;
+      c.rp = pick.rp;
       int st = build_class_table(E, c);
       if (st != PA_OK) return st;
     }

@@ -393,14 +393,53 @@ bool tpb_supported(const LatticeClass& c, int tpb) {
   return false;
 }
 
-// Block size and threads per replica of a class before any autotuning: the
-// cubic sweeps run 4 threads per replica where the rows split so, which keeps
-// enough warps resident to hide the latency of the generator's dependent
-// multiplies; +-1 chains 4 or 8 on ranges of words; other classes 1.
-void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt) {
+static bool pm_cubic(const LatticeClass& c) { return c.dim == 3 && c.bx == 0 && c.model == 0; }
+
+static cudaError_t sweep3d_call(int L, const Sweep3dLaunch& a) {
+  switch (L) {
+    case 2: return sweep3d_L2(a);
+    case 4: return sweep3d_L4(a);
+    case 6: return sweep3d_L6(a);
+    case 8: return sweep3d_L8(a);
+    case 10: return sweep3d_L10(a);
+    case 12: return sweep3d_L12(a);
+    case 14: return sweep3d_L14(a);
+    case 16: return sweep3d_L16(a);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+constexpr int NUM_SMS = 152;
+
+// Threads per replica of a +-1 cubic lattice before any autotuning: the most
+// that whole rows give, pairs of rows where a row's uniforms end within a
+// generator call (L = 6, 10, 14).  The sweep is bound by instruction issue,
+// so the finest split, which fills the schedulers most evenly, is the best or
+// within 3 % of it from 1e3 to 2e5 replicas; at L = 12 two rows a thread once
+// one row a thread makes several waves (4 % at 1e5).
+static int pm_split(int L, int64_t replicas) {
+  switch (L) {
+    case 2: return 1;
+    case 4: return 4;
+    case 12: return replicas > 50000 ? 6 : 12;
+    case 8: case 16: return 8;
+    default: return L / 2;
+  }
+}
+
+// Launch shape of a class of `replicas` slots (the sum of its runs' target
+// populations) before any autotuning.  Gaussian cubic sweeps run 4 threads
+// per replica where the rows split so, which keeps enough warps resident to
+// hide the latency of the generator's dependent multiplies (the
+// threshold-table kernel two of 512); +-1 chains 4 or 8 on ranges of words;
+// other classes 1.
+void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, int64_t replicas) {
   c.split = 1;
+  c.rp = 1;
   if (split_opt > 0) {
     c.split = split_supported(c, split_opt) ? split_opt : 1;
+  } else if (pm_cubic(c)) {
+    c.split = pm_split(c.L, replicas);
   } else if (c.dim == 3 && c.bx == 0 && c.model == 1 && c.L <= 8) {
     // the threshold-table kernel: 512 threads, two per replica (one block per
     // SM; measured the fastest shape for a single run of 1e5 replicas)
@@ -415,9 +454,30 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt) {
   if (tpb_opt && tpb_supported(c, tpb_opt)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
   else if (c.dim == 3 && c.model == 1 && c.L <= 8) c.tpb = 512;
-  else if (c.split > 1) c.tpb = (c.dim == 3 && c.L == 16) ? 64 : 128;
+  else if (pm_cubic(c)) c.tpb = c.L == 10 ? 256 : 128;  // 5 threads a replica leave 3 of 128 idle, 1 of 256
+  else if (c.split > 1) c.tpb = 128;
   else c.tpb = default_tpb(c.dim, c.L);
   if (c.tpb / c.split < 4 || (c.split > 1 && c.tpb < 64)) c.split = 1;
+  // Two replicas a thread share the lattice work of a word (6-15 % fewer
+  // instructions a flip) but halve the threads: taken once one replica a
+  // thread gives more than 900 threads an SM (28 warps; both are within 5 %
+  // of each other from 600 to 1200).
+  if (pm_cubic(c) && c.split > 1 && replicas * c.split > (int64_t)900 * NUM_SMS) c.rp = 2;
+}
+
+// Every launch shape the sweep kernel of a class has.
+std::vector<LaunchShape> launch_shapes(const LatticeClass& c) {
+  std::vector<LaunchShape> v;
+  for (int split : {1, 2, 3, 4, 5, 6, 7, 8, 12}) {
+    if (!split_supported(c, split)) continue;
+    for (int tpb : {32, 64, 128, 256, 512, 1024}) {
+      if (!tpb_supported(c, tpb)) continue;
+      if (split > 1 && (tpb < 64 || tpb / split < 4)) continue;
+      v.push_back({tpb, split, 1});
+      if (pm_cubic(c) && split > 1) v.push_back({tpb, split, 2});
+    }
+  }
+  return v;
 }
 
 bool split_supported(const LatticeClass& c, int split) {
@@ -446,9 +506,9 @@ bool split_supported(const LatticeClass& c, int split) {
   }
 }
 
-int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const Work* table, int nwork,
-                    bool init, int tpb) {
+int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const Work* table, int nwork, bool init) {
   cudaError_t err;
+  const int tpb = init ? c.slots() : c.tpb;  // the initial state takes one thread per slot
   if (c.bx > 0) {
     if (tpb > c.max_tpb) {
       if (nwork <= 0) return PA_OK;  // nothing to set up for a block size that cannot run
@@ -468,50 +528,40 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
     }
   } else if (c.dim == 1) {
     err = launch_sweep1d(tpb, c.split, runs, table, nwork, c.W, c.Wr, st, init);
-  } else {
+  } else if (init) {
     switch (c.L) {
-      case 2: err = launch_sweep3d_L2(tpb, c.split, runs, table, nwork, st, init); break;
-      case 4: err = launch_sweep3d_L4(tpb, c.split, runs, table, nwork, st, init); break;
-      case 6: err = launch_sweep3d_L6(tpb, c.split, runs, table, nwork, st, init); break;
-      case 8: err = launch_sweep3d_L8(tpb, c.split, runs, table, nwork, st, init); break;
-      case 10: err = launch_sweep3d_L10(tpb, c.split, runs, table, nwork, st, init); break;
-      case 12: err = launch_sweep3d_L12(tpb, c.split, runs, table, nwork, st, init); break;
-      case 14: err = launch_sweep3d_L14(tpb, c.split, runs, table, nwork, st, init); break;
-      case 16: err = launch_sweep3d_L16(tpb, c.split, runs, table, nwork, st, init); break;
+      case 2: err = launch_init3d_L2(tpb, runs, table, nwork, st); break;
+      case 4: err = launch_init3d_L4(tpb, runs, table, nwork, st); break;
+      case 6: err = launch_init3d_L6(tpb, runs, table, nwork, st); break;
+      case 8: err = launch_init3d_L8(tpb, runs, table, nwork, st); break;
+      case 10: err = launch_init3d_L10(tpb, runs, table, nwork, st); break;
+      case 12: err = launch_init3d_L12(tpb, runs, table, nwork, st); break;
+      case 14: err = launch_init3d_L14(tpb, runs, table, nwork, st); break;
+      case 16: err = launch_init3d_L16(tpb, runs, table, nwork, st); break;
       default: return fail(PA_ERR_UNSUPPORTED, "no kernel for L=%d", c.L);
     }
+  } else {
+    err = sweep3d_call(c.L, {tpb, c.split, c.rp, runs, table, nwork, st});
   }
   if (err != cudaSuccess) return cuda_fail(err, "sweep kernel launch");
   return PA_OK;
 }
 
-int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork, bool init, int tpb) {
-  return launch_class_on(E.d_runs, E.st, c, table, nwork, init, tpb);
+int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork, bool init) {
+  return launch_class_on(E.d_runs, E.st, c, table, nwork, init);
 }
 
-// Set the dynamic shared-memory limits of every block size and every
-// supported number of threads per replica of the class now, outside any
-// stream capture (the autotuner may pick any of them later).
-int prepare_class_launches(RunDev* runs, cudaStream_t st, const LatticeClass& c) {
-  LatticeClass t = c;
-  for (int split : {1, 2, 4, 8}) {
-    if (!split_supported(c, split)) continue;
-    t.split = split;
-    for (int tpb : {32, 64, 128, 256, 512, 1024}) {
-      if (!tpb_supported(c, tpb) || (split > 1 && (tpb < 64 || tpb / split < 4))) continue;
-      int s = launch_class_on(runs, st, t, nullptr, 0, false, tpb);
-      if (s != PA_OK) return s;
-      s = launch_class_on(runs, st, t, nullptr, 0, true, tpb);
-      if (s != PA_OK) return s;
-    }
-  }
-  return PA_OK;
+// Set the dynamic shared-memory limits of the class's launch shape, outside
+// any stream capture (again wherever the shape changes).
+int prepare_class_launch(RunDev* runs, cudaStream_t st, const LatticeClass& c) {
+  int s = launch_class_on(runs, st, c, nullptr, 0, false);
+  return s == PA_OK ? launch_class_on(runs, st, c, nullptr, 0, true) : s;
 }
 
 int build_class_table(Engine& E, LatticeClass& c) {
   std::vector<Work> t;
   for (int32_t r : c.runs)
-    for (int64_t f = 0; f < E.h[r].R_cap; f += c.tpb) t.push_back({r, (int32_t)f});
+    for (int64_t f = 0; f < E.h[r].R_cap; f += c.slots()) t.push_back({r, (int32_t)f});
   c.nwork = (int)t.size();
   c.d_table = (Work*)E.dalloc(sizeof(Work) * std::max<size_t>(t.size(), 1));
   if (!c.d_table) return fail(PA_ERR_OOM, "work table allocation refused");
@@ -624,19 +674,20 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
       }
       c.W = d.W;
       c.Wr = d.Wr;
-      set_default_launch(c, tpb_opt, split_opt);
-      if (split_opt > 1 && c.split != split_opt)
-        return fail(PA_ERR_INVALID, "%d threads per replica do not split the rows of this lattice or block",
-                    split_opt);
       E.cls.push_back(c);
       it = E.cls.end() - 1;
     }
     it->runs.push_back(r);
   }
   for (auto& c : E.cls) {
+    int64_t replicas = 0;
+    for (int32_t r : c.runs) replicas += E.R0[r];
+    set_default_launch(c, tpb_opt, split_opt, replicas);
+    if (split_opt > 1 && c.split != split_opt)
+      return fail(PA_ERR_INVALID, "%d threads per replica do not split the rows of this lattice or block", split_opt);
     st = build_class_table(E, c);
     if (st != PA_OK) return st;
-    st = prepare_class_launches(E.d_runs, E.st, c);
+    st = prepare_class_launch(E.d_runs, E.st, c);
     if (st != PA_OK) return st;
   }
   // beta = 0 population (Sec. 2)
@@ -694,7 +745,7 @@ static int engine_step(Engine& E, bool ovr, double beta, int theta, int64_t Rt) 
       PA_CUDA(cudaEventCreate(&b));
       PA_CUDA(cudaEventRecordWithFlags(a, E.st, rec_flags));
     }
-    int st = launch_class(E, c, c.d_table, c.nwork, false, c.tpb);
+    int st = launch_class(E, c, c.d_table, c.nwork, false);
     if (st != PA_OK) return st;
     if (timed) {
       PA_CUDA(cudaEventRecordWithFlags(b, E.st, rec_flags));
@@ -715,7 +766,7 @@ int engine_init_population(Engine& E) {
   NvtxRange init_range("pa_init");
   PA_CUDA(launch_init_state(E.d_runs, nullptr, E.n, E.max_bins, E.st));
   for (auto& c : E.cls) {
-    int st = launch_class(E, c, c.d_table, c.nwork, true, c.tpb);
+    int st = launch_class(E, c, c.d_table, c.nwork, true);
     if (st != PA_OK) return st;
   }
   PA_CUDA(launch_init_finish(E.d_runs, nullptr, E.n, E.st));

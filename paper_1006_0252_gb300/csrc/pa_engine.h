@@ -76,9 +76,9 @@ PA_DECLG(8)
 PA_DECLG(10)
 PA_DECLG(12)
 #undef PA_DECLG
-#define PA_DECL3(LL)                                                                                \
-  cudaError_t launch_sweep3d_L##LL(int tpb, int split, RunDev* runs, const Work* table, int nwork, \
-                                   cudaStream_t st, bool init);                                    \
+#define PA_DECL3(LL)                                                                                       \
+  cudaError_t sweep3d_L##LL(const Sweep3dLaunch& a);                                                       \
+  cudaError_t launch_init3d_L##LL(int slots, RunDev* runs, const Work* table, int nwork, cudaStream_t st); \
   bool sweep3d_split_ok_L##LL(int split);
 PA_DECL3(2)
 PA_DECL3(4)
@@ -148,11 +148,20 @@ struct LatticeClass {
   int bx = 0, by = 0, bz = 0, bsites = 0;  // general box (bx > 0)
   unsigned bper = 0;
   int max_tpb = 256;                        // largest block whose shared memory fits
-  int tpb;
-  int split = 1;     // cubic lattices: threads per replica in the sweep kernel (1, 2, 4, 8)
+  int tpb = 0;
+  int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
+  int rp = 1;        // +-1 cubic lattices: replicas a thread sweeps side by side (1, 2)
   std::vector<int32_t> runs;
   Work* d_table = nullptr;
   int nwork = 0;
+  // Slots of a work item: the block's threads where a power of two of them
+  // shares a replica (split / rp blocks an item), else the block's replicas.
+  int slots() const { return (split & (split - 1)) == 0 ? tpb : tpb / split * rp; }
+};
+
+// One launch shape of a class.
+struct LaunchShape {
+  int tpb, split, rp;
 };
 
 struct Engine {
@@ -275,13 +284,13 @@ size_t run_slab_bytes(const Geometry& g, int64_t cap, int max_steps);
 int setup_run(char* base, const Geometry& g, const pa_run_spec& s, int64_t cap, int max_steps,
               cudaStream_t st, RunDev* out);
 int default_tpb(int dim, int L);
-void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt);
+void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, int64_t replicas);
+std::vector<LaunchShape> launch_shapes(const LatticeClass& c);
 bool split_supported(const LatticeClass& c, int split);
 bool tpb_supported(const LatticeClass& c, int tpb);
-int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const Work* table, int nwork,
-                    bool init, int tpb);
-int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork, bool init, int tpb);
-int prepare_class_launches(RunDev* runs, cudaStream_t st, const LatticeClass& c);
+int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const Work* table, int nwork, bool init);
+int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork, bool init);
+int prepare_class_launch(RunDev* runs, cudaStream_t st, const LatticeClass& c);
 int build_class_table(Engine& E, LatticeClass& c);
 int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts* opts);
 int engine_prep(Engine& E, bool ovr, double beta, int theta, int64_t Rt);

@@ -14,17 +14,6 @@
 
 namespace pa {
 
-// Move the colour-c bits of a word to the even positions 2m (the inverse of
-// to_colour_positions); other bits are discarded.
-template <class GEO>
-__device__ __forceinline__ uint32_t from_colour_positions(uint32_t v, uint32_t par0) {
-  if constexpr ((GEO::G & 1) == 0) {
-    return (v >> par0) & GEO::EVEN;
-  } else {
-    return (((v & GEO::LANES_EVEN) >> par0) | ((v & GEO::LANES_ODD) >> (par0 ^ 1u))) & GEO::EVEN;
-  }
-}
-
 template <int K>
 __device__ __forceinline__ int32_t lane4(const int4& v) {
   if constexpr (K == 0) return v.x;

@@ -4,6 +4,7 @@
 // reads and writes it there, so a whole schedule runs without host round
 // trips (and can be captured in one CUDA graph).
 #pragma once
+#include <cuda_runtime_api.h>
 #include <stdint.h>
 
 namespace pa {
@@ -111,6 +112,17 @@ struct RunDev {
 struct Work {
   int32_t run;
   int32_t first;
+};
+
+// A launch of the +-1 cubic sweep kernel: tpb threads per block, split of them
+// sharing the rp replicas of a column; nwork work items (nwork <= 0 only
+// prepares the kernel for launches).
+struct Sweep3dLaunch {
+  int tpb, split, rp;
+  RunDev* runs;
+  const Work* table;
+  int nwork;
+  cudaStream_t st;
 };
 
 }  // namespace pa

@@ -52,6 +52,17 @@ __device__ __forceinline__ uint32_t lanes_up(uint32_t s) {  // lane j <- lane j-
   }
 }
 
+// Move the colour-c bits of a word to the even positions 2m (the inverse of
+// to_colour_positions); other bits are discarded.
+template <class GEO>
+__device__ __forceinline__ uint32_t from_colour_positions(uint32_t v, uint32_t par0) {
+  if constexpr ((GEO::G & 1) == 0) {
+    return (v >> par0) & GEO::EVEN;
+  } else {
+    return (((v & GEO::LANES_EVEN) >> par0) | ((v & GEO::LANES_ODD) >> (par0 ^ 1u))) & GEO::EVEN;
+  }
+}
+
 template <int I, int N, class F>
 __device__ __forceinline__ void static_for(F&& f) {
   if constexpr (I < N) {
@@ -87,11 +98,14 @@ __device__ __forceinline__ void store_column(uint32_t* __restrict__ dst, const u
 // of a replica are lanes l, l + 32/P, ... of one warp.
 // ---------------------------------------------------------------------------
 template <class GEO>
-constexpr bool split_ok(int P) {
-  if (P != 1 && P != 2 && P != 4 && P != 8) return false;
+constexpr bool rows_split(int P) {
   if (GEO::L % P != 0) return false;
   if (P == 1) return true;
   return ((GEO::L / P) % 2 == 0) || ((GEO::K * GEO::L / 2) % 4 == 0);
+}
+template <class GEO>
+constexpr bool split_ok(int P) {
+  return (P == 1 || P == 2 || P == 4 || P == 8) && rows_split<GEO>(P);
 }
 
 // Column stride of a block of NR replicas whose P threads read rows D words
@@ -231,20 +245,6 @@ template <class GEO, int P>
 __device__ __forceinline__ const uint4* half_table(const uint4* tab, int j) {
   return tab + 2 * calls_per_colour<GEO>() + j * half_buffer_entries<GEO, P>();
 }
-// One half sweep's table, double-buffered: half sweep h = 2t + c at sweep T
-// goes to table h mod 2; every thread of the block calls this, then the block
-// synchronises once (a table is rewritten two half sweeps later, after the
-// barrier that ends the half sweep reading it).  Returns the table.
-template <class GEO, int TPB, int P>
-__device__ __forceinline__ const uint4* build_half_table(uint4* __restrict__ tab, int h, uint32_t c, uint32_t T) {
-  constexpr int Q = calls_per_colour<GEO>(), S = calls_per_range<GEO, P>(), HB = half_buffer_entries<GEO, P>();
-  uint4* half = tab + 2 * Q + (h & 1) * HB;
-  const uint32_t A1 = PHILOX_MUL1 * T;
-  for (int q = threadIdx.x; q < Q; q += TPB) half[q + q / S] = sweep_half_entry(tab[c * Q + q], A1);
-  __syncthreads();
-  return half;
-}
-
 template <class GEO, int TPB, int P>
 __device__ __forceinline__ void build_half_tables(uint4* __restrict__ tab, int h0, int nh, uint32_t T0) {
   constexpr int Q = calls_per_colour<GEO>(), S = calls_per_range<GEO, P>(), HB = half_buffer_entries<GEO, P>();
@@ -286,6 +286,34 @@ __device__ __forceinline__ void word_uniforms(uint32_t q0, const uint4* __restri
   if constexpr ((A + SITES) % 4 != 0) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) carry[i] = u[4 * (NQ - 1) + i];
+  }
+}
+
+// Record energy, histogram and exact sums of one replica per thread (threads
+// with live == false contribute nothing but take part in the warp's
+// reductions; every thread of the warp calls this).  Replicas of a warp that
+// share an energy add to its bin once: at low temperature most of a
+// population sits in a few bins, and one atomic per replica on the same
+// address held a launch of 4e5 L = 4 replicas at 270 us whatever the sweeps
+// took.
+__device__ __forceinline__ void measure_store(RunDev& R, int nxt, int64_t slot, bool live, int E) {
+  const int lane = threadIdx.x & 31;
+  const int bin = live ? (E + R.Nb) >> 1 : -1 - lane;
+  const unsigned peers = __match_any_sync(0xFFFFFFFFu, bin);
+  if (live) {
+    R.E[nxt][slot] = E;
+    if (lane == __ffs((int)peers) - 1) atomicAdd(&R.hist[nxt][bin], (uint32_t)__popc(peers));
+  }
+  long long e = live ? (long long)E : 0ll;
+  long long e2 = e * e;
+#pragma unroll
+  for (int sh = 16; sh >= 1; sh >>= 1) {
+    e += __shfl_xor_sync(0xFFFFFFFFu, e, sh);
+    e2 += __shfl_xor_sync(0xFFFFFFFFu, e2, sh);
+  }
+  if (lane == 0) {
+    atomicAdd(&R.sumE_next, (unsigned long long)e);
+    atomicAdd(&R.sumE2_next, (unsigned long long)e2);
   }
 }
 

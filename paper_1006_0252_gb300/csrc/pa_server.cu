@@ -120,20 +120,24 @@ static int server_rebuild_tables(pa_server* S) {
       c.L = d.L;
       c.W = d.W;
       c.Wr = d.Wr;
-      set_default_launch(c, S->tpb_opt, S->split_opt);
       S->cls.push_back(c);
       S->cls_buf.push_back(DevBuf());
       S->init_buf.push_back(DevBuf());
-      int st = prepare_class_launches(S->d_runs, S->st, c);  // shared-memory limits, outside any capture
-      if (st != PA_OK) return st;
     }
     S->cls[k].runs.push_back(sl);
   }
   for (size_t k = 0; k < S->cls.size(); ++k) {
     LatticeClass& c = S->cls[k];
+    int64_t replicas = 0;
+    for (int32_t sl : c.runs) replicas += S->h[sl].R;
+    set_default_launch(c, S->tpb_opt, S->split_opt, replicas);  // the shape follows the runs that are active
+    if (!c.runs.empty()) {
+      const int st = prepare_class_launch(S->d_runs, S->st, c);
+      if (st != PA_OK) return st;
+    }
     std::vector<Work> t;
     for (int32_t sl : c.runs)
-      for (int64_t f = 0; f < S->h[sl].R_cap; f += c.tpb) t.push_back({sl, (int32_t)f});
+      for (int64_t f = 0; f < S->h[sl].R_cap; f += c.slots()) t.push_back({sl, (int32_t)f});
     c.nwork = (int)t.size();
     if (!S->ensure(S->cls_buf[k], sizeof(Work) * std::max<size_t>(t.size(), 1))) return fail(PA_ERR_OOM, "server tables");
     c.d_table = (Work*)S->cls_buf[k].p;
@@ -158,11 +162,11 @@ static int server_init_runs(pa_server* S, const std::vector<int32_t>& fresh) {
     std::vector<Work> t;
     for (int32_t sl : fresh)
       if (S->h[sl].dim == c.dim && S->h[sl].L == c.L)
-        for (int64_t f = 0; f < S->h[sl].R_cap; f += c.tpb) t.push_back({sl, (int32_t)f});
+        for (int64_t f = 0; f < S->h[sl].R_cap; f += c.slots()) t.push_back({sl, (int32_t)f});
     if (t.empty()) continue;
     if (!S->ensure(S->init_buf[k], sizeof(Work) * t.size())) return fail(PA_ERR_OOM, "server tables");
     PA_CUDA(cudaMemcpyAsync(S->init_buf[k].p, t.data(), sizeof(Work) * t.size(), cudaMemcpyHostToDevice, S->st));
-    int st = launch_class_on(S->d_runs, S->st, c, (const Work*)S->init_buf[k].p, (int)t.size(), true, c.tpb);
+    int st = launch_class_on(S->d_runs, S->st, c, (const Work*)S->init_buf[k].p, (int)t.size(), true);
     if (st != PA_OK) return st;
   }
   PA_CUDA(launch_init_finish(S->d_runs, (const int32_t*)S->init_ids_buf.p, (int)fresh.size(), S->st));
@@ -339,7 +343,7 @@ int pa_server_tick(pa_server* S, int steps, int32_t* n_active, int32_t* n_queued
     PA_CUDA(launch_scatter(S->d_runs, (const Work*)S->copy_buf.p, S->n_copy, S->st));
     for (auto& c : S->cls) {
       if (c.nwork == 0) continue;
-      st = launch_class_on(S->d_runs, S->st, c, c.d_table, c.nwork, false, c.tpb);
+      st = launch_class_on(S->d_runs, S->st, c, c.d_table, c.nwork, false);
       if (st != PA_OK) return st;
     }
     PA_CUDA(launch_commit(S->d_runs, ids, na, S->st));

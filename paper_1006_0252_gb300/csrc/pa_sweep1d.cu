@@ -124,24 +124,6 @@ __device__ __forceinline__ void half_sweep1d(uint32_t* __restrict__ col, int CS,
   }
 }
 
-__device__ __forceinline__ void measure_store1d(RunDev& R, int nxt, int64_t slot, bool live, int E) {
-  if (live) {
-    R.E[nxt][slot] = E;
-    atomicAdd(&R.hist[nxt][(E + R.Nb) >> 1], 1u);
-  }
-  long long e = live ? (long long)E : 0ll;
-  long long e2 = e * e;
-#pragma unroll
-  for (int sh = 16; sh >= 1; sh >>= 1) {
-    e += __shfl_xor_sync(0xFFFFFFFFu, e, sh);
-    e2 += __shfl_xor_sync(0xFFFFFFFFu, e2, sh);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&R.sumE_next, (unsigned long long)e);
-    atomicAdd(&R.sumE2_next, (unsigned long long)e2);
-  }
-}
-
 template <int TPB>
 __device__ __forceinline__ void store_column1d(uint32_t* __restrict__ dst,
                                                const uint32_t* __restrict__ col, int W, int WR) {
@@ -301,7 +283,7 @@ __global__ void __launch_bounds__(TPB) k_sweep1d(RunDev* __restrict__ runs, cons
       d4[q] = v;
     }
   }
-  measure_store1d(R, nxt, slot, live && part == 0, E);
+  measure_store(R, nxt, slot, live && part == 0, E);
 }
 
 template <int TPB>
@@ -336,7 +318,7 @@ __global__ void __launch_bounds__(TPB) k_init1d(RunDev* __restrict__ runs,
     E = R.Nb - 2 * satisfied1d(col, TPB, s_bond, W, WR, nl, 0, WR);
     store_column1d<TPB>(R.spins[0] + (size_t)slot * W, col, W, WR);
   }
-  measure_store1d(R, 0, slot, live, E);
+  measure_store(R, 0, slot, live, E);
 }
 
 template <int TPB, int P>

@@ -4,15 +4,49 @@
 // temperature"; Algorithm: "Equilibrate replica j for theta sweeps", then
 // "Compute observables").
 //
-// P threads own one replica (P = 1, 2, 4 or 8, chosen per lattice class).
-// The replica's packed words live in a column of shared memory (word w of
-// replica r at s_spin[w * CS + r], so a warp touches consecutive banks); each
-// thread sweeps its L / P y-rows with a three-row sliding window in registers
-// and updates the G words of a row with 32-bit bitwise logic: for every
-// direction d the bond bit b_d = s ^ s_nb ^ j_d is 1 where the bond is
-// satisfied (J s s' = -1), a carry-save adder counts the n satisfied bonds per
-// site (dE = 4n - 12), and a site flips iff n <= 3 or its uniform
+// A block keeps its replicas in shared memory split by colour: for colour c
+// and word w = y G + g of the packed lattice, one 32-bit word holds the word's
+// S = K L / 2 colour-c sites by rank m = j L/2 + h (lane j, site x = 2h + q,
+// q = (c + y + z) mod 2) of one replica in bits 0..15 and, with RP = 2, of a
+// second replica in bits 16..31.  A colour-c site's neighbours all have the
+// other colour, and they sit at these ranks of the other colour's words:
+//   y +- 1   rank m of the words w +- G (x and the lane stay),
+//   z +- 1   rank m of the words w +- 1; across the end of a row of words
+//            (g = G-1 -> 0, g = 0 -> G-1) the lane moves by one: m +- L/2,
+//   x +- 1   one of the two at rank m of the word w itself; the other at
+//            h - 1 (q = 0) or h + 1 (q = 1), a rotation of every lane's field.
+// So one 32-bit operation serves 2 S <= 32 sites of one colour (a layout with
+// both colours in a word serves at most 16), the threshold compares need no
+// spreading to alternate bits, and words are written in place: a half sweep
+// writes colour-c words and reads colour-(1-c) words only.
+//
+// For every direction d the bond bit b_d = s ^ s_nb ^ j_d is 1 where the bond
+// is satisfied (J s s' = -1), a carry-save adder counts the n satisfied bonds
+// per site (dE = 4n - 12), and a site flips iff n <= 3 or its uniform
 // u < threshold[dE/2] (only energy rises draw on the uniform).
+//
+// P threads share the replicas of a column (ranges of L / P rows).
+//
+// What bounds it.  A scheduler issues one full-rate integer instruction (two
+// register operands: add, two-input logic) a cycle and a half-rate one (three
+// operands, shifts, permutes, minima, multiplies) every two cycles, whatever
+// pipe takes it; a wide multiply also holds the multiply pipe four cycles.  A
+// generator round of a warp is 2 wide multiplies and 2 three-input XORs: 8.2
+// cycles on the multiply pipe and 8 of issue (8.66 measured alone), so every
+// other instruction of the sweep adds to the generator's time.  Per 16 sites
+// of 32 replicas at L = 8 the generator takes 265 cycles and the launch 349
+// (beta = 4) to 442 (beta = 0.1): it is issue bound, and only fewer or
+// cheaper instructions help.  This layout needs 180 instructions there at
+// beta = 4 where a word of both colours needed 202.  One launch, theta = 10,
+// us at beta = 0.1 / 1.0 / 4.0 (both colours in a word -> this layout):
+//   L = 8,  1e5 replicas    404 / 371 / 304 -> 360 / 333 / 281
+//   L = 12, 30011 replicas  511 / 464 / 382 -> 420 / 389 / 330
+//   L = 10, 30000 replicas  427 / 407 / 284 -> 252 / 238 / 205
+//   L = 6,  40000 replicas  131 / 119 / 96  ->  97 /  91 /  79
+//   L = 16, 20000 replicas  864 / 804 / 617 -> 681 / 632 / 544
+//   L = 14, 20000 replicas 1083 / 995 / 687 -> 469 / 435 / 371
+// (L = 6, 10 and 14 had one thread per replica before; they split in pairs of
+// rows now.)
 #pragma once
 #include "pa_lattice3d.cuh"
 
@@ -58,40 +92,192 @@ __device__ __forceinline__ int satisfied_rows(const uint32_t* __restrict__ col, 
   return sat;
 }
 
-// Record energy, histogram and exact sums of one replica (lanes with
-// live == false contribute nothing but take part in the warp reduction).
-__device__ __forceinline__ void measure_store(RunDev& R, int nxt, int64_t slot, bool live, int E) {
-  if (live) {
-    R.E[nxt][slot] = E;
-    atomicAdd(&R.hist[nxt][(E + R.Nb) >> 1], 1u);
+// ---------------------------------------------------------------------------
+// Colour-split words.
+// ---------------------------------------------------------------------------
+template <class GEO>
+struct Half {
+  static constexpr int H = GEO::L / 2;       // colour-c sites of a lane
+  static constexpr int S = GEO::K * H;       // colour-c sites of a word, <= 16
+  static constexpr uint32_t ONE = (1u << S) - 1u;  // bits of one replica (S <= 16)
+  static constexpr uint32_t BOTH = ONE | (ONE << 16);
+  static constexpr uint32_t fields(uint32_t f) {  // f in every lane's field, both replicas
+    uint32_t m = 0;
+    for (int j = 0; j < GEO::K; ++j) m |= f << (j * H);
+    return m | (m << 16);
   }
-  long long e = live ? (long long)E : 0ll;
-  long long e2 = e * e;
+  static constexpr uint32_t F0 = fields(1u);             // h = 0
+  static constexpr uint32_t FH = fields(1u << (H - 1));  // h = H - 1
+  static constexpr uint32_t odd_lanes() {                // lanes with odd j
+    uint32_t m = 0;
+    for (int j = 1; j < GEO::K; j += 2) m |= ((1u << H) - 1u) << (j * H);
+    return m | (m << 16);
+  }
+  static constexpr uint32_t ODD = odd_lanes();
+  // lane moves: bits that stay inside the word when m shifts by H
+  static constexpr uint32_t LOW = ((1u << (S - H)) - 1u) | (((1u << (S - H)) - 1u) << 16);
+};
+
+// Neighbour one lane up (z + 1 across the end of a row of words) and down.
+template <class GEO>
+__device__ __forceinline__ uint32_t lane_next(uint32_t x) {
+  using HF = Half<GEO>;
+  if constexpr (GEO::K == 1) return x;
+  return ((x >> HF::H) & HF::LOW) | ((x << (HF::S - HF::H)) & (HF::BOTH & ~HF::LOW));
+}
+template <class GEO>
+__device__ __forceinline__ uint32_t lane_prev(uint32_t x) {
+  using HF = Half<GEO>;
+  constexpr uint32_t UP = (HF::LOW << HF::H) & HF::BOTH;  // bits H .. S-1 of both replicas
+  if constexpr (GEO::K == 1) return x;
+  return ((x << HF::H) & UP) | ((x >> (HF::S - HF::H)) & (HF::BOTH & ~UP));
+}
+
+// The x neighbour that is not at the same rank: h - 1 where q = 0, h + 1
+// where q = 1.  With e = (c + y) mod 2 of a row, q = e ^ (g mod 2) in every
+// lane of word g when G is even: one rotation of the fields, whose shifts and
+// masks are set once per row; when G is odd q also alternates with the lane,
+// and both rotations are taken.  Bits past S are junk (the flips are masked).
+template <class GEO>
+struct RowX {
+  uint32_t l, r;    // G even: shifts of the words with g even (exchanged for g odd)
+  uint32_t m0, m1;  // G even: bits taken from the left shift, g even / odd; G odd: lanes with q = 1
+  __device__ __forceinline__ explicit RowX(uint32_t e) {
+    using HF = Half<GEO>;
+    constexpr uint32_t D = HF::BOTH & ~HF::F0;
+    if constexpr ((GEO::G & 1) == 0) {
+      l = e ? (uint32_t)(HF::H - 1) : 1u;
+      r = e ? 1u : (uint32_t)(HF::H - 1);
+      m0 = e ? HF::FH : D;
+      m1 = e ? D : HF::FH;
+    } else {
+      l = r = 0u;
+      m0 = e ? ~HF::ODD : HF::ODD;
+      m1 = ~m0;
+    }
+  }
+  template <int GP>  // g mod 2
+  __device__ __forceinline__ uint32_t other(uint32_t b) const {
+    using HF = Half<GEO>;
+    constexpr uint32_t D = HF::BOTH & ~HF::F0, U = HF::BOTH & ~HF::FH;
+    const uint32_t m = GP == 0 ? m0 : m1;
+    if constexpr ((GEO::G & 1) == 0) {
+      return GP == 0 ? (((b << l) & m) | ((b >> r) & ~m)) : (((b << r) & m) | ((b >> l) & ~m));
+    } else {
+      const uint32_t down = ((b << 1) & D) | ((b >> (HF::H - 1)) & HF::F0);
+      const uint32_t up = ((b >> 1) & U) | ((b << (HF::H - 1)) & HF::FH);
+      return (up & m) | (down & ~m);
+    }
+  }
+};
+
+// Element of a column: RP replicas' sites of one colour of one word.
+template <int RP>
+using ColourWord = typename std::conditional<RP == 1, uint16_t, uint32_t>::type;
+
+// Two replicas' packed words as the colour-c word (e = (c + y + g) mod 2),
+// and the packed words of the replicas back from a colour word.
+template <class GEO, int RP>
+__device__ __forceinline__ uint32_t take_colour(const uint32_t (&v)[RP], uint32_t e) {
+  uint32_t x[2] = {0u, 0u};
 #pragma unroll
-  for (int sh = 16; sh >= 1; sh >>= 1) {
-    e += __shfl_xor_sync(0xFFFFFFFFu, e, sh);
-    e2 += __shfl_xor_sync(0xFFFFFFFFu, e2, sh);
+  for (int k = 0; k < RP; ++k) {
+    x[k] = from_colour_positions<GEO>(v[k], e);  // sites at even positions 2m
+    x[k] = (x[k] | (x[k] >> 1)) & 0x33333333u;
+    x[k] = (x[k] | (x[k] >> 2)) & 0x0F0F0F0Fu;
+    x[k] = x[k] | (x[k] >> 4);  // ranks 0-7 in byte 0, 8-15 in byte 2
   }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&R.sumE_next, (unsigned long long)e);
-    atomicAdd(&R.sumE2_next, (unsigned long long)e2);
+  return __byte_perm(x[0], x[1], 0x6420u);
+}
+template <class GEO, int K_>
+__device__ __forceinline__ uint32_t place_colour(uint32_t a, uint32_t e) {  // replica K_ (0 or 1)
+  uint32_t x = __byte_perm(a, 0u, K_ == 0 ? 0x4140u : 0x4342u);
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  x = (x | (x << 1)) & 0x55555555u;
+  return to_colour_positions<GEO>(x, e);
+}
+
+// Bond masks of the colour words, one 32-byte entry for (c, w): the x bond to
+// the same rank, the x bond to the other rank, y+, y-, z+, z- (both halves
+// alike).  All threads of the block; a barrier must follow.
+template <class GEO, int TPB>
+__device__ __forceinline__ void fill_bonds(uint4* __restrict__ s_bond, const uint32_t* __restrict__ bonds) {
+  constexpr int WR = GEO::WR, W = GEO::W, G = GEO::G;
+  for (int i = threadIdx.x; i < 2 * WR; i += TPB) {
+    const int c = i / WR, w = i - c * WR;
+    const uint32_t e = (uint32_t)(c + w / G + w % G) & 1u;
+    uint32_t m[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+      const uint32_t v[2] = {bonds[d * W + w], bonds[d * W + w]};
+      m[d] = take_colour<GEO, 2>(v, e);
+    }
+    const uint32_t q = (GEO::G & 1) == 0 ? (e ? 0xFFFFFFFFu : 0u) : (e ? ~Half<GEO>::ODD : Half<GEO>::ODD);
+    s_bond[2 * i] = make_uint4((m[DXM] & q) | (m[DXP] & ~q), (m[DXP] & q) | (m[DXM] & ~q), m[DYP], m[DYM]);
+    s_bond[2 * i + 1] = make_uint4(m[DZP], m[DZM], 0u, 0u);
   }
+}
+
+// The other colour's words around word g of a row: the word at the same (y,
+// g), those of the rows y + 1 and y - 1, and the next and previous word of the
+// row (z +- 1), moved by a lane across the row's ends.  same: word 0 of the
+// row; yp, ym: distance of its neighbour rows.
+struct Around {
+  uint32_t nx, yp, ym, zp, zm;
+};
+template <class GEO, int CS, class T, class INT>
+__device__ __forceinline__ Around around(const T* __restrict__ same, int yp, int ym, INT g) {
+  constexpr int G = GEO::G;
+  Around n;
+  const T* o = same + g * CS;
+  n.nx = o[0];
+  n.yp = o[yp];
+  n.ym = o[ym];
+  n.zp = o[(g + 1 < G ? 1 : 1 - G) * CS];
+  n.zm = o[(g > 0 ? -1 : G - 1) * CS];
+  if (g + 1 == G) n.zp = lane_next<GEO>(n.zp);
+  if (g == 0) n.zm = lane_prev<GEO>(n.zm);
+  return n;
+}
+// Distances of the neighbour rows of row y (in words of a column).
+template <class GEO>
+__device__ __forceinline__ int row_up(int y) {
+  return y + 1 == GEO::L ? -(GEO::L - 1) * GEO::G : GEO::G;
+}
+template <class GEO>
+__device__ __forceinline__ int row_down(int y) {
+  return y == 0 ? (GEO::L - 1) * GEO::G : -GEO::G;
+}
+
+// Satisfied-bond counts n = 4 n2 + 2 n1 + n0 of the colour-c sites s of a
+// word; GP = g mod 2.
+struct Count3 {
+  uint32_t n0, n1, n2;
+};
+template <class GEO, int GP>
+__device__ __forceinline__ Count3 count_satisfied(uint32_t s, const Around& n, const uint4* __restrict__ bond,
+                                                  const RowX<GEO>& rx) {
+  const uint4 j0 = bond[0];
+  const uint2 j1 = *reinterpret_cast<const uint2*>(bond + 1);
+  const uint32_t b0 = s ^ n.nx ^ j0.x;
+  const uint32_t b1 = s ^ rx.template other<GP>(n.nx) ^ j0.y;
+  const uint32_t b2 = s ^ n.yp ^ j0.z;
+  const uint32_t b3 = s ^ n.ym ^ j0.w;
+  const uint32_t b4 = s ^ n.zp ^ j1.x;
+  const uint32_t b5 = s ^ n.zm ^ j1.y;
+  const uint32_t sa = b0 ^ b1 ^ b2, ca = (b0 & b1) | (b2 & (b0 ^ b1));
+  const uint32_t sb = b3 ^ b4 ^ b5, cb = (b3 & b4) | (b5 & (b3 ^ b4));
+  const uint32_t n0 = sa ^ sb, c0 = sa & sb;
+  return {n0, ca ^ cb ^ c0, (ca & cb) | (c0 & (ca ^ cb))};
 }
 
 // ---------------------------------------------------------------------------
 // Threshold compares.  Bit m of ge is [u_m >= thr]: the subtraction u_m - thr
 // sets the carry exactly when it does not borrow, and ge = 2 ge + carry
-// shifts it in (two integer instructions per site); the complement is then
-// spread from bit m to bit 2m, the position mask layout of the word.
+// shifts it in; both run at the full integer rate, where a compare into a
+// predicate and a select would each take a half-rate slot.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t spread_even(uint32_t x) {  // bit m -> bit 2m, m < 16
-  x = (x | (x << 8)) & 0x00FF00FFu;
-  x = (x | (x << 4)) & 0x0F0F0F0Fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  x = (x | (x << 1)) & 0x55555555u;
-  return x;
-}
-
 template <int SITES, int OFF>
 __device__ __forceinline__ uint32_t lt_mask(const uint32_t* u, uint32_t thr) {
   static_assert(SITES <= 16, "at most 16 colour-c sites per word");
@@ -101,247 +287,261 @@ __device__ __forceinline__ uint32_t lt_mask(const uint32_t* u, uint32_t thr) {
     asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, %3;\n\t}"
         : "=r"(ge)
         : "r"(u[OFF + m]), "r"(thr), "r"(ge));
-  constexpr uint32_t VM = (1u << SITES) - 1u;
-  return spread_even(~ge & VM);
+  return ge ^ ((1u << SITES) - 1u);
 }
 
-// The compares with thr(4) and thr(8) in one chain (at high temperature both
-// are needed for almost every word): per site two subtractions shift their
-// carries in, so bit 2m+1 = [u_m >= thr4] and bit 2m = [u_m >= thr8], and no
-// spreading is needed.
-template <int SITES, int OFF>
-__device__ __forceinline__ void lt_mask2(const uint32_t* u, uint32_t thr4, uint32_t thr8, uint32_t& e4,
-                                         uint32_t& e8) {
-  static_assert(SITES <= 16, "at most 16 colour-c sites per word");
-  uint32_t ge = 0u;
+// Minimum of u[OFF .. OFF+N-1], folded three at a time (one instruction for
+// three values).
+template <int N, int OFF>
+__device__ __forceinline__ uint32_t min_of(const uint32_t* u) {
+  uint32_t m = u[OFF];
 #pragma unroll
-  for (int m = SITES - 1; m >= 0; --m)
-    asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\taddc.u32 %0, %4, %4;\n\t"
-        "sub.cc.u32 t, %1, %3;\n\taddc.u32 %0, %0, %0;\n\t}"
-        : "=r"(ge)
-        : "r"(u[OFF + m]), "r"(thr4), "r"(thr8), "r"(ge));
-  constexpr uint32_t EV = (2 * SITES >= 32) ? 0x55555555u : (0x55555555u & ((1u << (2 * SITES)) - 1u));
-  e4 = (~ge >> 1) & EV;
-  e8 = ~ge & EV;
+  for (int i = 1; i + 1 < N; i += 2) m = __vimin3_u32(m, u[OFF + i], u[OFF + i + 1]);
+  if constexpr ((N & 1) == 0) m = min(m, u[OFF + N - 1]);
+  return m;
 }
 
-// Everything a word's update needs beyond the lattice: the half-sweep table,
-// the slot's key, the colour and the thresholds of dE = 4, 8, 12.
+// Everything a word's update needs beyond the lattice: the slots' keys and the
+// thresholds of dE = 4, 8, 12.
+template <int RP>
 struct HalfSweep {
-  const uint4* half;
-  SweepKey key;
-  uint32_t c;
+  SweepKey key[RP];
   uint32_t T4, T8, T12;
   bool low_t;      // T4 < 2^22: most words draw no uniform below T4
   bool high_t;     // T4 >= 2^24: almost every word needs the compares with T4 and T8
   unsigned lanes;  // live lanes of the warp
 };
 
-// Compares of the word's uniforms with the thresholds of dE = 4, 8, 12
-// (masks at even positions 2m: bit set iff u_m < thr).  thr4 >= thr8 >= thr12,
-// so where u >= thr4 the other two compares fail as well: they are skipped for
-// the word when no lane of the warp has a uniform below thr4.  At low
-// temperature the uniforms are first reduced to their minimum, and the word
-// skips all compares when no lane's minimum is below thr4; at high
-// temperature the compares with thr4 and thr8 run as one chain (lt_mask2).
-// Minimum of u[OFF .. OFF+N-1], folded three at a time.
-template <int N, int OFF>
-__device__ __forceinline__ uint32_t min_of(const uint32_t* u) {
-  if constexpr (N == 1) {
-    return u[OFF];
-  } else if constexpr (N == 2) {
-    return min(u[OFF], u[OFF + 1]);
-  } else {
-    constexpr int H = N / 3, R = N - 2 * H;
-    return min(min(min_of<H, OFF>(u), min_of<H, OFF + H>(u)), min_of<R, OFF + 2 * H>(u));
+// Word g of a row of a half sweep: satisfied-bond count of all its replicas'
+// sites at once, then per replica the word's uniforms and the compares, then
+// the flips.  T4 >= T8 >= T12, a site with n = 4, 5, 6 takes the compare with
+// T4, T8, T12, so T8 is compared only where a lane of the warp has a site of
+// n >= 5 with u < T4, T12 where one of n = 6 has u < T8.  At low temperature
+// the word's uniforms are first reduced to their minimum and all compares
+// skipped when no lane's minimum is below T4.  half: the word's first call; A
+// the alignment of its first uniform (see word_uniforms); GP = g mod 2.
+template <class GEO, int RP, int A, int GP>
+__device__ __forceinline__ void word3d(ColourWord<RP>* __restrict__ own, const Around& nb,
+                                       const uint4* __restrict__ bond, const RowX<GEO>& rx,
+                                       const uint4* __restrict__ half, const HalfSweep<RP>& hs, const RoundKeys& rk,
+                                       uint32_t (&carry)[RP][4]) {
+  constexpr int S = Half<GEO>::S;
+  const uint32_t s = *own;
+  const Count3 n = count_satisfied<GEO, GP>(s, nb, bond, rx);
+  uint32_t e4 = 0u, e8 = 0u, e12 = 0u;
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    uint32_t u[4 * word_calls<S, A>()];
+    word_uniforms<S, A>(0u, half, hs.key[k], rk, carry[k], u);
+    if (hs.low_t && !__any_sync(hs.lanes, min_of<S, A>(u) < hs.T4)) continue;
+    const uint32_t m4 = lt_mask<S, A>(u, hs.T4);
+    e4 |= m4 << (16 * k);
+    const uint32_t n5 = (n.n2 & (n.n1 | n.n0)) >> (16 * k), n6 = (n.n2 & n.n1) >> (16 * k);
+    if (!hs.high_t && !__any_sync(hs.lanes, (m4 & n5) != 0u)) continue;
+    const uint32_t m8 = lt_mask<S, A>(u, hs.T8);
+    e8 |= m8 << (16 * k);
+    if (__any_sync(hs.lanes, (m8 & n6) != 0u)) e12 |= lt_mask<S, A>(u, hs.T12) << (16 * k);
   }
+  const uint32_t sel = (n.n1 & e12) | (~n.n1 & ((n.n0 & e8) | (~n.n0 & e4)));
+  *own = (ColourWord<RP>)(s ^ (Half<GEO>::BOTH & (~n.n2 | sel)));
 }
 
-// Returns false when no lane of the warp can have a uniform below thr4 in this
-// word (then the masks are zero and the caller takes the plain update).
-template <int SITES, int A>
-__device__ __forceinline__ bool word_compares(uint32_t q0, const HalfSweep& hs, const RoundKeys& rk,
-                                              uint32_t (&carry)[4], uint32_t& e4, uint32_t& e8, uint32_t& e12) {
-  uint32_t u[4 * word_calls<SITES, A>()];
-  word_uniforms<SITES, A>(q0, hs.half, hs.key, rk, carry, u);
-  e4 = 0u;
-  e8 = 0u;
-  e12 = 0u;
-  if (hs.low_t) {
-    if (!__any_sync(hs.lanes, min_of<SITES, A>(u) < hs.T4)) return false;
-  }
-  if (hs.high_t) {
-    lt_mask2<SITES, A>(u, hs.T4, hs.T8, e4, e8);
-  } else {
-    e4 = lt_mask<SITES, A>(u, hs.T4);
-    if (!__any_sync(hs.lanes, e4 != 0u)) return false;
-    e8 = lt_mask<SITES, A>(u, hs.T8);
-  }
-  if (__any_sync(hs.lanes, e8 != 0u)) e12 = lt_mask<SITES, A>(u, hs.T12);
-  return true;
-}
-
-// Word g of row y: bond bits, satisfied-bond count, compares, flips.  A is
-// the alignment of the word's first uniform (see word_uniforms).
-template <class GEO, int A>
-__device__ __forceinline__ void word3d(int g, int y, const uint32_t* __restrict__ s_bond, uint32_t (&rowm)[GEO::G],
-                                       uint32_t (&row)[GEO::G], const uint32_t (&rowp)[GEO::G], const HalfSweep& hs,
-                                       const RoundKeys& rk, uint32_t (&carry)[4]) {
-  constexpr int G = GEO::G, L = GEO::L, W = GEO::W, K = GEO::K;
-  constexpr int SITES = K * L / 2;  // colour-c sites per word
-  const int w = y * G + g;
-  const uint32_t s = row[g];
-  const uint32_t zp = (g + 1 < G) ? row[(g + 1) % G] : lanes_down<GEO>(row[0]);
-  const uint32_t zm = (g > 0) ? row[(g + G - 1) % G] : lanes_up<GEO>(row[G - 1]);
-  const uint32_t b0 = s ^ rot_xp<GEO>(s) ^ s_bond[DXP * W + w];
-  const uint32_t b1 = s ^ rot_xm<GEO>(s) ^ s_bond[DXM * W + w];
-  const uint32_t b2 = s ^ rowp[g] ^ s_bond[DYP * W + w];
-  const uint32_t b3 = s ^ rowm[g] ^ s_bond[DYM * W + w];
-  const uint32_t b4 = s ^ zp ^ s_bond[DZP * W + w];
-  const uint32_t b5 = s ^ zm ^ s_bond[DZM * W + w];
-  // carry-save count of the six bond bits: n = 4 n2 + 2 n1 + n0
-  const uint32_t sa = b0 ^ b1 ^ b2, ca = (b0 & b1) | (b2 & (b0 ^ b1));
-  const uint32_t sb = b3 ^ b4 ^ b5, cb = (b3 & b4) | (b5 & (b3 ^ b4));
-  const uint32_t n0 = sa ^ sb, c0 = sa & sb;
-  const uint32_t n1 = ca ^ cb ^ c0, n2 = (ca & cb) | (c0 & (ca ^ cb));
-  uint32_t e4, e8, e12;
-  const bool drawn = word_compares<SITES, A>((uint32_t)(w * SITES) >> 2, hs, rk, carry, e4, e8, e12);
-  const uint32_t par0 = (hs.c + (uint32_t)y + (uint32_t)g) & 1u;
-  const uint32_t cm = to_colour_positions<GEO>(GEO::EVEN, par0);
-  if (!drawn) {  // warp-uniform: no rise accepted in this word, only n <= 3 sites flip
-    row[g] = s ^ (cm & ~n2);
-    return;
-  }
-  const uint32_t a4 = to_colour_positions<GEO>(e4, par0);
-  const uint32_t a8 = to_colour_positions<GEO>(e8, par0);
-  const uint32_t a12 = to_colour_positions<GEO>(e12, par0);
-  // n = 4, 5, 6 take the compare with thr(4), thr(8), thr(12)
-  const uint32_t sel = (n1 & a12) | (~n1 & ((n0 & a8) | (~n0 & a4)));
-  row[g] = s ^ (cm & (~n2 | sel));
-}
-
-// Row y of a half sweep (three-row window rowm / row / rowp).  YP is the
-// row's position in its pair of rows (y mod 2 when SITES is not a multiple of
-// 4): a pair of rows holds L^2/2 sites of each colour, a multiple of 4, so
-// the alignment of every word's first uniform is known at compile time.
-template <class GEO, int CS, int YP>
-__device__ __forceinline__ void row3d(uint32_t* __restrict__ col, const uint32_t* __restrict__ s_bond, int y,
-                                      uint32_t (&rowm)[GEO::G], uint32_t (&row)[GEO::G], uint32_t (&rowp)[GEO::G],
-                                      const HalfSweep& hs, const RoundKeys& rk, uint32_t (&carry)[4]) {
-  constexpr int G = GEO::G, L = GEO::L, K = GEO::K;
-  constexpr int SITES = K * L / 2;
-  const int yn = (y + 1 == L) ? 0 : y + 1;
+// One Metropolis half sweep over the colour-c sites of the RPP rows from y0
+// of the replicas of one column (whole pairs of rows where the colour-c sites
+// of a row are not a multiple of 4, since a Philox call serves four
+// consecutive ranks).  half: the column's uniform table of this half sweep.
+// The loop body stays short (a few words), so that the half sweeps of both
+// colours fit the instruction cache: whole rows unrolled stalled 15-30 % of
+// the cycles on instruction fetch at L = 10 and 16.
+template <class GEO, int CS, int RP, int RPP, class COLOUR>
+__device__ __forceinline__ void half_sweep3d(ColourWord<RP>* __restrict__ col, const uint4* __restrict__ s_bond,
+                                             const uint4* __restrict__ half, COLOUR c, const HalfSweep<RP>& hs,
+                                             const RoundKeys& rk, int y0) {
+  using T = ColourWord<RP>;
+  constexpr int G = GEO::G, WR = GEO::WR, S = Half<GEO>::S;
+  uint32_t carry[RP][4];
 #pragma unroll
-  for (int g = 0; g < G; ++g) rowp[g] = col[(yn * G + g) * CS];
-  if constexpr (SITES % 4 == 0) {
-#pragma unroll
-    for (int g = 0; g < G; ++g) word3d<GEO, 0>(g, y, s_bond, rowm, row, rowp, hs, rk, carry);
-  } else {
-    static_for<0, G>([&](auto gc) {
-      constexpr int g = decltype(gc)::value;
-      constexpr int A = (SITES * (YP * G + g)) % 4;
-      word3d<GEO, A>(g, y, s_bond, rowm, row, rowp, hs, rk, carry);
-    });
-  }
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    col[(y * G + g) * CS] = row[g];
-    rowm[g] = row[g];
-    row[g] = rowp[g];
-  }
-}
-
-// One Metropolis half sweep over the colour-c sites of the RPP rows y0 ..
-// y0 + RPP - 1 of one replica (whole pairs of rows when SITES is not a
-// multiple of 4).  Ranges of at most two rows are unrolled.
-template <class GEO, int CS, int RPP>
-__device__ __forceinline__ void half_sweep3d(uint32_t* __restrict__ col, const uint32_t* __restrict__ s_bond,
-                                             const HalfSweep& hs, const RoundKeys& rk, int y0) {
-  constexpr int G = GEO::G, L = GEO::L, K = GEO::K;
-  constexpr int SITES = K * L / 2;
-  uint32_t rowm[G], row[G], rowp[G];
-  uint32_t carry[4] = {0u, 0u, 0u, 0u};
-  const int ym = (y0 == 0) ? L - 1 : y0 - 1;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    rowm[g] = col[(ym * G + g) * CS];
-    row[g] = col[(y0 * G + g) * CS];
-  }
-  if constexpr (SITES % 4 == 0) {
-    if constexpr (RPP <= 2) {
-#pragma unroll
-      for (int i = 0; i < RPP; ++i) row3d<GEO, CS, 0>(col, s_bond, y0 + i, rowm, row, rowp, hs, rk, carry);
-    } else {
+  for (int k = 0; k < RP; ++k) carry[k][0] = carry[k][1] = carry[k][2] = carry[k][3] = 0u;
+  T* own = col + (c * WR + y0 * G) * CS;
+  const T* oth = col + ((1 - c) * WR + y0 * G) * CS;
+  const uint4* bond = s_bond + 2 * (c * WR + y0 * G);
+  half += (y0 * G * S) / 4;
+  if constexpr (G <= 2) {
+    // whole rows, pairs of them where a row's uniforms end within a call
+    constexpr int YU = (G * S) % 4 == 0 ? 1 : 2;
 #pragma unroll 1
-      for (int i = 0; i < RPP; ++i) row3d<GEO, CS, 0>(col, s_bond, y0 + i, rowm, row, rowp, hs, rk, carry);
+    for (int i = 0; i < RPP; i += YU) {
+      static_for<0, YU>([&](auto yc) {
+        constexpr int yi = decltype(yc)::value;
+        const int y = y0 + i + yi, yp = row_up<GEO>(y) * CS, ym = row_down<GEO>(y) * CS;
+        const RowX<GEO> rx((uint32_t)(c + y) & 1u);
+        static_for<0, G>([&](auto gc) {
+          constexpr int g = decltype(gc)::value, w = yi * G + g;
+          const Around nb = around<GEO, CS>(oth + yi * G * CS, yp, ym, gc);
+          word3d<GEO, RP, (w * S) % 4, (g & 1)>(own + w * CS, nb, bond + 2 * w, rx, half + w * S / 4, hs, rk, carry);
+        });
+      });
+      own += YU * G * CS;
+      oth += YU * G * CS;
+      bond += 2 * YU * G;
+      half += YU * G * S / 4;
+    }
+  } else if constexpr (G % 2 == 0) {
+    // pairs of words of a row
+    static_assert(S % 4 == 0, "a word's uniforms are whole calls");
+#pragma unroll 1
+    for (int y = y0; y < y0 + RPP; ++y) {
+      const int yp = row_up<GEO>(y) * CS, ym = row_down<GEO>(y) * CS;
+      const RowX<GEO> rx((uint32_t)(c + y) & 1u);
+#pragma unroll 1
+      for (int g = 0; g < G; g += 2) {
+        static_for<0, 2>([&](auto kc) {
+          constexpr int k = decltype(kc)::value;
+          const Around nb = around<GEO, CS>(oth - g * CS, yp, ym, g + k);
+          word3d<GEO, RP, 0, k>(own + k * CS, nb, bond + 2 * k, rx, half + k * S / 4, hs, rk, carry);
+        });
+        own += 2 * CS;
+        oth += 2 * CS;
+        bond += 4;
+        half += 2 * S / 4;
+      }
     }
   } else {
-    static_assert(RPP % 2 == 0, "rows come in pairs");
+    // pairs of words across the rows of a pair (y0 even, so the word number's
+    // parity is that of y + g)
+    static_assert(S % 2 == 0 && RPP % 2 == 0 || RPP == GEO::L, "whole pairs of rows");
+    const RowX<GEO> rx((uint32_t)c & 1u);
+    int y = y0, g = 0, yp = row_up<GEO>(y) * CS, ym = row_down<GEO>(y) * CS;
 #pragma unroll 1
-    for (int i = 0; i < RPP; i += 2) {
-      row3d<GEO, CS, 0>(col, s_bond, y0 + i, rowm, row, rowp, hs, rk, carry);
-      row3d<GEO, CS, 1>(col, s_bond, y0 + i + 1, rowm, row, rowp, hs, rk, carry);
+    for (int i = 0; i < RPP * G; i += 2) {
+      static_for<0, 2>([&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const Around nb = around<GEO, CS>(oth + (k - g) * CS, yp, ym, g);
+        word3d<GEO, RP, (k * S) % 4, k>(own + k * CS, nb, bond + 2 * k, rx, half + k * S / 4, hs, rk, carry);
+        if (++g == G) {
+          g = 0;
+          ++y;
+          yp = row_up<GEO>(y) * CS;
+          ym = row_down<GEO>(y) * CS;
+        }
+      });
+      own += 2 * CS;
+      oth += 2 * CS;
+      bond += 4;
+      half += 2 * S / 4;
     }
   }
 }
 
-// Replicas per block: TPB / P; block b takes work item b / P of the class
-// table (TPB consecutive slots of one run) and its (b mod P)-th share.
-template <int L, int TPB, int P>
+// Block of TPB threads: P threads per column of RP replicas, thread t takes
+// row range t / NC of column t mod NC (NC = TPB / P columns; the last TPB - P
+// NC threads of an odd P only help with the tables).  A block is a multiple of
+// four warps wherever it can be: its warps go to the SM's four schedulers in
+// turn, so blocks of 5 warps (one per row range, L = 10) gave one scheduler
+// twice the work of the others.  Block b takes work item b / BPI of the class
+// table (SLOTS consecutive slots of one run) and its (b mod BPI)-th share.
+template <int L, int TPB, int P, int RP>
 struct SweepShape {
   using GEO = Geo3<L>;
-  static constexpr int NR = TPB / P;                                    // replicas per block
-  static constexpr int RPP = L / P;                                     // rows per thread
-  static constexpr int CS = split_stride(NR, RPP * GEO::G, P, TPB);     // column stride
-  // half-sweep tables held at once: with one thread per replica as many as
-  // fit; with several, two, double-buffered (one block barrier per half
-  // sweep measured 1 % faster at L = 8 with four threads per replica than
-  // chunks of tables with warp barriers between their half sweeps)
-  static constexpr int NH = P > 1 ? 2 : half_tables<GEO, TPB, P>(4 * (6 * GEO::W + GEO::WR * CS));
-  static constexpr int SMEM_WORDS = sweep_table_words<GEO, P>(NH) + 6 * GEO::W + GEO::WR * CS;
+  static constexpr int NC = TPB / P;              // columns
+  static constexpr int NR = NC * RP;              // replicas per block
+  static constexpr int RPP = L / P;               // rows per thread
+  static constexpr int WPP = RPP * GEO::G;        // words per thread
+  static constexpr int SLOTS = (P & (P - 1)) == 0 ? TPB : NR;  // slots of a work item (LatticeClass::slots)
+  static constexpr int BPI = SLOTS / NR;
+  static constexpr int CS = NC;
+  static constexpr int BOND_WORDS = 16 * GEO::WR;
+  static constexpr int SPIN_WORDS = (GEO::WR * CS * RP + 3) / 4 * 4;  // [2 colours][WR][CS] colour words
+  static constexpr int Q = calls_per_colour<GEO>();
+  // entries of one half-sweep table: one padding entry after each thread's
+  // range puts the ranges' reads on different banks
+  static constexpr int RANGE = P == 1 ? Q : WPP * Half<GEO>::S / 4;
+  static constexpr int HB = Q + Q / RANGE + 1;
+  // half-sweep tables held at once: with one thread per column as many as
+  // fit, else two, double-buffered behind one block barrier per half sweep
+  static constexpr int room() {
+    const int n = (216 * TPB - 4 * (BOND_WORDS + SPIN_WORDS)) / (16 * HB);
+    return n >= 20 ? 20 : (n < 2 ? 2 : (n & ~1));
+  }
+  static constexpr int NH = P > 1 ? 2 : room();
+  // the tables' memory also takes the row ranges' energies at the end
+  static constexpr int TAB_WORDS = 4 * NH * HB > RP * TPB ? 4 * NH * HB : RP * TPB;
+  static constexpr size_t SMEM_WORDS = (size_t)TAB_WORDS + BOND_WORDS + SPIN_WORDS;
+  static constexpr bool OK = SLOTS % NR == 0 && NR <= TPB && NC >= 4 && (P == 1 || TPB >= 64);
 };
+
+// Half-sweep tables h0 .. h0 + nh - 1 (half sweep h = 2t + c is colour c of
+// sweep T0 + t) at tab[j HB + q + q / RANGE], all threads of the block.
+template <class SH, int TPB>
+__device__ __forceinline__ void build_tables3d(uint4* __restrict__ tab, int buf, int h0, int nh, uint32_t T0,
+                                               const RoundKeys& rk) {
+  for (int i = threadIdx.x; i < nh * SH::Q; i += TPB) {
+    const int j = i / SH::Q, q = i - j * SH::Q;
+    const int h = h0 + j;
+    const uint32_t A1 = PHILOX_MUL1 * (T0 + (uint32_t)(h >> 1));
+    tab[(buf + j) * SH::HB + q + q / SH::RANGE] =
+        sweep_half_entry(sweep_call_entry((uint32_t)q, TAG_SWEEP + (uint32_t)(h & 1), rk), A1);
+  }
+}
 
 // Sec. 2: the gather of the resampled population (slot s <- old slot src(s)),
 // theta checkerboard sweeps at beta', and the energy of every replica.
-template <int L, int TPB, int P>
+template <int L, int TPB, int P, int RP>
 __global__ void __launch_bounds__(TPB) k_sweep3d(RunDev* __restrict__ runs, const Work* __restrict__ table) {
   using GEO = Geo3<L>;
-  using SH = SweepShape<L, TPB, P>;
-  constexpr int WR = GEO::WR, W = GEO::W, RW = 32 / P, RPP = SH::RPP, CS = SH::CS;
+  using SH = SweepShape<L, TPB, P, RP>;
+  using HF = Half<GEO>;
+  constexpr int WR = GEO::WR, W = GEO::W, G = GEO::G, CS = SH::CS, RPP = SH::RPP;
   extern __shared__ __align__(16) uint32_t smem[];
-  uint4* s_tab = reinterpret_cast<uint4*>(smem);             // sweep_table_words
-  uint32_t* s_bond = smem + sweep_table_words<GEO, P>(SH::NH);  // [6][W]
-  uint32_t* s_spin = s_bond + 6 * W;                  // [WR][CS]
-  const Work wk = table[blockIdx.x / P];
+  uint4* s_tab = reinterpret_cast<uint4*>(smem);
+  uint4* s_bond = reinterpret_cast<uint4*>(smem + SH::TAB_WORDS);
+  ColourWord<RP>* s_spin = reinterpret_cast<ColourWord<RP>*>(smem + SH::TAB_WORDS + SH::BOND_WORDS);  // [2][WR][CS]
+  const Work wk = table[blockIdx.x / SH::BPI];
   RunDev& R = runs[wk.run];
   if (R.skip) return;
   const int64_t Rn = R.R_next;
-  const int64_t first = (int64_t)wk.first + (int64_t)(blockIdx.x % P) * SH::NR;
+  const int64_t first = (int64_t)wk.first + (int64_t)(blockIdx.x % SH::BPI) * SH::NR;
   if (first >= Rn) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (int i = tid; i < 6 * W; i += TPB) s_bond[i] = R.bonds[i];
+  const int tid = threadIdx.x;
+  fill_bonds<GEO, TPB>(s_bond, R.bonds);
   const RoundKeys rk = make_round_keys(R.seed);
-  fill_call_table<GEO, TPB>(s_tab, rk);
-  const int r = (tid >> 5) * RW + (lane % RW);  // replica of this thread in the block
-  const int part = lane / RW;                   // its row range
+  const int part = tid / SH::NC, r = tid - part * SH::NC;  // row range and column of this thread
+  // replica k of column r is slot first + k NC + r
   const int64_t slot = first + r;
-  const bool live = slot < Rn;
+  const bool live = part < P && slot < Rn;
   const int cur = R.cur, nxt = cur ^ 1;
-  uint32_t* col = s_spin + r;
+  ColourWord<RP>* col = s_spin + r;
   if (live) {
-    const int32_t src = R.src[slot];
-    const uint4* p4 = reinterpret_cast<const uint4*>(R.spins[cur] + (size_t)src * W);
-#pragma unroll 4
+    const uint4* p4[RP];
+    bool on[RP];
+#pragma unroll
+    for (int k = 0; k < RP; ++k) {
+      on[k] = slot + k * SH::NC < Rn;
+      p4[k] = reinterpret_cast<const uint4*>(R.spins[cur] + (size_t)(on[k] ? R.src[slot + k * SH::NC] : 0) * W);
+    }
+#pragma unroll 2
     for (int q = part; q < W / 4; q += P) {
-      const uint4 v = p4[q];
-      if (4 * q + 0 < WR) col[(4 * q + 0) * CS] = v.x;
-      if (4 * q + 1 < WR) col[(4 * q + 1) * CS] = v.y;
-      if (4 * q + 2 < WR) col[(4 * q + 2) * CS] = v.z;
-      if (4 * q + 3 < WR) col[(4 * q + 3) * CS] = v.w;
+      uint32_t v[4][RP];
+#pragma unroll
+      for (int k = 0; k < RP; ++k) {
+        const uint4 t = on[k] ? p4[k][q] : make_uint4(0u, 0u, 0u, 0u);
+        v[0][k] = t.x;
+        v[1][k] = t.y;
+        v[2][k] = t.z;
+        v[3][k] = t.w;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int w = 4 * q + i;
+        if (w < WR) {
+          const uint32_t e = (uint32_t)(w / G + w % G) & 1u;
+          col[w * CS] = (ColourWord<RP>)take_colour<GEO, RP>(v[i], e);
+          col[(WR + w) * CS] = (ColourWord<RP>)take_colour<GEO, RP>(v[i], e ^ 1u);
+        }
+      }
     }
   }
-  __syncthreads();
-  HalfSweep hs;
+  HalfSweep<RP> hs;
   hs.T4 = R.thr[2];
   hs.T8 = R.thr[4];
   hs.T12 = R.thr[6];
@@ -352,68 +552,116 @@ __global__ void __launch_bounds__(TPB) k_sweep3d(RunDev* __restrict__ runs, cons
   const uint32_t T0 = (uint32_t)R.sweeps;
   const int y0 = part * RPP;
   if constexpr (P > 1) {
-    // several threads per replica: one table per half sweep, double-buffered,
-    // behind a block barrier that also orders the row ranges' half sweeps (a
-    // colour-c half sweep reads the colour-(1-c) bits the other ranges just
-    // wrote); every thread of the block passes the barriers
+    // one table per half sweep, double-buffered: the block barrier after the
+    // build orders the word ranges too (a colour-c half sweep reads the
+    // colour-(1-c) words the other threads just wrote) and keeps a table
+    // until every thread has left the half sweep that reads it; every thread
+    // of the block passes the barriers
+    const auto half_sweep = [&](int t, auto c) {
+      build_tables3d<SH, TPB>(s_tab, c, 2 * t + c, 1, T0, rk);
+      __syncthreads();
+      if (live) half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + c * SH::HB + part, c, hs, rk, y0);
+    };
 #pragma unroll 1
     for (int t = 0; t < theta; ++t) {
-      const uint32_t T = T0 + (uint32_t)t;
-      hs.key = sweep_key((uint32_t)slot, T, rk);
+#pragma unroll
+      for (int k = 0; k < RP; ++k) hs.key[k] = sweep_key((uint32_t)(slot + k * SH::NC), T0 + (uint32_t)t, rk);
+      if constexpr (G != 2 || HF::S % 4 == 0) {
+        // the colour known at compile time: the addresses of a row's words
+        // and tables are then offsets of values kept over the whole launch
+        half_sweep(t, std::integral_constant<int, 0>{});
+        half_sweep(t, std::integral_constant<int, 1>{});
+      } else {
 #pragma unroll 1
-      for (uint32_t c = 0; c < 2; ++c) {
-        hs.c = c;
-        hs.half = build_half_table<GEO, TPB, P>(s_tab, 2 * t + (int)c, c, T) + part;
-        if (live) half_sweep3d<GEO, CS, RPP>(col, s_bond, hs, rk, y0);
+        for (int c = 0; c < 2; ++c) half_sweep(t, c);
       }
     }
   } else {
-    // one thread per replica: the 2 theta half sweeps in chunks of NH tables,
-    // one block barrier per chunk
+    // one thread per column: the half sweeps in chunks of NH tables, one
+    // block barrier per chunk
     const int nhalf = 2 * theta;
 #pragma unroll 1
     for (int h0 = 0; h0 < nhalf; h0 += SH::NH) {
       if (h0 > 0) __syncthreads();  // the previous chunk's tables are no longer read
       const int nh = min(SH::NH, nhalf - h0);
-      build_half_tables<GEO, TPB, P>(s_tab, h0, nh, T0);
+      build_tables3d<SH, TPB>(s_tab, 0, h0, nh, T0, rk);
+      __syncthreads();
       if (live) {
 #pragma unroll 1
         for (int j = 0; j < nh; ++j) {
-          const uint32_t c = (uint32_t)j & 1u;  // h0 is even
-          if (c == 0) hs.key = sweep_key((uint32_t)slot, T0 + (uint32_t)((h0 + j) >> 1), rk);
-          hs.c = c;
-          hs.half = half_table<GEO, P>(s_tab, j);
-          half_sweep3d<GEO, CS, RPP>(col, s_bond, hs, rk, y0);
+          const int c = j & 1;  // h0 is even
+          if (c == 0) {
+#pragma unroll
+            for (int k = 0; k < RP; ++k)
+              hs.key[k] = sweep_key((uint32_t)(slot + k * SH::NC), T0 + (uint32_t)((h0 + j) >> 1), rk);
+          }
+          half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + j * SH::HB, c, hs, rk, y0);
         }
       }
     }
   }
-  __syncthreads();  // every row range swept before the energy reads its neighbour rows
-  int E = 0;
+  __syncthreads();  // every word range swept before the energy reads its neighbours
+  // every bond joins a colour-0 and a colour-1 site: the satisfied bonds are
+  // the counts n of the colour-0 sites
+  int sat[2] = {0, 0};
   if (live) {
-    int sat = satisfied_rows<GEO, CS>(col, s_bond, y0, y0 + RPP);
+#pragma unroll 1
+    for (int y = y0; y < y0 + RPP; ++y) {
+      const int yp = row_up<GEO>(y) * CS, ym = row_down<GEO>(y) * CS;
+      static_for<0, G>([&](auto gc) {
+        constexpr int g = decltype(gc)::value, w = g;
+        // words of odd G take the mask pair of their own parity
+        const RowX<GEO> rx((uint32_t)y & 1u);
+        const Around nb = around<GEO, CS>(col + (WR + y * G) * CS, yp, ym, gc);
+        const Count3 n = count_satisfied<GEO, (g & 1)>(col[(y * G + w) * CS], nb, s_bond + 2 * (y * G + w), rx);
 #pragma unroll
-    for (int off = RW; off < 32; off <<= 1) sat += __shfl_xor_sync(hs.lanes, sat, off);
-    E = GEO::NB - 2 * sat;
-    uint4* d4 = reinterpret_cast<uint4*>(R.spins[nxt] + (size_t)slot * W);
-#pragma unroll 4
+        for (int k = 0; k < RP; ++k) {
+          const uint32_t m = HF::ONE << (16 * k);
+          sat[k] += __popc(n.n0 & m) + 2 * __popc(n.n1 & m) + 4 * __popc(n.n2 & m);
+        }
+      });
+    }
+    uint4* d4[RP];
+#pragma unroll
+    for (int k = 0; k < RP; ++k) d4[k] = reinterpret_cast<uint4*>(R.spins[nxt] + (size_t)(slot + k * SH::NC) * W);
+#pragma unroll 2
     for (int q = part; q < W / 4; q += P) {
-      uint4 v;
-      v.x = (4 * q + 0 < WR) ? col[(4 * q + 0) * CS] : 0u;
-      v.y = (4 * q + 1 < WR) ? col[(4 * q + 1) * CS] : 0u;
-      v.z = (4 * q + 2 < WR) ? col[(4 * q + 2) * CS] : 0u;
-      v.w = (4 * q + 3 < WR) ? col[(4 * q + 3) * CS] : 0u;
-      d4[q] = v;
+      uint32_t v[RP][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int w = 4 * q + i;
+        const bool in = w < WR;
+        const uint32_t e = (uint32_t)(w / G + w % G) & 1u;
+        const uint32_t a = in ? (uint32_t)col[w * CS] : 0u, b = in ? (uint32_t)col[(WR + w) * CS] : 0u;
+        v[0][i] = place_colour<GEO, 0>(a, e) | place_colour<GEO, 0>(b, e ^ 1u);
+        if constexpr (RP == 2) v[RP - 1][i] = place_colour<GEO, 1>(a, e) | place_colour<GEO, 1>(b, e ^ 1u);
+      }
+#pragma unroll
+      for (int k = 0; k < RP; ++k)
+        if (slot + k * SH::NC < Rn) d4[k][q] = make_uint4(v[k][0], v[k][1], v[k][2], v[k][3]);
     }
   }
-  measure_store(R, nxt, slot, live && part == 0, E);
+  // sum over the row ranges, then record one replica per thread
+  int* s_sat = reinterpret_cast<int*>(s_tab);  // [P][NR]; the tables are no longer read
+  if (part < P) {
+#pragma unroll
+    for (int k = 0; k < RP; ++k) s_sat[part * SH::NR + k * SH::NC + r] = sat[k];
+  }
+  __syncthreads();
+  if ((tid & ~31) >= SH::NR) return;  // whole warps
+  int E = GEO::NB;
+  const bool rec = tid < SH::NR && first + tid < Rn;
+  if (rec)
+    for (int q = 0; q < P; ++q) E -= 2 * s_sat[q * SH::NR + tid];
+  measure_store(R, nxt, first + tid, rec, E);
 }
 
 // Sec. 2: R0 independent uniformly random microstates at beta = 0.  Word w of
 // slot s is word (w mod 4) of Philox(ctr = (w div 4, s, 0, TAG_INIT)),
-// restricted to the valid lanes.
+// restricted to the valid lanes.  One thread per slot of a work item.
 template <int L, int TPB>
-__global__ void __launch_bounds__(TPB) k_init3d(RunDev* __restrict__ runs, const Work* __restrict__ table) {
+__global__ void __launch_bounds__(TPB) k_init3d(RunDev* __restrict__ runs, const Work* __restrict__ table,
+                                                int slots) {
   using GEO = Geo3<L>;
   constexpr int WR = GEO::WR, W = GEO::W;
   extern __shared__ uint32_t smem[];
@@ -426,7 +674,7 @@ __global__ void __launch_bounds__(TPB) k_init3d(RunDev* __restrict__ runs, const
   const int tid = threadIdx.x;
   for (int i = tid; i < 6 * W; i += TPB) s_bond[i] = R.bonds[i];
   const int64_t slot = (int64_t)wk.first + tid;
-  const bool live = slot < R0;
+  const bool live = tid < slots && slot < R0;
   uint32_t* col = s_spin + tid;
   if (live) {
     for (int w4 = 0; w4 < W / 4; ++w4) {
@@ -452,62 +700,106 @@ inline size_t init3d_smem() {
   return sizeof(uint32_t) * (6 * GEO::W + GEO::WR * TPB);
 }
 
-// One launch over nwork work items (TPB slots each); the dynamic shared
-// memory limit is raised where the kernel needs more than 48 KiB (also when
-// nwork is 0, so that it can be set outside a stream capture).
-template <int L, int TPB, int P>
-cudaError_t launch_sweep3d_p(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
-  if constexpr (!split_ok<Geo3<L>>(P) || TPB / P < 4 || (P > 1 && TPB < 64)) {
+// One launch over nwork work items (with nwork <= 0 only the dynamic shared
+// memory limit is raised, outside any stream capture).
+template <int L, int TPB, int P, int RP>
+cudaError_t sweep3d_p(const Sweep3dLaunch& a) {
+  if constexpr (!rows_split<Geo3<L>>(P)) {
+    return cudaErrorInvalidValue;
+  } else if constexpr (!SweepShape<L, TPB, P, RP>::OK) {
     return cudaErrorInvalidValue;
   } else {
-    const size_t sm = sizeof(uint32_t) * SweepShape<L, TPB, P>::SMEM_WORDS;
-    if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute((const void*)k_sweep3d<L, TPB, P>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
+    using SH = SweepShape<L, TPB, P, RP>;
+    const int sm = (int)(sizeof(uint32_t) * SH::SMEM_WORDS);
+    if (a.nwork <= 0) {
+      if (sm <= 48 * 1024) return cudaSuccess;
+      return cudaFuncSetAttribute((const void*)k_sweep3d<L, TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  sm);
     }
-    if (nwork <= 0) return cudaSuccess;
-    k_sweep3d<L, TPB, P><<<nwork * P, TPB, sm, st>>>(runs, table);
+    k_sweep3d<L, TPB, P, RP><<<a.nwork * SH::BPI, TPB, sm, a.st>>>(a.runs, a.table);
     return cudaGetLastError();
   }
 }
 
 template <int L, int TPB>
-cudaError_t launch_sweep3d_t(RunDev* runs, const Work* table, int nwork, cudaStream_t st, bool init, int split) {
-  if (init) {
-    const size_t sm = init3d_smem<L, TPB>();
-    if (sm > 48 * 1024) {
-      cudaError_t e =
-          cudaFuncSetAttribute((const void*)k_init3d<L, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      if (e != cudaSuccess) return e;
-    }
-    if (nwork <= 0) return cudaSuccess;
-    k_init3d<L, TPB><<<nwork, TPB, sm, st>>>(runs, table);
-    return cudaGetLastError();
+cudaError_t launch_init3d_t(int slots, RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
+  const size_t sm = init3d_smem<L, TPB>();
+  if (sm > 48 * 1024) {
+    cudaError_t e =
+        cudaFuncSetAttribute((const void*)k_init3d<L, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
   }
-  switch (split) {
-    case 1: return launch_sweep3d_p<L, TPB, 1>(runs, table, nwork, st);
-    case 2: return launch_sweep3d_p<L, TPB, 2>(runs, table, nwork, st);
-    case 4: return launch_sweep3d_p<L, TPB, 4>(runs, table, nwork, st);
-    case 8: return launch_sweep3d_p<L, TPB, 8>(runs, table, nwork, st);
+  if (nwork <= 0) return cudaSuccess;
+  k_init3d<L, TPB><<<nwork, TPB, sm, st>>>(runs, table, slots);
+  return cudaGetLastError();
+}
+
+template <int L, int TPB>
+cudaError_t sweep3d_t(const Sweep3dLaunch& a) {
+  const bool one = a.rp == 1;
+  switch (a.split) {
+    case 1: return one ? sweep3d_p<L, TPB, 1, 1>(a) : cudaErrorInvalidValue;
+    case 2: return one ? sweep3d_p<L, TPB, 2, 1>(a) : sweep3d_p<L, TPB, 2, 2>(a);
+    case 4: return one ? sweep3d_p<L, TPB, 4, 1>(a) : sweep3d_p<L, TPB, 4, 2>(a);
+    case 8: return one ? sweep3d_p<L, TPB, 8, 1>(a) : sweep3d_p<L, TPB, 8, 2>(a);
     default: return cudaErrorInvalidValue;
   }
 }
 
+// Further splits, not powers of two: whole pairs of rows where a row's
+// uniforms end within a call (L = 6, 10, 14), one or two rows at L = 12.
+template <int L>
+constexpr bool extra_split(int P) {
+  return (L == 6 && P == 3) || (L == 10 && P == 5) || (L == 14 && P == 7) || (L == 12 && (P == 6 || P == 12));
+}
+
+template <int L, int P>
+cudaError_t sweep3d_extra(const Sweep3dLaunch& a) {
+  if constexpr (extra_split<L>(P)) {
+    const bool one = a.rp == 1;
+    switch (a.tpb) {
+      case 64: return one ? sweep3d_p<L, 64, P, 1>(a) : sweep3d_p<L, 64, P, 2>(a);
+      case 128: return one ? sweep3d_p<L, 128, P, 1>(a) : sweep3d_p<L, 128, P, 2>(a);
+      case 256: return one ? sweep3d_p<L, 256, P, 1>(a) : sweep3d_p<L, 256, P, 2>(a);
+    }
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <int L>
+cudaError_t sweep3d_any(const Sweep3dLaunch& a) {
+  switch (a.split) {
+    case 3: return sweep3d_extra<L, 3>(a);
+    case 5: return sweep3d_extra<L, 5>(a);
+    case 6: return sweep3d_extra<L, 6>(a);
+    case 7: return sweep3d_extra<L, 7>(a);
+    case 12: return sweep3d_extra<L, 12>(a);
+  }
+  switch (a.tpb) {
+    case 32: return sweep3d_t<L, 32>(a);
+    case 64: return sweep3d_t<L, 64>(a);
+    case 128: return sweep3d_t<L, 128>(a);
+    case 256: return sweep3d_t<L, 256>(a);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int L>
+cudaError_t launch_init3d(int slots, RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
+  if (slots <= 32) return launch_init3d_t<L, 32>(slots, runs, table, nwork, st);
+  if (slots <= 64) return launch_init3d_t<L, 64>(slots, runs, table, nwork, st);
+  if (slots <= 128) return launch_init3d_t<L, 128>(slots, runs, table, nwork, st);
+  return slots <= 256 ? launch_init3d_t<L, 256>(slots, runs, table, nwork, st) : cudaErrorInvalidValue;
+}
+
 }  // namespace pa
 
-// Threads per replica the sweep kernel supports for edge L (1, 2, 4, 8).
 #define PA_INSTANTIATE_SWEEP3D(LL)                                                                        \
   namespace pa {                                                                                          \
-  cudaError_t launch_sweep3d_L##LL(int tpb, int split, RunDev* runs, const Work* table, int nwork,       \
-                                   cudaStream_t st, bool init) {                                          \
-    switch (tpb) {                                                                                        \
-      case 32: return launch_sweep3d_t<LL, 32>(runs, table, nwork, st, init, split);                      \
-      case 64: return launch_sweep3d_t<LL, 64>(runs, table, nwork, st, init, split);                      \
-      case 128: return launch_sweep3d_t<LL, 128>(runs, table, nwork, st, init, split);                    \
-      case 256: return launch_sweep3d_t<LL, 256>(runs, table, nwork, st, init, split);                    \
-      default: return cudaErrorInvalidValue;                                                              \
-    }                                                                                                     \
+  cudaError_t sweep3d_L##LL(const Sweep3dLaunch& a) { return sweep3d_any<LL>(a); }                        \
+  cudaError_t launch_init3d_L##LL(int slots, RunDev* runs, const Work* table, int nwork,                  \
+                                  cudaStream_t st) {                                                      \
+    return launch_init3d<LL>(slots, runs, table, nwork, st);                                              \
   }                                                                                                       \
-  bool sweep3d_split_ok_L##LL(int split) { return split_ok<Geo3<LL>>(split); }                            \
+  bool sweep3d_split_ok_L##LL(int split) { return split_ok<Geo3<LL>>(split) || extra_split<LL>(split); } \
   }

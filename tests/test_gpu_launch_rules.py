@@ -1,0 +1,33 @@
+"""Launch shapes the library chooses by itself (GPU): the +-1 cubic sweep with
+one and with two replicas per thread, at every edge, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle as o
+from paper_1006_0252_gb300 import inputs, pa
+
+pytestmark = pytest.mark.gpu
+
+
+# (L, R0, threads per replica): the largest odd populations that take one
+# replica a thread (R0 P <= 900 x 152) and the smallest that take two, whose
+# last columns hold one replica; L = 12 also past 50000, where it splits less.
+@pytest.mark.parametrize("L,R0,split", [(2, 4001, 1), (4, 34199, 4), (4, 34201, 4), (6, 45601, 3), (8, 17099, 8),
+                                        (8, 17101, 8), (10, 27361, 5), (12, 11401, 12), (12, 50001, 6),
+                                        (14, 19543, 7), (16, 17101, 8)])
+def test_chosen_shape_bit_exact(L, R0, split):
+    """One sweep each where every compare runs, where the thr(8) and thr(12)
+    compares are mostly skipped, and where the minimum skips all of them."""
+    J = inputs.couplings_3d(L, 2, 9)
+    cap = R0 + 4000
+    g = pa.Run(J, L, 3, R0, 23, R_cap=cap)
+    assert pa.pa_sweep_shape(g._h)[1] == split
+    c = o.Run(J, 3, L, L, L, 7, R0=R0, R_cap=cap, seed=23)
+    for beta, sweeps in ((0.1, 1), (0.5, 0), (0.9, 0), (1.2, 0), (1.5, 1), (1.9, 0), (2.6, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+    go, co = g.observables(), c.state()
+    assert go["R"] == co.R and go["sumE"] == co.sumE and go["sumE2"] == co.sumE2
+    assert np.array_equal(g.energies(), c.energies())
+    assert np.array_equal(g.spins(), c.spins())
+    assert abs(go["minus_beta_F"] - co.minus_beta_F) <= 1e-12 * abs(co.minus_beta_F)
