@@ -295,11 +295,14 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
     float best = 1e30f;
     LaunchShape pick = {c.tpb, c.split, c.rp};
     LatticeClass trial = c;
+    std::vector<int64_t> R0;
+    for (int32_t r : c.runs) R0.push_back(E.R0[r]);
     for (const LaunchShape& cand : launch_shapes(c)) {
       if (cand.split == 1 && cand.tpb == 256) continue;
       trial.tpb = cand.tpb;
       trial.split = cand.split;
       trial.rp = cand.rp;
+      spread_blocks(trial, R0);
       trial.d_table = nullptr;
       int st = prepare_class_launch(E.d_runs, E.st, trial);
       if (st == PA_OK) st = build_class_table(E, trial);
@@ -326,6 +329,7 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
       c.tpb = pick.tpb;
       c.split = pick.split;
       c.rp = pick.rp;
+      spread_blocks(c, R0);
       int st = build_class_table(E, c);
       if (st != PA_OK) return st;
     }

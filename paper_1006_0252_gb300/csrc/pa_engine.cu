@@ -394,6 +394,8 @@ bool tpb_supported(const LatticeClass& c, int tpb) {
 }
 
 static bool pm_cubic(const LatticeClass& c) { return c.dim == 3 && c.bx == 0 && c.model == 0; }
+// Classes whose sweep kernel can hold two replicas in a thread.
+static bool sweeps_pairs(const LatticeClass& c) { return c.bx == 0 && c.model == 0; }
 
 static cudaError_t sweep3d_call(int L, const Sweep3dLaunch& a) {
   switch (L) {
@@ -427,15 +429,36 @@ static int pm_split(int L, int64_t replicas) {
   }
 }
 
-// Launch shape of a class of `replicas` slots (the sum of its runs' target
-// populations) before any autotuning.  Gaussian cubic sweeps run 4 threads
+// While a launch's blocks fit the SMs at once, the SM that gets the most of
+// them sets its time, and the hardware does not deal them out evenly: 296
+// blocks of 256 threads, two an SM, ran 1.44 times as long wherever three
+// fitted one.  So a block asks for as much shared memory as leaves an SM no
+// room for more than its even share of the blocks that hold replicas (a
+// population stays within three standard deviations, sqrt(R0), of its target;
+// a larger one only takes longer).  With more blocks than that it changes
+// nothing.
+void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
+  constexpr int SM_SMEM = 228 * 1024, BLOCK_RESERVED = 1024;
+  c.min_smem = 0;
+  if (!sweeps_pairs(c)) return;
+  const int64_t per_block = c.tpb / c.split * c.rp;
+  int64_t blocks = 0;
+  for (int64_t r : R0) blocks += (r + (int64_t)(3.0 * std::sqrt((double)r)) + per_block - 1) / per_block;
+  const int64_t most = std::max<int64_t>(1, (blocks + NUM_SMS - 1) / NUM_SMS);
+  c.min_smem = std::max<int>(0, std::min<int>((int)SMEM_LIMIT, (int)(SM_SMEM / most) / 128 * 128 - BLOCK_RESERVED));
+}
+
+// Launch shape of a class before any autotuning; R0: the target populations
+// of its runs.  Gaussian cubic sweeps run 4 threads
 // per replica where the rows split so, which keeps enough warps resident to
 // hide the latency of the generator's dependent multiplies (the
 // threshold-table kernel two of 512); +-1 chains 4 or 8 on ranges of words;
 // other classes 1.
-void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, int64_t replicas) {
+void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0) {
   c.split = 1;
   c.rp = 1;
+  int64_t replicas = 0;
+  for (int64_t r : R0) replicas += r;
   if (split_opt > 0) {
     c.split = split_supported(c, split_opt) ? split_opt : 1;
   } else if (pm_cubic(c)) {
@@ -448,21 +471,24 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, int64_t rep
     if (split_supported(c, 4)) c.split = 4;
   } else if (c.dim == 1 && c.model == 0) {
     // +-1 chains: the word ranges keep the uniform tables and the columns of
-    // a block within shared memory at long chains
-    c.split = c.Wr >= 16 ? 8 : (c.Wr >= 4 ? 4 : 1);
+    // a block within shared memory at long chains (8 rather than 4 ranges of
+    // 8 words: 25 against 33 us at 2000 replicas of 256 spins, 3 % at 20000)
+    c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : 1);
   }
   if (tpb_opt && tpb_supported(c, tpb_opt)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
   else if (c.dim == 3 && c.model == 1 && c.L <= 8) c.tpb = 512;
-  else if (pm_cubic(c)) c.tpb = c.L == 10 ? 256 : 128;  // 5 threads a replica leave 3 of 128 idle, 1 of 256
+  else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * NUM_SMS ? 256 : 128;  // 5 threads a replica: 25 or 51 of
+                                                                                  // them a block
   else if (c.split > 1) c.tpb = 128;
   else c.tpb = default_tpb(c.dim, c.L);
   if (c.tpb / c.split < 4 || (c.split > 1 && c.tpb < 64)) c.split = 1;
-  // Two replicas a thread share the lattice work of a word (6-15 % fewer
-  // instructions a flip) but halve the threads: taken once one replica a
+  // Two replicas a thread share the lattice work of a word (6-15 % less time a
+  // flip in full launches) but halve the threads: taken once one replica a
   // thread gives more than 900 threads an SM (28 warps; both are within 5 %
   // of each other from 600 to 1200).
-  if (pm_cubic(c) && c.split > 1 && replicas * c.split > (int64_t)900 * NUM_SMS) c.rp = 2;
+  if (sweeps_pairs(c) && c.split > 1 && replicas * c.split > (int64_t)900 * NUM_SMS) c.rp = 2;
+  spread_blocks(c, R0);
 }
 
 // Every launch shape the sweep kernel of a class has.
@@ -474,7 +500,7 @@ std::vector<LaunchShape> launch_shapes(const LatticeClass& c) {
       if (!tpb_supported(c, tpb)) continue;
       if (split > 1 && (tpb < 64 || tpb / split < 4)) continue;
       v.push_back({tpb, split, 1});
-      if (pm_cubic(c) && split > 1) v.push_back({tpb, split, 2});
+      if (sweeps_pairs(c) && split > 1) v.push_back({tpb, split, 2});
     }
   }
   return v;
@@ -527,7 +553,7 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
       default: return fail(PA_ERR_UNSUPPORTED, "no Gaussian kernel for L=%d", c.L);
     }
   } else if (c.dim == 1) {
-    err = launch_sweep1d(tpb, c.split, runs, table, nwork, c.W, c.Wr, st, init);
+    err = launch_sweep1d(tpb, c.split, c.rp, runs, table, nwork, c.W, c.Wr, st, init, c.min_smem);
   } else if (init) {
     switch (c.L) {
       case 2: err = launch_init3d_L2(tpb, runs, table, nwork, st); break;
@@ -541,7 +567,7 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
       default: return fail(PA_ERR_UNSUPPORTED, "no kernel for L=%d", c.L);
     }
   } else {
-    err = sweep3d_call(c.L, {tpb, c.split, c.rp, runs, table, nwork, st});
+    err = sweep3d_call(c.L, {tpb, c.split, c.rp, runs, table, nwork, c.min_smem, st});
   }
   if (err != cudaSuccess) return cuda_fail(err, "sweep kernel launch");
   return PA_OK;
@@ -680,9 +706,9 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
     it->runs.push_back(r);
   }
   for (auto& c : E.cls) {
-    int64_t replicas = 0;
-    for (int32_t r : c.runs) replicas += E.R0[r];
-    set_default_launch(c, tpb_opt, split_opt, replicas);
+    std::vector<int64_t> R0;
+    for (int32_t r : c.runs) R0.push_back(E.R0[r]);
+    set_default_launch(c, tpb_opt, split_opt, R0);
     if (split_opt > 1 && c.split != split_opt)
       return fail(PA_ERR_INVALID, "%d threads per replica do not split the rows of this lattice or block", split_opt);
     st = build_class_table(E, c);

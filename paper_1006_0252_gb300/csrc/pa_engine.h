@@ -42,8 +42,8 @@ cudaError_t launch_weighted_pairs(int G, int M, const double* x1, const double* 
 cudaError_t launch_bootstrap(int M, const double* x, const double* A, const double* Rw, int B, uint64_t seed,
                              double* bmean, double* bfbar, cudaStream_t st, int GK = 1);
 bool sweep1d_split_ok(int split);
-cudaError_t launch_sweep1d(int tpb, int split, RunDev* runs, const Work* table, int nwork, int W, int WR,
-                           cudaStream_t st, bool init);
+cudaError_t launch_sweep1d(int tpb, int split, int rp, RunDev* runs, const Work* table, int nwork, int W, int WR,
+                           cudaStream_t st, bool init, int min_smem);
 cudaError_t launch_setup_gauss3d(const int32_t* J, int L, int32_t* gJ, int32_t* gS, cudaStream_t st);
 cudaError_t launch_gprep_head(RunDev* runs, const int32_t* ids, int n, bool ovr, double beta, int theta, int64_t Rt,
                               cudaStream_t st);
@@ -150,7 +150,8 @@ struct LatticeClass {
   int max_tpb = 256;                        // largest block whose shared memory fits
   int tpb = 0;
   int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
-  int rp = 1;        // +-1 cubic lattices: replicas a thread sweeps side by side (1, 2)
+  int rp = 1;        // +-1 cubic lattices and chains: replicas a thread sweeps side by side (1, 2)
+  int min_smem = 0;  // shared memory of a sweep block that keeps the blocks even over the SMs (spread_blocks)
   std::vector<int32_t> runs;
   Work* d_table = nullptr;
   int nwork = 0;
@@ -284,7 +285,8 @@ size_t run_slab_bytes(const Geometry& g, int64_t cap, int max_steps);
 int setup_run(char* base, const Geometry& g, const pa_run_spec& s, int64_t cap, int max_steps,
               cudaStream_t st, RunDev* out);
 int default_tpb(int dim, int L);
-void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, int64_t replicas);
+void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0);
+void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0);
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c);
 bool split_supported(const LatticeClass& c, int split);
 bool tpb_supported(const LatticeClass& c, int tpb);

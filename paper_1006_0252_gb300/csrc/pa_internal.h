@@ -116,12 +116,14 @@ struct Work {
 
 // A launch of the +-1 cubic sweep kernel: tpb threads per block, split of them
 // sharing the rp replicas of a column; nwork work items (nwork <= 0 only
-// prepares the kernel for launches).
+// prepares the kernel for launches); at least min_smem bytes of shared memory
+// a block.
 struct Sweep3dLaunch {
   int tpb, split, rp;
   RunDev* runs;
   const Work* table;
   int nwork;
+  int min_smem;
   cudaStream_t st;
 };
 

@@ -317,4 +317,61 @@ __device__ __forceinline__ void measure_store(RunDev& R, int nxt, int64_t slot, 
   }
 }
 
+// ---------------------------------------------------------------------------
+// Colour words: the colour-c sites of one packed word by rank, of one replica
+// in bits 0..15 and, with RP = 2, of a second one in bits 16..31.
+// ---------------------------------------------------------------------------
+template <int RP>
+using ColourWord = typename std::conditional<RP == 1, uint16_t, uint32_t>::type;
+
+// RP words with bits at even positions 2m only, as one colour word, and
+// replica K_ of a colour word back at even positions.
+template <int RP>
+__device__ __forceinline__ uint32_t gather_even(const uint32_t (&v)[RP]) {
+  uint32_t x[2] = {0u, 0u};
+#pragma unroll
+  for (int k = 0; k < RP; ++k) {
+    x[k] = (v[k] | (v[k] >> 1)) & 0x33333333u;
+    x[k] = (x[k] | (x[k] >> 2)) & 0x0F0F0F0Fu;
+    x[k] = x[k] | (x[k] >> 4);  // ranks 0-7 in byte 0, 8-15 in byte 2
+  }
+  return __byte_perm(x[0], x[1], 0x6420u);
+}
+template <int K_>
+__device__ __forceinline__ uint32_t spread_even(uint32_t a) {
+  uint32_t x = __byte_perm(a, 0u, K_ == 0 ? 0x4140u : 0x4342u);
+  x = (x | (x << 4)) & 0x0F0F0F0Fu;
+  x = (x | (x << 2)) & 0x33333333u;
+  return (x | (x << 1)) & 0x55555555u;
+}
+
+// ---------------------------------------------------------------------------
+// Threshold compares.  Bit m of ge is [u_m >= thr]: the subtraction u_m - thr
+// sets the carry exactly when it does not borrow, and ge = 2 ge + carry
+// shifts it in; both run at the full integer rate, where a compare into a
+// predicate and a select would each take a half-rate slot.
+// ---------------------------------------------------------------------------
+template <int SITES, int OFF>
+__device__ __forceinline__ uint32_t lt_mask(const uint32_t* u, uint32_t thr) {
+  static_assert(SITES <= 16, "at most 16 colour-c sites per word");
+  uint32_t ge = 0u;
+#pragma unroll
+  for (int m = SITES - 1; m >= 0; --m)
+    asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, %3;\n\t}"
+        : "=r"(ge)
+        : "r"(u[OFF + m]), "r"(thr), "r"(ge));
+  return ge ^ ((1u << SITES) - 1u);
+}
+
+// Minimum of u[OFF .. OFF+N-1], folded three at a time (one instruction for
+// three values).
+template <int N, int OFF>
+__device__ __forceinline__ uint32_t min_of(const uint32_t* u) {
+  uint32_t m = u[OFF];
+#pragma unroll
+  for (int i = 1; i + 1 < N; i += 2) m = __vimin3_u32(m, u[OFF + i], u[OFF + i + 1]);
+  if constexpr ((N & 1) == 0) m = min(m, u[OFF + N - 1]);
+  return m;
+}
+
 }  // namespace pa

@@ -128,9 +128,9 @@ static int server_rebuild_tables(pa_server* S) {
   }
   for (size_t k = 0; k < S->cls.size(); ++k) {
     LatticeClass& c = S->cls[k];
-    int64_t replicas = 0;
-    for (int32_t sl : c.runs) replicas += S->h[sl].R;
-    set_default_launch(c, S->tpb_opt, S->split_opt, replicas);  // the shape follows the runs that are active
+    std::vector<int64_t> R0;
+    for (int32_t sl : c.runs) R0.push_back(S->h[sl].R);
+    set_default_launch(c, S->tpb_opt, S->split_opt, R0);  // the shape follows the runs that are active
     if (!c.runs.empty()) {
       const int st = prepare_class_launch(S->d_runs, S->st, c);
       if (st != PA_OK) return st;

@@ -171,31 +171,18 @@ struct RowX {
   }
 };
 
-// Element of a column: RP replicas' sites of one colour of one word.
-template <int RP>
-using ColourWord = typename std::conditional<RP == 1, uint16_t, uint32_t>::type;
-
 // Two replicas' packed words as the colour-c word (e = (c + y + g) mod 2),
 // and the packed words of the replicas back from a colour word.
 template <class GEO, int RP>
 __device__ __forceinline__ uint32_t take_colour(const uint32_t (&v)[RP], uint32_t e) {
-  uint32_t x[2] = {0u, 0u};
+  uint32_t x[RP];
 #pragma unroll
-  for (int k = 0; k < RP; ++k) {
-    x[k] = from_colour_positions<GEO>(v[k], e);  // sites at even positions 2m
-    x[k] = (x[k] | (x[k] >> 1)) & 0x33333333u;
-    x[k] = (x[k] | (x[k] >> 2)) & 0x0F0F0F0Fu;
-    x[k] = x[k] | (x[k] >> 4);  // ranks 0-7 in byte 0, 8-15 in byte 2
-  }
-  return __byte_perm(x[0], x[1], 0x6420u);
+  for (int k = 0; k < RP; ++k) x[k] = from_colour_positions<GEO>(v[k], e);  // sites at even positions 2m
+  return gather_even<RP>(x);
 }
 template <class GEO, int K_>
 __device__ __forceinline__ uint32_t place_colour(uint32_t a, uint32_t e) {  // replica K_ (0 or 1)
-  uint32_t x = __byte_perm(a, 0u, K_ == 0 ? 0x4140u : 0x4342u);
-  x = (x | (x << 4)) & 0x0F0F0F0Fu;
-  x = (x | (x << 2)) & 0x33333333u;
-  x = (x | (x << 1)) & 0x55555555u;
-  return to_colour_positions<GEO>(x, e);
+  return to_colour_positions<GEO>(spread_even<K_>(a), e);
 }
 
 // Bond masks of the colour words, one 32-byte entry for (c, w): the x bond to
@@ -270,35 +257,6 @@ __device__ __forceinline__ Count3 count_satisfied(uint32_t s, const Around& n, c
   const uint32_t sb = b3 ^ b4 ^ b5, cb = (b3 & b4) | (b5 & (b3 ^ b4));
   const uint32_t n0 = sa ^ sb, c0 = sa & sb;
   return {n0, ca ^ cb ^ c0, (ca & cb) | (c0 & (ca ^ cb))};
-}
-
-// ---------------------------------------------------------------------------
-// Threshold compares.  Bit m of ge is [u_m >= thr]: the subtraction u_m - thr
-// sets the carry exactly when it does not borrow, and ge = 2 ge + carry
-// shifts it in; both run at the full integer rate, where a compare into a
-// predicate and a select would each take a half-rate slot.
-// ---------------------------------------------------------------------------
-template <int SITES, int OFF>
-__device__ __forceinline__ uint32_t lt_mask(const uint32_t* u, uint32_t thr) {
-  static_assert(SITES <= 16, "at most 16 colour-c sites per word");
-  uint32_t ge = 0u;
-#pragma unroll
-  for (int m = SITES - 1; m >= 0; --m)
-    asm("{\n\t.reg .u32 t;\n\tsub.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, %3;\n\t}"
-        : "=r"(ge)
-        : "r"(u[OFF + m]), "r"(thr), "r"(ge));
-  return ge ^ ((1u << SITES) - 1u);
-}
-
-// Minimum of u[OFF .. OFF+N-1], folded three at a time (one instruction for
-// three values).
-template <int N, int OFF>
-__device__ __forceinline__ uint32_t min_of(const uint32_t* u) {
-  uint32_t m = u[OFF];
-#pragma unroll
-  for (int i = 1; i + 1 < N; i += 2) m = __vimin3_u32(m, u[OFF + i], u[OFF + i + 1]);
-  if constexpr ((N & 1) == 0) m = min(m, u[OFF + N - 1]);
-  return m;
 }
 
 // Everything a word's update needs beyond the lattice: the slots' keys and the
@@ -453,25 +411,21 @@ struct SweepShape {
   static constexpr int BOND_WORDS = 16 * GEO::WR;
   static constexpr int SPIN_WORDS = (GEO::WR * CS * RP + 3) / 4 * 4;  // [2 colours][WR][CS] colour words
   static constexpr int Q = calls_per_colour<GEO>();
-  // entries of one half-sweep table: one padding entry after each thread's
-  // range puts the ranges' reads on different banks
-  static constexpr int RANGE = P == 1 ? Q : WPP * Half<GEO>::S / 4;
-  static constexpr int HB = Q + Q / RANGE + 1;
   // half-sweep tables held at once: with one thread per column as many as
   // fit, else two, double-buffered behind one block barrier per half sweep
   static constexpr int room() {
-    const int n = (216 * TPB - 4 * (BOND_WORDS + SPIN_WORDS)) / (16 * HB);
+    const int n = (216 * TPB - 4 * (BOND_WORDS + SPIN_WORDS)) / (16 * Q);
     return n >= 20 ? 20 : (n < 2 ? 2 : (n & ~1));
   }
   static constexpr int NH = P > 1 ? 2 : room();
   // the tables' memory also takes the row ranges' energies at the end
-  static constexpr int TAB_WORDS = 4 * NH * HB > RP * TPB ? 4 * NH * HB : RP * TPB;
+  static constexpr int TAB_WORDS = 4 * NH * Q > RP * TPB ? 4 * NH * Q : RP * TPB;
   static constexpr size_t SMEM_WORDS = (size_t)TAB_WORDS + BOND_WORDS + SPIN_WORDS;
   static constexpr bool OK = SLOTS % NR == 0 && NR <= TPB && NC >= 4 && (P == 1 || TPB >= 64);
 };
 
 // Half-sweep tables h0 .. h0 + nh - 1 (half sweep h = 2t + c is colour c of
-// sweep T0 + t) at tab[j HB + q + q / RANGE], all threads of the block.
+// sweep T0 + t) at tab[(buf + j) Q + q], all threads of the block.
 template <class SH, int TPB>
 __device__ __forceinline__ void build_tables3d(uint4* __restrict__ tab, int buf, int h0, int nh, uint32_t T0,
                                                const RoundKeys& rk) {
@@ -479,7 +433,7 @@ __device__ __forceinline__ void build_tables3d(uint4* __restrict__ tab, int buf,
     const int j = i / SH::Q, q = i - j * SH::Q;
     const int h = h0 + j;
     const uint32_t A1 = PHILOX_MUL1 * (T0 + (uint32_t)(h >> 1));
-    tab[(buf + j) * SH::HB + q + q / SH::RANGE] =
+    tab[(buf + j) * SH::Q + q] =
         sweep_half_entry(sweep_call_entry((uint32_t)q, TAG_SWEEP + (uint32_t)(h & 1), rk), A1);
   }
 }
@@ -560,7 +514,7 @@ __global__ void __launch_bounds__(TPB) k_sweep3d(RunDev* __restrict__ runs, cons
     const auto half_sweep = [&](int t, auto c) {
       build_tables3d<SH, TPB>(s_tab, c, 2 * t + c, 1, T0, rk);
       __syncthreads();
-      if (live) half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + c * SH::HB + part, c, hs, rk, y0);
+      if (live) half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + c * SH::Q, c, hs, rk, y0);
     };
 #pragma unroll 1
     for (int t = 0; t < theta; ++t) {
@@ -595,7 +549,7 @@ __global__ void __launch_bounds__(TPB) k_sweep3d(RunDev* __restrict__ runs, cons
             for (int k = 0; k < RP; ++k)
               hs.key[k] = sweep_key((uint32_t)(slot + k * SH::NC), T0 + (uint32_t)((h0 + j) >> 1), rk);
           }
-          half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + j * SH::HB, c, hs, rk, y0);
+          half_sweep3d<GEO, CS, RP, RPP>(col, s_bond, s_tab + j * SH::Q, c, hs, rk, y0);
         }
       }
     }
@@ -710,7 +664,7 @@ cudaError_t sweep3d_p(const Sweep3dLaunch& a) {
     return cudaErrorInvalidValue;
   } else {
     using SH = SweepShape<L, TPB, P, RP>;
-    const int sm = (int)(sizeof(uint32_t) * SH::SMEM_WORDS);
+    const int need = (int)(sizeof(uint32_t) * SH::SMEM_WORDS), sm = need > a.min_smem ? need : a.min_smem;
     if (a.nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
       return cudaFuncSetAttribute((const void*)k_sweep3d<L, TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -1,5 +1,5 @@
-"""Launch shapes the library chooses by itself (GPU): the +-1 cubic sweep with
-one and with two replicas per thread, at every edge, against the oracle."""
+"""Launch shapes the library chooses by itself (GPU): the +-1 cubic and chain
+sweeps with one and with two replicas per thread against the oracle."""
 import numpy as np
 import pytest
 
@@ -31,3 +31,23 @@ def test_chosen_shape_bit_exact(L, R0, split):
     assert np.array_equal(g.energies(), c.energies())
     assert np.array_equal(g.spins(), c.spins())
     assert abs(go["minus_beta_F"] - co.minus_beta_F) <= 1e-12 * abs(co.minus_beta_F)
+
+
+# (N, open, R0): chains of 3, 5, 8, 32 and 128 words, short last words, odd
+# length, one and two replicas a thread.
+@pytest.mark.parametrize("N,is_open,R0", [(70, False, 40001), (130, True, 34201), (256, False, 17099),
+                                          (256, False, 17101), (1001, True, 17101), (1000, False, 17101),
+                                          (4096, True, 17101), (4094, False, 17103)])
+def test_chosen_chain_shape_bit_exact(N, is_open, R0):
+    J = inputs.couplings_chain(N, 2, 9, open_chain=is_open)
+    J[N // 3] = 0  # a diluted chain: two sites inside have one bond
+    cap = R0 + 4000
+    g = pa.Run(J, N, 1, R0, 29, R_cap=cap)
+    c = o.Run(J, 1, N, R0=R0, R_cap=cap, seed=29)
+    for beta, sweeps in ((0.1, 1), (0.5, 0), (1.0, 1), (1.5, 0), (2.0, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+    go, co = g.observables(), c.state()
+    assert go["R"] == co.R and go["sumE"] == co.sumE and go["sumE2"] == co.sumE2
+    assert np.array_equal(g.energies(), c.energies())
+    assert np.array_equal(g.spins(), c.spins())
