@@ -380,7 +380,7 @@ int default_tpb(int dim, int L) {
 // Block sizes the sweep kernels of a class support: 32 .. 256 threads for
 // every class (general boxes and Gaussian chains up to what their
 // shared-memory tables allow);
-// 512 and 1024 too for Gaussian cubic lattices of L <= 8, whose kernel at
+// 512 and 1024 too for Gaussian cubic lattices of L <= 10, whose kernel at
 // those sizes tabulates the acceptance thresholds of every site and pattern
 // in shared memory (the table is shared by all the block's replicas).
 bool tpb_supported(const LatticeClass& c, int tpb) {
@@ -389,11 +389,14 @@ bool tpb_supported(const LatticeClass& c, int tpb) {
     if (c.dim == 1 && c.model == 1) return gauss1d_smem_bytes(tpb, c.Wr) <= SMEM_LIMIT;
     return true;
   }
-  if (tpb == 512 || tpb == 1024) return c.bx == 0 && c.dim == 3 && c.model == 1 && c.L <= 8;
+  if (tpb == 512 || tpb == 1024) return c.bx == 0 && c.dim == 3 && c.model == 1 && c.L <= 10;
   return false;
 }
 
 static bool pm_cubic(const LatticeClass& c) { return c.dim == 3 && c.bx == 0 && c.model == 0; }
+static bool gauss_cubic(const LatticeClass& c) { return c.dim == 3 && c.bx == 0 && c.model == 1; }
+// Gaussian cubic lattices on the threshold-table kernel.
+static bool gauss_table(const LatticeClass& c) { return gauss_cubic(c) && c.tpb >= 512 && gtab_finest(c.L) > 0; }
 // Classes whose sweep kernel can hold two replicas in a thread.
 static bool sweeps_pairs(const LatticeClass& c) { return c.bx == 0 && c.model == 0; }
 
@@ -429,6 +432,36 @@ static int pm_split(int L, int64_t replicas) {
   }
 }
 
+// Largest share of a block of the threshold-table kernel in slots.  One block
+// fills an SM, so the launch takes ceil(blocks / SMs) rounds; of the shares that
+// fill whole warps the one with the fewest slots over all rounds is taken (a
+// block's tables cost as much as ten sweeps of 16 replicas).  The sum of the
+// populations stays within three standard deviations, its square root.
+static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
+  const int most = c.tpb / c.split * c.rp;
+  const int step = (c.split & (c.split - 1)) == 0 ? 32 / c.split * c.rp : 4 * c.rp;
+  const int64_t resident = NUM_SMS * (c.L >= 8 ? 1 : 1024 / c.tpb);
+  double sum = 0.0;
+  for (int64_t r : R0) sum += (double)r;
+  const double more = 1.0 + 3.0 / std::sqrt(std::max(1.0, sum));
+  int best = most;
+  int64_t cost = INT64_MAX;
+  for (int item = most; item >= step; item -= step) {
+    int64_t blocks = 0, share = 1;
+    for (int64_t r : R0) {
+      const int64_t n = (int64_t)((double)r * more) + 1, b = (n + item - 1) / item;
+      blocks += b;
+      share = std::max(share, (n + b - 1) / b);
+    }
+    const int64_t t = (blocks + resident - 1) / resident * (share + 16);
+    if (t < cost) {
+      cost = t;
+      best = item;
+    }
+  }
+  return best;
+}
+
 // While a launch's blocks fit the SMs at once, the SM that gets the most of
 // them sets its time, and the hardware does not deal them out evenly: 296
 // blocks of 256 threads, two an SM, ran 1.44 times as long wherever three
@@ -440,6 +473,7 @@ static int pm_split(int L, int64_t replicas) {
 void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
   constexpr int SM_SMEM = 228 * 1024, BLOCK_RESERVED = 1024;
   c.min_smem = 0;
+  c.item = gauss_table(c) ? table_item(c, R0) : 0;
   if (!sweeps_pairs(c)) return;
   const int64_t per_block = c.tpb / c.split * c.rp;
   int64_t blocks = 0;
@@ -449,11 +483,10 @@ void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
 }
 
 // Launch shape of a class before any autotuning; R0: the target populations
-// of its runs.  Gaussian cubic sweeps run 4 threads
-// per replica where the rows split so, which keeps enough warps resident to
-// hide the latency of the generator's dependent multiplies (the
-// threshold-table kernel two of 512); +-1 chains 4 or 8 on ranges of words;
-// other classes 1.
+// of its runs.  Gaussian cubic sweeps of L <= 10 take the threshold-table
+// kernel on its finest split, of L = 12 four threads per replica, which keeps
+// enough warps resident to hide the latency of the generator's dependent
+// multiplies; +-1 chains 4 or 8 on ranges of words; other classes 1.
 void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0) {
   c.split = 1;
   c.rp = 1;
@@ -463,9 +496,9 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
     c.split = split_supported(c, split_opt) ? split_opt : 1;
   } else if (pm_cubic(c)) {
     c.split = pm_split(c.L, replicas);
-  } else if (c.dim == 3 && c.bx == 0 && c.model == 1 && c.L <= 8) {
-    // the threshold-table kernel: 512 threads, two per replica (one block per
-    // SM; measured the fastest shape for a single run of 1e5 replicas)
+  } else if (gauss_cubic(c) && gtab_finest(c.L) > 0 && (tpb_opt == 0 || tpb_opt >= 512)) {
+    c.split = gtab_finest(c.L);
+  } else if (gauss_cubic(c) && c.L <= 8) {
     if (split_supported(c, 2)) c.split = 2;
   } else if (c.dim == 3 && c.bx == 0) {
     if (split_supported(c, 4)) c.split = 4;
@@ -477,7 +510,7 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   }
   if (tpb_opt && tpb_supported(c, tpb_opt)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
-  else if (c.dim == 3 && c.model == 1 && c.L <= 8) c.tpb = 512;
+  else if (gauss_cubic(c) && gtab_finest(c.L) > 0) c.tpb = 1024;
   else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * NUM_SMS ? 256 : 128;  // 5 threads a replica: 25 or 51 of
                                                                                   // them a block
   else if (c.split > 1) c.tpb = 128;
@@ -488,6 +521,16 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   // thread gives more than 900 threads an SM (28 warps; both are within 5 %
   // of each other from 600 to 1200).
   if (sweeps_pairs(c) && c.split > 1 && replicas * c.split > (int64_t)900 * NUM_SMS) c.rp = 2;
+  // The threshold-table kernel: from 600 threads an SM, from 400 where a word
+  // holds few sites (L = 6, 10: 9, 10).  us of a launch with one and with two
+  // replicas a thread: L = 8 70 / 74 at 526 threads an SM, 91 / 91 at 790; L = 10
+  // 160 / 178 at 329, 192 / 179 at 460; L = 6 47 / 45 at 197, 72 / 62 at 395.
+  if (gauss_table(c)) {
+    const int64_t from = c.L == 6 || c.L == 10 ? 400 : 600;
+    if (!gtab_shape_ok(c.L, c.split, 1) ||
+        (gtab_shape_ok(c.L, c.split, 2) && replicas * c.split > from * NUM_SMS))
+      c.rp = 2;
+  }
   spread_blocks(c, R0);
 }
 
@@ -495,9 +538,14 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c) {
   std::vector<LaunchShape> v;
   for (int split : {1, 2, 3, 4, 5, 6, 7, 8, 12}) {
-    if (!split_supported(c, split)) continue;
     for (int tpb : {32, 64, 128, 256, 512, 1024}) {
       if (!tpb_supported(c, tpb)) continue;
+      if (gauss_cubic(c) && tpb >= 512) {
+        for (int rp : {1, 2})
+          if (gtab_shape_ok(c.L, split, rp)) v.push_back({tpb, split, rp});
+        continue;
+      }
+      if (!split_supported(c, split)) continue;
       if (split > 1 && (tpb < 64 || tpb / split < 4)) continue;
       v.push_back({tpb, split, 1});
       if (sweeps_pairs(c) && split > 1) v.push_back({tpb, split, 2});
@@ -544,12 +592,13 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
   } else if (c.model == 1 && c.dim == 1) {
     err = launch_gauss1d(tpb, runs, table, nwork, c.Wr, st, init);
   } else if (c.model == 1) {
+    const Sweep3dLaunch a{c.tpb, c.split, c.rp, c.slots(), runs, table, nwork, 0, st};
     switch (c.L) {
-      case 4: err = launch_gauss3d_L4(tpb, c.split, runs, table, nwork, st, init); break;
-      case 6: err = launch_gauss3d_L6(tpb, c.split, runs, table, nwork, st, init); break;
-      case 8: err = launch_gauss3d_L8(tpb, c.split, runs, table, nwork, st, init); break;
-      case 10: err = launch_gauss3d_L10(tpb, c.split, runs, table, nwork, st, init); break;
-      case 12: err = launch_gauss3d_L12(tpb, c.split, runs, table, nwork, st, init); break;
+      case 4: err = launch_gauss3d_L4(a, init); break;
+      case 6: err = launch_gauss3d_L6(a, init); break;
+      case 8: err = launch_gauss3d_L8(a, init); break;
+      case 10: err = launch_gauss3d_L10(a, init); break;
+      case 12: err = launch_gauss3d_L12(a, init); break;
       default: return fail(PA_ERR_UNSUPPORTED, "no Gaussian kernel for L=%d", c.L);
     }
   } else if (c.dim == 1) {
@@ -567,7 +616,7 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
       default: return fail(PA_ERR_UNSUPPORTED, "no kernel for L=%d", c.L);
     }
   } else {
-    err = sweep3d_call(c.L, {tpb, c.split, c.rp, runs, table, nwork, c.min_smem, st});
+    err = sweep3d_call(c.L, {tpb, c.split, c.rp, c.slots(), runs, table, nwork, c.min_smem, st});
   }
   if (err != cudaSuccess) return cuda_fail(err, "sweep kernel launch");
   return PA_OK;

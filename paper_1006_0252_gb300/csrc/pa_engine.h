@@ -67,8 +67,7 @@ cudaError_t launch_gauss1d(int tpb, RunDev* runs, const Work* table, int nwork, 
 // Shared memory of the Gaussian chain kernel (thresholds, uniform tables, couplings, columns).
 size_t gauss1d_smem_bytes(int tpb, int WR);
 #define PA_DECLG(LL)                                                                                \
-  cudaError_t launch_gauss3d_L##LL(int tpb, int split, RunDev* runs, const Work* table, int nwork, \
-                                   cudaStream_t st, bool init);                                    \
+  cudaError_t launch_gauss3d_L##LL(const Sweep3dLaunch& a, bool init);                              \
   bool gauss3d_split_ok_L##LL(int split);
 PA_DECLG(4)
 PA_DECLG(6)
@@ -150,14 +149,15 @@ struct LatticeClass {
   int max_tpb = 256;                        // largest block whose shared memory fits
   int tpb = 0;
   int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
-  int rp = 1;        // +-1 cubic lattices and chains: replicas a thread sweeps side by side (1, 2)
+  int rp = 1;        // +-1 lattices and chains, Gaussian threshold tables: replicas a thread sweeps side by side (1, 2)
   int min_smem = 0;  // shared memory of a sweep block that keeps the blocks even over the SMs (spread_blocks)
   std::vector<int32_t> runs;
   Work* d_table = nullptr;
   int nwork = 0;
+  int item = 0;      // slots of a work item where they are chosen by the populations (spread_blocks), else 0
   // Slots of a work item: the block's threads where a power of two of them
   // shares a replica (split / rp blocks an item), else the block's replicas.
-  int slots() const { return (split & (split - 1)) == 0 ? tpb : tpb / split * rp; }
+  int slots() const { return item > 0 ? item : ((split & (split - 1)) == 0 ? tpb : tpb / split * rp); }
 };
 
 // One launch shape of a class.

@@ -242,9 +242,10 @@ __device__ __forceinline__ int energy_gauss3d(const uint32_t* __restrict__ col, 
 __device__ __forceinline__ void measure_store_gauss(RunDev& R, int nxt, int64_t slot, bool live, int E) {
   long long e = 0ll;
   unsigned long long lo = 0ull, hi = 0ull;
+  const int low = __reduce_min_sync(0xFFFFFFFFu, live ? E : 0x7FFFFFFF);
+  const bool any = __any_sync(0xFFFFFFFFu, live);
   if (live) {
     R.E[nxt][slot] = E;
-    atomicMin(&R.emin_next, (long long)E);
     e = E;
     const unsigned long long q = (unsigned long long)((long long)E * (long long)E);  // < 2^62
     lo = q & 0xFFFFFFFFull;
@@ -257,6 +258,7 @@ __device__ __forceinline__ void measure_store_gauss(RunDev& R, int nxt, int64_t 
     hi += __shfl_xor_sync(0xFFFFFFFFu, hi, sh);
   }
   if ((threadIdx.x & 31) == 0) {
+    if (any) atomicMin(&R.emin_next, (long long)low);
     atomicAdd(&R.sumE_next, (unsigned long long)e);
     atomicAdd(&R.sumE2_next, lo);
     atomicAdd(&R.sumE2hi_next, hi);
@@ -385,9 +387,10 @@ __global__ void __launch_bounds__(TPB) k_sweep_gauss3d(RunDev* __restrict__ runs
 }
 
 // Sec. 2: R0 independent uniformly random microstates at beta = 0 (keying as
-// k_init3d) and their fixed-point energies.
+// k_init3d) and their fixed-point energies; one thread per slot of a work item.
 template <int L, int TPB>
-__global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs, const Work* __restrict__ table) {
+__global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs, const Work* __restrict__ table,
+                                                      int slots) {
   using GEO = Geo3<L>;
   constexpr int WR = GEO::WR, W = GEO::W, SP = ((GEO::K * L / 2) + 3) & ~3;
   constexpr int NJ = 2 * 6 * WR * SP;
@@ -401,7 +404,7 @@ __global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs,
   const int tid = threadIdx.x;
   for (int i = tid; i < NJ; i += TPB) s_J[i] = R.gJ[i];
   const int64_t slot = (int64_t)wk.first + tid;
-  const bool live = slot < R0;
+  const bool live = tid < slots && slot < R0;
   uint32_t* col = s_spin + tid;
   if (live) {
     for (int w4 = 0; w4 < W / 4; ++w4) {
@@ -422,7 +425,7 @@ __global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs,
 }
 
 template <int L, int TPB, int P>
-cudaError_t launch_gauss3d_p(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
+cudaError_t launch_gauss3d_p(const Sweep3dLaunch& a) {
   if constexpr (!split_ok<Geo3<L>>(P) || TPB / P < 4 || (P > 1 && TPB < 64)) {
     return cudaErrorInvalidValue;
   } else {
@@ -432,14 +435,14 @@ cudaError_t launch_gauss3d_p(RunDev* runs, const Work* table, int nwork, cudaStr
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (e != cudaSuccess) return e;
     }
-    if (nwork <= 0) return cudaSuccess;
-    k_sweep_gauss3d<L, TPB, P><<<nwork * P, TPB, sm, st>>>(runs, table);
+    if (a.nwork <= 0) return cudaSuccess;
+    k_sweep_gauss3d<L, TPB, P><<<a.nwork * P, TPB, sm, a.st>>>(a.runs, a.table);
     return cudaGetLastError();
   }
 }
 
 template <int L, int TPB>
-cudaError_t launch_gauss3d_init(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
+cudaError_t launch_gauss3d_init(const Sweep3dLaunch& a) {
   using GEO = Geo3<L>;
   const size_t sm = 4 * (gauss_tables_words<L>() + (size_t)GEO::WR * TPB);
   if (sm > 48 * 1024) {
@@ -447,35 +450,54 @@ cudaError_t launch_gauss3d_init(RunDev* runs, const Work* table, int nwork, cuda
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  if (nwork <= 0) return cudaSuccess;
-  k_init_gauss3d<L, TPB><<<nwork, TPB, sm, st>>>(runs, table);
+  if (a.nwork <= 0) return cudaSuccess;
+  k_init_gauss3d<L, TPB><<<a.nwork, TPB, sm, a.st>>>(a.runs, a.table, a.slots);
   return cudaGetLastError();
 }
 
+// The initial state in blocks of the smallest size that holds a work item.
+template <int L>
+cudaError_t launch_gauss3d_init_any(const Sweep3dLaunch& a) {
+  if (a.slots <= 32) return launch_gauss3d_init<L, 32>(a);
+  if (a.slots <= 64) return launch_gauss3d_init<L, 64>(a);
+  if (a.slots <= 128) return launch_gauss3d_init<L, 128>(a);
+  if (a.slots <= 256) return launch_gauss3d_init<L, 256>(a);
+  if constexpr (L <= 10) {
+    if (a.slots <= 512) return launch_gauss3d_init<L, 512>(a);
+  }
+  if constexpr (L <= 8) {
+    if (a.slots <= 1024) return launch_gauss3d_init<L, 1024>(a);
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <int L, int TPB>
-cudaError_t launch_gauss3d_t(RunDev* runs, const Work* table, int nwork, cudaStream_t st, bool init, int split) {
-  if (init) return launch_gauss3d_init<L, TPB>(runs, table, nwork, st);
-  switch (split) {
-    case 1: return launch_gauss3d_p<L, TPB, 1>(runs, table, nwork, st);
-    case 2: return launch_gauss3d_p<L, TPB, 2>(runs, table, nwork, st);
-    case 4: return launch_gauss3d_p<L, TPB, 4>(runs, table, nwork, st);
+cudaError_t launch_gauss3d_t(const Sweep3dLaunch& a) {
+  switch (a.split) {
+    case 1: return launch_gauss3d_p<L, TPB, 1>(a);
+    case 2: return launch_gauss3d_p<L, TPB, 2>(a);
+    case 4: return launch_gauss3d_p<L, TPB, 4>(a);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int L>
+cudaError_t launch_gauss3d_any(const Sweep3dLaunch& a) {
+  switch (a.tpb) {
+    case 32: return launch_gauss3d_t<L, 32>(a);
+    case 64: return launch_gauss3d_t<L, 64>(a);
+    case 128: return launch_gauss3d_t<L, 128>(a);
+    case 256: return launch_gauss3d_t<L, 256>(a);
     default: return cudaErrorInvalidValue;
   }
 }
 
 }  // namespace pa
 
-#define PA_INSTANTIATE_GAUSS3D(LL)                                                                     \
-  namespace pa {                                                                                       \
-  cudaError_t launch_gauss3d_L##LL(int tpb, int split, RunDev* runs, const Work* table, int nwork,    \
-                                   cudaStream_t st, bool init) {                                       \
-    switch (tpb) {                                                                                     \
-      case 32: return launch_gauss3d_t<LL, 32>(runs, table, nwork, st, init, split);                   \
-      case 64: return launch_gauss3d_t<LL, 64>(runs, table, nwork, st, init, split);                   \
-      case 128: return launch_gauss3d_t<LL, 128>(runs, table, nwork, st, init, split);                 \
-      case 256: return launch_gauss3d_t<LL, 256>(runs, table, nwork, st, init, split);                 \
-      default: return cudaErrorInvalidValue;                                                           \
-    }                                                                                                  \
-  }                                                                                                    \
-  bool gauss3d_split_ok_L##LL(int split) { return split <= 4 && split_ok<Geo3<LL>>(split); }          \
+#define PA_INSTANTIATE_GAUSS3D(LL)                                                               \
+  namespace pa {                                                                                 \
+  cudaError_t launch_gauss3d_L##LL(const Sweep3dLaunch& a, bool init) {                          \
+    return init ? launch_gauss3d_init_any<LL>(a) : launch_gauss3d_any<LL>(a);                    \
+  }                                                                                              \
+  bool gauss3d_split_ok_L##LL(int split) { return split <= 4 && split_ok<Geo3<LL>>(split); }     \
   }

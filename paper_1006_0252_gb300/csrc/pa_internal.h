@@ -120,6 +120,7 @@ struct Work {
 // a block.
 struct Sweep3dLaunch {
   int tpb, split, rp;
+  int slots;  // of a work item
   RunDev* runs;
   const Work* table;
   int nwork;
@@ -127,4 +128,17 @@ struct Sweep3dLaunch {
   cudaStream_t st;
 };
 
+// Gaussian threshold-table kernel (pa_gauss3d_tab.cuh): the finest split of an
+// edge (whole rows, pairs of them where a row's uniforms end within a generator
+// call; 0: no such kernel) and the shapes it is built for: the finest split
+// with one and with two replicas a thread, one thread a replica with one (two
+// would not fit shared memory), the others with two.
+constexpr int gtab_finest(int L) { return L == 4 ? 4 : (L == 6 ? 3 : (L == 8 ? 8 : (L == 10 ? 5 : 0))); }
+constexpr bool gtab_shape_ok(int L, int split, int rp) {
+  const int finest = gtab_finest(L);
+  if (finest == 0 || rp < 1 || rp > 2) return false;
+  if (split == finest) return true;
+  if (split == 1) return L <= 8 && rp == 1;
+  return (L == 4 || L == 8) && (split == 2 || split == 4) && rp == 2;
+}
 }  // namespace pa

@@ -1,5 +1,6 @@
 """Launch shapes the library chooses by itself (GPU): the +-1 cubic and chain
-sweeps with one and with two replicas per thread against the oracle."""
+sweeps and the Gaussian cubic sweep with one and with two replicas per thread
+against the oracle."""
 import numpy as np
 import pytest
 
@@ -49,5 +50,25 @@ def test_chosen_chain_shape_bit_exact(N, is_open, R0):
         c.step(beta, sweeps, R0)
     go, co = g.observables(), c.state()
     assert go["R"] == co.R and go["sumE"] == co.sumE and go["sumE2"] == co.sumE2
+    assert np.array_equal(g.energies(), c.energies())
+    assert np.array_equal(g.spins(), c.spins())
+
+
+# (L, R0): Gaussian couplings; the largest odd populations that take one replica
+# a thread and the smallest that take two (600 threads an SM; 400 at L = 6, 10).
+# The betas give thresholds of 2^24 to rises (1e-6), ordinary ones, and 0 (60).
+@pytest.mark.parametrize("L,R0,split", [(4, 22799, 4), (4, 22801, 4), (6, 20265, 3), (6, 20267, 3), (8, 301, 8),
+                                        (8, 11399, 8), (8, 11401, 8), (10, 12159, 5), (10, 12161, 5)])
+def test_chosen_gauss_shape_bit_exact(L, R0, split):
+    J = inputs.gaussian_couplings_3d(L, 4, 1)
+    cap = R0 + 4000
+    g = pa.Run(J, L, 3, R0, 31, R_cap=cap, gaussian=True)
+    assert pa.pa_sweep_shape(g._h) == (1024, split)
+    c = o.GaussRun(J, 3, L, L, L, 7, R0=R0, R_cap=cap, seed=31)
+    for beta, sweeps in ((1e-6, 1), (0.4, 1), (0.9, 0), (1.5, 1), (3.0, 0), (8.0, 0), (20.0, 0), (60.0, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+        assert g.observables()["R"] == c.state().R, beta
+    assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.energies(), c.energies())
     assert np.array_equal(g.spins(), c.spins())
