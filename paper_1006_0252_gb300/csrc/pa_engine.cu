@@ -386,7 +386,7 @@ int default_tpb(int dim, int L) {
 bool tpb_supported(const LatticeClass& c, int tpb) {
   if (tpb == 32 || tpb == 64 || tpb == 128 || tpb == 256) {
     if (c.bx > 0) return tpb <= c.max_tpb;
-    if (c.dim == 1 && c.model == 1) return gauss1d_smem_bytes(tpb, c.Wr) <= SMEM_LIMIT;
+    if (c.dim == 1 && c.model == 1) return gauss1d_smem_bytes(tpb, 1, 1, c.Wr) <= SMEM_LIMIT;
     return true;
   }
   if (tpb == 512 || tpb == 1024) return c.bx == 0 && c.dim == 3 && c.model == 1 && c.L <= 10;
@@ -398,7 +398,8 @@ static bool gauss_cubic(const LatticeClass& c) { return c.dim == 3 && c.bx == 0 
 // Gaussian cubic lattices on the threshold-table kernel.
 static bool gauss_table(const LatticeClass& c) { return gauss_cubic(c) && c.tpb >= 512 && gtab_finest(c.L) > 0; }
 // Classes whose sweep kernel can hold two replicas in a thread.
-static bool sweeps_pairs(const LatticeClass& c) { return c.bx == 0 && c.model == 0; }
+static bool sweeps_pairs(const LatticeClass& c) { return c.bx == 0 && (c.model == 0 || c.dim == 1); }
+static bool gauss_chain(const LatticeClass& c) { return c.bx == 0 && c.dim == 1 && c.model == 1; }
 
 static cudaError_t sweep3d_call(int L, const Sweep3dLaunch& a) {
   switch (L) {
@@ -486,7 +487,7 @@ void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
 // of its runs.  Gaussian cubic sweeps of L <= 10 take the threshold-table
 // kernel on its finest split, of L = 12 four threads per replica, which keeps
 // enough warps resident to hide the latency of the generator's dependent
-// multiplies; +-1 chains 4 or 8 on ranges of words; other classes 1.
+// multiplies; chains up to 8 on ranges of words; other classes 1.
 void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0) {
   c.split = 1;
   c.rp = 1;
@@ -507,6 +508,8 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
     // a block within shared memory at long chains (8 rather than 4 ranges of
     // 8 words: 25 against 33 us at 2000 replicas of 256 spins, 3 % at 20000)
     c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : 1);
+  } else if (gauss_chain(c) && tpb_opt == 0) {
+    c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : (c.Wr >= 2 ? 2 : 1));
   }
   if (tpb_opt && tpb_supported(c, tpb_opt)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
@@ -520,7 +523,12 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   // flip in full launches) but halve the threads: taken once one replica a
   // thread gives more than 900 threads an SM (28 warps; both are within 5 %
   // of each other from 600 to 1200).
-  if (sweeps_pairs(c) && c.split > 1 && replicas * c.split > (int64_t)900 * NUM_SMS) c.rp = 2;
+  // (A Gaussian chain of more than 32 words takes two in any population: its
+  // tables, not its threads, limit the blocks of an SM.  N = 4096, 5000
+  // replicas, theta = 10: 394 us with one, 285 with two.)
+  if (sweeps_pairs(c) && c.split > 1 &&
+      (replicas * c.split > (int64_t)900 * NUM_SMS || (gauss_chain(c) && c.Wr > 32)))
+    c.rp = 2;
   // The threshold-table kernel: from 600 threads an SM, from 400 where a word
   // holds few sites (L = 6, 10: 9, 10).  us of a launch with one and with two
   // replicas a thread: L = 8 70 / 74 at 526 threads an SM, 91 / 91 at 790; L = 10
@@ -543,6 +551,12 @@ std::vector<LaunchShape> launch_shapes(const LatticeClass& c) {
       if (gauss_cubic(c) && tpb >= 512) {
         for (int rp : {1, 2})
           if (gtab_shape_ok(c.L, split, rp)) v.push_back({tpb, split, rp});
+        continue;
+      }
+      if (gauss_chain(c) && split > 1) {
+        if (tpb < 64 || !sweep1d_split_ok(split)) continue;
+        for (int rp : {1, 2})
+          if (gauss1d_smem_bytes(tpb, split, rp, c.Wr) <= SMEM_LIMIT) v.push_back({tpb, split, rp});
         continue;
       }
       if (!split_supported(c, split)) continue;
@@ -590,7 +604,7 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
     }
     err = launch_box(tpb, runs, table, nwork, c.Wr, c.bsites, st, init);
   } else if (c.model == 1 && c.dim == 1) {
-    err = launch_gauss1d(tpb, runs, table, nwork, c.Wr, st, init);
+    err = launch_gauss1d(tpb, c.split, c.rp, runs, table, nwork, c.Wr, st, init, c.min_smem);
   } else if (c.model == 1) {
     const Sweep3dLaunch a{c.tpb, c.split, c.rp, c.slots(), runs, table, nwork, 0, st};
     switch (c.L) {

@@ -63,9 +63,10 @@ cudaError_t launch_box(int tpb, RunDev* runs, const Work* table, int nwork, int 
                        bool init);
 size_t box_smem_bytes(int WR, int S, int tpb);
 cudaError_t launch_gauss_thresholds(int64_t n, double beta, const int32_t* dE, uint32_t* thr);
-cudaError_t launch_gauss1d(int tpb, RunDev* runs, const Work* table, int nwork, int WR, cudaStream_t st, bool init);
+cudaError_t launch_gauss1d(int tpb, int split, int rp, RunDev* runs, const Work* table, int nwork, int WR,
+                           cudaStream_t st, bool init, int min_smem);
 // Shared memory of the Gaussian chain kernel (thresholds, uniform tables, couplings, columns).
-size_t gauss1d_smem_bytes(int tpb, int WR);
+size_t gauss1d_smem_bytes(int tpb, int split, int rp, int WR);
 #define PA_DECLG(LL)                                                                                \
   cudaError_t launch_gauss3d_L##LL(const Sweep3dLaunch& a, bool init);                              \
   bool gauss3d_split_ok_L##LL(int split);
@@ -149,7 +150,7 @@ struct LatticeClass {
   int max_tpb = 256;                        // largest block whose shared memory fits
   int tpb = 0;
   int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
-  int rp = 1;        // +-1 lattices and chains, Gaussian threshold tables: replicas a thread sweeps side by side (1, 2)
+  int rp = 1;        // +-1 lattices, chains, Gaussian threshold tables: replicas a thread sweeps side by side (1, 2)
   int min_smem = 0;  // shared memory of a sweep block that keeps the blocks even over the SMs (spread_blocks)
   std::vector<int32_t> runs;
   Work* d_table = nullptr;

@@ -151,4 +151,33 @@ __device__ __forceinline__ bool gauss_accept_fast(int dE, float beta_f, uint32_t
   return gauss_accept(dE, beta_f, u);
 }
 
+// Record the energy and the exact sums of one replica per thread (threads with
+// live == false contribute nothing but take part in the warp's reductions;
+// every thread of the warp calls this).
+__device__ __forceinline__ void measure_store_gauss(RunDev& R, int nxt, int64_t slot, bool live, int E) {
+  long long e = 0ll;
+  unsigned long long lo = 0ull, hi = 0ull;
+  const int low = __reduce_min_sync(0xFFFFFFFFu, live ? E : 0x7FFFFFFF);
+  const bool any = __any_sync(0xFFFFFFFFu, live);
+  if (live) {
+    R.E[nxt][slot] = E;
+    e = E;
+    const unsigned long long q = (unsigned long long)((long long)E * (long long)E);  // < 2^62
+    lo = q & 0xFFFFFFFFull;
+    hi = q >> 32;
+  }
+#pragma unroll
+  for (int sh = 16; sh >= 1; sh >>= 1) {
+    e += __shfl_xor_sync(0xFFFFFFFFu, e, sh);
+    lo += __shfl_xor_sync(0xFFFFFFFFu, lo, sh);
+    hi += __shfl_xor_sync(0xFFFFFFFFu, hi, sh);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (any) atomicMin(&R.emin_next, (long long)low);
+    atomicAdd(&R.sumE_next, (unsigned long long)e);
+    atomicAdd(&R.sumE2_next, lo);
+    atomicAdd(&R.sumE2hi_next, hi);
+  }
+}
+
 }  // namespace pa

@@ -239,32 +239,6 @@ __device__ __forceinline__ int energy_gauss3d(const uint32_t* __restrict__ col, 
   return C0 - 2 * anti_rows_gauss3d<GEO, TPB>(col, s_J, one, 0, GEO::L);
 }
 
-__device__ __forceinline__ void measure_store_gauss(RunDev& R, int nxt, int64_t slot, bool live, int E) {
-  long long e = 0ll;
-  unsigned long long lo = 0ull, hi = 0ull;
-  const int low = __reduce_min_sync(0xFFFFFFFFu, live ? E : 0x7FFFFFFF);
-  const bool any = __any_sync(0xFFFFFFFFu, live);
-  if (live) {
-    R.E[nxt][slot] = E;
-    e = E;
-    const unsigned long long q = (unsigned long long)((long long)E * (long long)E);  // < 2^62
-    lo = q & 0xFFFFFFFFull;
-    hi = q >> 32;
-  }
-#pragma unroll
-  for (int sh = 16; sh >= 1; sh >>= 1) {
-    e += __shfl_xor_sync(0xFFFFFFFFu, e, sh);
-    lo += __shfl_xor_sync(0xFFFFFFFFu, lo, sh);
-    hi += __shfl_xor_sync(0xFFFFFFFFu, hi, sh);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (any) atomicMin(&R.emin_next, (long long)low);
-    atomicAdd(&R.sumE_next, (unsigned long long)e);
-    atomicAdd(&R.sumE2_next, lo);
-    atomicAdd(&R.sumE2hi_next, hi);
-  }
-}
-
 // Per-site table words: [2][6][WR][SP] couplings + [2][WR][SP] sums, SP = the
 // colour-c sites per word rounded up to a multiple of 4 (16-byte rows).
 template <int L>

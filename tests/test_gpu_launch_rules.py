@@ -72,3 +72,24 @@ def test_chosen_gauss_shape_bit_exact(L, R0, split):
     assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.energies(), c.energies())
     assert np.array_equal(g.spins(), c.spins())
+
+
+# (N, open, R0, threads per replica): Gaussian chains of 1, 2, 4, 8, 32 and 128
+# words, short last words, odd length, one and two replicas a thread.
+@pytest.mark.parametrize("N,is_open,R0,split", [(30, False, 501, 1), (64, False, 501, 2), (34, False, 68401, 2),
+                                                (103, True, 34201, 4), (256, False, 17099, 8), (258, False, 17101, 8),
+                                                (1001, True, 17101, 8), (4096, False, 301, 8)])
+def test_chosen_gauss_chain_shape_bit_exact(N, is_open, R0, split):
+    J = inputs.gaussian_couplings_chain(N, 2, 9, open_chain=is_open)
+    J[N // 3] = 0  # both neighbours' alignments give the same energy change
+    cap = R0 + 4000
+    g = pa.Run(J, N, 1, R0, 37, R_cap=cap, gaussian=True)
+    assert pa.pa_sweep_shape(g._h)[1] == split
+    c = o.GaussRun(J, 1, N, R0=R0, R_cap=cap, seed=37)
+    for beta, sweeps in ((1e-6, 1), (0.5, 1), (1.0, 0), (2.0, 1), (5.0, 0), (12.0, 0), (30.0, 0), (80.0, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+        assert g.observables()["R"] == c.state().R, beta
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.energies(), c.energies())
+    assert np.array_equal(g.spins(), c.spins())
