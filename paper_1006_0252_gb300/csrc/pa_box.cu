@@ -11,6 +11,10 @@
 // points back to the site and carries J = 0), its six couplings and their sum.
 // Sites of one colour only read sites of the other, so a half sweep may update
 // the column in place, site by site.
+//
+// The initial state of every box, and the sweeps of boxes whose threshold table
+// does not fit shared memory or that ask for a block size; the others take
+// pa_boxtab.cuh.
 #include "pa_gauss.cuh"
 #include "pa_internal.h"
 
@@ -121,9 +125,11 @@ __device__ __forceinline__ void measure_box(RunDev& R, int nxt, int64_t slot, bo
 
 template <int TPB>
 __global__ void __launch_bounds__(TPB) k_sweep_box(RunDev* __restrict__ runs, const Work* __restrict__ table,
-                                                   int init) {
+                                                   int init, int slots) {
   extern __shared__ uint32_t smem[];
-  const Work wk = table[blockIdx.x];
+  const int per = (slots + TPB - 1) / TPB;  // blocks of a work item
+  const int at = (int)(blockIdx.x % per) * TPB + threadIdx.x;
+  const Work wk = table[blockIdx.x / per];
   RunDev& R = runs[wk.run];
   if (!init && R.skip) return;
   const int64_t Rn = init ? R.R : R.R_next;
@@ -140,8 +146,8 @@ __global__ void __launch_bounds__(TPB) k_sweep_box(RunDev* __restrict__ runs, co
   for (int i = tid; i < 12 * plane; i += TPB) s_J[i] = R.gJ[i];
   for (int i = tid; i < 2 * plane; i += TPB) s_S[i] = R.gS[i];
   if (tid < 8) s_thr[tid] = R.thr[tid];
-  const int64_t slot = (int64_t)wk.first + tid;
-  const bool live = slot < Rn;
+  const int64_t slot = (int64_t)wk.first + at;
+  const bool live = at < slots && slot < Rn;
   const int cur = R.cur, nxt = init ? 0 : cur ^ 1;
   uint32_t* col = s_spin + tid;
   const uint32_t valid = R.bvalid;
@@ -204,7 +210,7 @@ size_t box_smem_bytes(int WR, int S, int tpb) {
 }
 
 template <int TPB>
-static cudaError_t launch_box_t(RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
+static cudaError_t launch_box_t(int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
                                 bool init) {
   const size_t sm = box_smem_bytes(WR, S, TPB);
   if (sm > BOX_SMEM_MAX) return nwork > 0 ? cudaErrorInvalidValue : cudaSuccess;
@@ -213,17 +219,17 @@ static cudaError_t launch_box_t(RunDev* runs, const Work* table, int nwork, int 
     if (e != cudaSuccess) return e;
   }
   if (nwork <= 0) return cudaSuccess;
-  k_sweep_box<TPB><<<nwork, TPB, sm, st>>>(runs, table, init ? 1 : 0);
+  k_sweep_box<TPB><<<nwork * ((slots + TPB - 1) / TPB), TPB, sm, st>>>(runs, table, init ? 1 : 0, slots);
   return cudaGetLastError();
 }
 
-cudaError_t launch_box(int tpb, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
+cudaError_t launch_box(int tpb, int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
                        bool init) {
   switch (tpb) {
-    case 32: return launch_box_t<32>(runs, table, nwork, WR, S, st, init);
-    case 64: return launch_box_t<64>(runs, table, nwork, WR, S, st, init);
-    case 128: return launch_box_t<128>(runs, table, nwork, WR, S, st, init);
-    case 256: return launch_box_t<256>(runs, table, nwork, WR, S, st, init);
+    case 32: return launch_box_t<32>(slots, runs, table, nwork, WR, S, st, init);
+    case 64: return launch_box_t<64>(slots, runs, table, nwork, WR, S, st, init);
+    case 128: return launch_box_t<128>(slots, runs, table, nwork, WR, S, st, init);
+    case 256: return launch_box_t<256>(slots, runs, table, nwork, WR, S, st, init);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -433,15 +433,48 @@ static int pm_split(int L, int64_t replicas) {
   }
 }
 
+// General boxes on their threshold-table kernel (blocks of BOX_TPB threads), and
+// the most slots a block of it takes: as many columns as it has threads for and
+// as fit shared memory, in whole warps (0: none fit).
+static bool box_table(const LatticeClass& c) { return c.bx > 0 && c.tpb == BOX_TPB; }
+static int box_most(const LatticeClass& c, int P, int reps) {
+  const int unit = 32 / P * reps;
+  for (int slots = BOX_TPB / P * reps; slots >= unit; slots -= unit) {
+    const BoxTabShape sh = boxtab_shape(c.Wr, c.bsites, {c.bx, c.Wr / c.by, c.by, P, reps, slots});
+    if (sizeof(uint32_t) * sh.words <= SMEM_LIMIT) return slots;
+  }
+  return 0;
+}
+// Threads a column (a power of two, whole periods of words each) and replicas a
+// thread of that kernel: the finest split that keeps the even share of an SM's
+// replicas in one block, as many replicas a word as it holds, fewer where that
+// would leave the block fewer than eight warps.  8 x 6 x 5, 20000 replicas, us a
+// launch for (split, replicas): (16, 4) 109, (32, 4) 120, (8, 4) 134, (16, 2)
+// 137, (16, 1) 169; 1000 replicas (32, 2) 29, (16, 1) 31, (16, 4) 47; 6 x 6 x 7,
+// 3000 replicas (16, 1) 64, (16, 2) 70, (8, 1) 87, (16, 4) 110.
+static bool set_box_table(LatticeClass& c, int64_t replicas) {
+  const int U = box_period(c.bsites), groups = (c.Wr + U - 1) / U;
+  const int64_t share = (replicas + NUM_SMS - 1) / NUM_SMS;
+  int P = 1, reps = box_replicas(c.bsites);
+  while (P < groups && P < 32) P *= 2;
+  while (reps > 1 && (share + reps - 1) / reps * P < 256) reps /= 2;
+  while (P > 1 && (share + reps - 1) / reps * P > BOX_TPB) P /= 2;
+  if (box_most(c, P, reps) == 0) return false;
+  c.tpb = BOX_TPB;
+  c.split = P;
+  c.rp = reps;
+  return true;
+}
+
 // Largest share of a block of the threshold-table kernel in slots.  One block
 // fills an SM, so the launch takes ceil(blocks / SMs) rounds; of the shares that
 // fill whole warps the one with the fewest slots over all rounds is taken (a
 // block's tables cost as much as ten sweeps of 16 replicas).  The sum of the
 // populations stays within three standard deviations, its square root.
 static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
-  const int most = c.tpb / c.split * c.rp;
   const int step = (c.split & (c.split - 1)) == 0 ? 32 / c.split * c.rp : 4 * c.rp;
-  const int64_t resident = NUM_SMS * (c.L >= 8 ? 1 : 1024 / c.tpb);
+  const int most = box_table(c) ? box_most(c, c.split, c.rp) : c.tpb / c.split * c.rp;
+  const int64_t resident = NUM_SMS * (c.tpb < 1024 && c.L < 8 ? 1024 / c.tpb : 1);
   double sum = 0.0;
   for (int64_t r : R0) sum += (double)r;
   const double more = 1.0 + 3.0 / std::sqrt(std::max(1.0, sum));
@@ -474,7 +507,7 @@ static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
 void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
   constexpr int SM_SMEM = 228 * 1024, BLOCK_RESERVED = 1024;
   c.min_smem = 0;
-  c.item = gauss_table(c) ? table_item(c, R0) : 0;
+  c.item = gauss_table(c) || box_table(c) ? table_item(c, R0) : 0;
   if (!sweeps_pairs(c)) return;
   const int64_t per_block = c.tpb / c.split * c.rp;
   int64_t blocks = 0;
@@ -493,6 +526,11 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   c.rp = 1;
   int64_t replicas = 0;
   for (int64_t r : R0) replicas += r;
+  c.tpb = 0;
+  if (c.bx > 0 && tpb_opt == 0 && split_opt == 0 && set_box_table(c, replicas)) {
+    spread_blocks(c, R0);
+    return;
+  }
   if (split_opt > 0) {
     c.split = split_supported(c, split_opt) ? split_opt : 1;
   } else if (pm_cubic(c)) {
@@ -545,6 +583,12 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
 // Every launch shape the sweep kernel of a class has.
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c) {
   std::vector<LaunchShape> v;
+  if (c.bx > 0) {
+    const int U = box_period(c.bsites), groups = (c.Wr + U - 1) / U;
+    for (int P = 1; P <= 32 && P < 2 * groups; P *= 2)
+      for (int reps = 1; reps <= box_replicas(c.bsites); reps *= 2)
+        if (box_most(c, P, reps) > 0) v.push_back({BOX_TPB, P, reps});
+  }
   for (int split : {1, 2, 3, 4, 5, 6, 7, 8, 12}) {
     for (int tpb : {32, 64, 128, 256, 512, 1024}) {
       if (!tpb_supported(c, tpb)) continue;
@@ -598,11 +642,20 @@ int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const 
   cudaError_t err;
   const int tpb = init ? c.slots() : c.tpb;  // the initial state takes one thread per slot
   if (c.bx > 0) {
+    if (box_table(c)) {
+      const int S = c.bsites;
+      const BoxShape box{c.bx, c.Wr / c.by, c.by, c.split, c.rp, c.item};
+      err = init ? launch_box(std::min(c.max_tpb, 256), c.item, runs, table, nwork, c.Wr, S, st, true)
+            : S <= 8 ? launch_boxtab_a(S, box, runs, table, nwork, c.Wr, st)
+                     : launch_boxtab_b(S, box, runs, table, nwork, c.Wr, st);
+      if (err != cudaSuccess) return cuda_fail(err, "sweep kernel launch");
+      return PA_OK;
+    }
     if (tpb > c.max_tpb) {
       if (nwork <= 0) return PA_OK;  // nothing to set up for a block size that cannot run
       return fail(PA_ERR_UNSUPPORTED, "block of %d threads exceeds shared memory for this box", tpb);
     }
-    err = launch_box(tpb, runs, table, nwork, c.Wr, c.bsites, st, init);
+    err = launch_box(tpb, tpb, runs, table, nwork, c.Wr, c.bsites, st, init);
   } else if (c.model == 1 && c.dim == 1) {
     err = launch_gauss1d(tpb, c.split, c.rp, runs, table, nwork, c.Wr, st, init, c.min_smem);
   } else if (c.model == 1) {

@@ -59,8 +59,12 @@ cudaError_t launch_overlap_hist(const RunDev* runs, const int32_t* ra, const int
                                 unsigned long long* hist, cudaStream_t st);
 cudaError_t launch_overlap_pairs(const RunDev* runs, const int32_t* ra, const int32_t* rb, int n_pairs, double qcut,
                                  unsigned long long* count, cudaStream_t st);
-cudaError_t launch_box(int tpb, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
+cudaError_t launch_box(int tpb, int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
                        bool init);
+cudaError_t launch_boxtab_a(int S, const BoxShape& box, RunDev* runs, const Work* table, int nwork, int WR,
+                            cudaStream_t st);
+cudaError_t launch_boxtab_b(int S, const BoxShape& box, RunDev* runs, const Work* table, int nwork, int WR,
+                            cudaStream_t st);
 size_t box_smem_bytes(int WR, int S, int tpb);
 cudaError_t launch_gauss_thresholds(int64_t n, double beta, const int32_t* dE, uint32_t* thr);
 cudaError_t launch_gauss1d(int tpb, int split, int rp, RunDev* runs, const Work* table, int nwork, int WR,

@@ -38,6 +38,7 @@
 // want the finest split.)
 #include "pa_gauss.cuh"
 #include "pa_lattice3d.cuh"
+#include "pa_patterns.cuh"
 
 namespace pa {
 
@@ -136,15 +137,6 @@ __device__ __forceinline__ GchainWord gchain_word(const T* __restrict__ own, con
   return {s, nx, o};
 }
 
-// 2 ge + [u >= 256 thr] from the threshold's entry.
-__device__ __forceinline__ uint32_t shift_in_reject(uint32_t ge, uint32_t u, uint32_t entry) {
-  uint32_t r;
-  asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, %3;\n\t}"
-      : "=r"(r)
-      : "r"(u), "r"(entry), "r"(ge));
-  return r;
-}
-
 // Colour-C half sweep of words w0 .. w1-1 of a column (colour-C word w at
 // own[w CS], the other colour's at oth[w CS]).  The uniforms of word w are
 // calls 4w .. 4w+3 of the colour; the calls are taken from the last, so that
@@ -167,14 +159,14 @@ __device__ __forceinline__ void half_sweep_gauss1d(ColourWord<RP>* __restrict__ 
       for (int k = 0; k < RP; ++k) {
         u32x4 v = philox_sweep(half[GCHAIN_CALLS * w + q], key[k], rk);
         if (never) v = {max(v.a, 1u), max(v.b, 1u), max(v.c, 1u), max(v.d, 1u)};
-        ga[k] = shift_in_reject(ga[k], v.d, a.w);
-        gb[k] = shift_in_reject(gb[k], v.d, b.w);
-        ga[k] = shift_in_reject(ga[k], v.c, a.z);
-        gb[k] = shift_in_reject(gb[k], v.c, b.z);
-        ga[k] = shift_in_reject(ga[k], v.b, a.y);
-        gb[k] = shift_in_reject(gb[k], v.b, b.y);
-        ga[k] = shift_in_reject(ga[k], v.a, a.x);
-        gb[k] = shift_in_reject(gb[k], v.a, b.x);
+        ga[k] = shift_in_carry(ga[k], v.d, a.w);
+        gb[k] = shift_in_carry(gb[k], v.d, b.w);
+        ga[k] = shift_in_carry(ga[k], v.c, a.z);
+        gb[k] = shift_in_carry(gb[k], v.c, b.z);
+        ga[k] = shift_in_carry(ga[k], v.b, a.y);
+        gb[k] = shift_in_carry(gb[k], v.b, b.y);
+        ga[k] = shift_in_carry(ga[k], v.a, a.x);
+        gb[k] = shift_in_carry(gb[k], v.a, b.x);
       }
     }
     uint32_t ra = ga[0], rb = gb[0];  // rejected as class A, as class B

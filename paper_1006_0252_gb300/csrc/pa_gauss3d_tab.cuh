@@ -52,6 +52,7 @@
 #pragma once
 #include "pa_colour3d.cuh"
 #include "pa_gauss3d.cuh"
+#include "pa_patterns.cuh"
 
 namespace pa {
 
@@ -139,39 +140,6 @@ __device__ __forceinline__ int fill_thresholds(uint32_t* __restrict__ s_thr, con
   return never;
 }
 
-// Patterns of the sites at bits b = 8 j + r of the words x[0..5]: byte j of
-// f[r], x_d at bit d + 2 of the byte (four times the pattern: a byte offset in
-// the site's entries).  Pairs of words are first merged into fields of two
-// bits (sites of even and of odd b), then fields of the three pairs into bytes.
-struct Patterns {
-  uint32_t f[8];
-  __device__ __forceinline__ explicit Patterns(const uint32_t (&x)[6]) {
-    uint32_t e[3], o[3];  // fields i of a byte: sites r = 2 i and 2 i + 1
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      e[d] = (x[2 * d] & 0x55555555u) | ((x[2 * d + 1] << 1) & 0xAAAAAAAAu);
-      o[d] = ((x[2 * d] >> 1) & 0x55555555u) | (x[2 * d + 1] & 0xAAAAAAAAu);
-    }
-    bytes(e, 0);
-    bytes(o, 1);
-  }
-  __device__ __forceinline__ void bytes(const uint32_t (&p)[3], int r) {
-    const uint32_t lo = (p[0] & 0x33333333u) | ((p[1] << 2) & 0xCCCCCCCCu);  // fields 0 and 2 of both pairs
-    const uint32_t hi = ((p[0] >> 2) & 0x33333333u) | (p[1] & 0xCCCCCCCCu);  // fields 1 and 3
-    f[r + 0] = ((lo << 2) & 0x3C3C3C3Cu) | ((p[2] << 6) & 0xC0C0C0C0u);
-    f[r + 2] = ((hi << 2) & 0x3C3C3C3Cu) | ((p[2] << 4) & 0xC0C0C0C0u);
-    f[r + 4] = ((lo >> 2) & 0x3C3C3C3Cu) | ((p[2] << 2) & 0xC0C0C0C0u);
-    f[r + 6] = ((hi >> 2) & 0x3C3C3C3Cu) | (p[2] & 0xC0C0C0C0u);
-  }
-};
-
-template <int OFF>
-__device__ __forceinline__ uint32_t load_shared(uint32_t addr) {
-  uint32_t t;
-  asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(t) : "r"(addr), "n"(OFF));
-  return t;
-}
-
 // The word updates of one half sweep, as walk_rows calls them.
 template <int L, int RP>
 struct TabUpdate {
@@ -236,9 +204,7 @@ struct TabUpdate {
             const uint32_t addr = __byte_perm(pat.f[b & 7], base, (uint32_t)(b >> 3) | 0x7650u);
             const uint32_t t = load_shared<m * EB>(addr);
             if constexpr (!FOLD) {
-              asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %3, %3;\n\t}"
-                  : "=r"(lo[k])
-                  : "r"(u[i]), "r"(t), "r"(lo[k]));
+              lo[k] = shift_in_carry(lo[k], u[i], t);
             } else {
               const uint32_t v = (u[i] >> 8) + t;
               uint32_t& acc = (m & 1) ? hi[k] : lo[k];

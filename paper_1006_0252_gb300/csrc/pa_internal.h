@@ -141,4 +141,45 @@ constexpr bool gtab_shape_ok(int L, int split, int rp) {
   if (split == 1) return L <= 8 && rp == 1;
   return (L == 4 || L == 8) && (split == 2 || split == 4) && rp == 2;
 }
+// Threshold-table kernel of general boxes (pa_boxtab.cuh): the geometry (extent
+// in x, words of a row, rows), P threads a column of `reps` replicas, `slots`
+// slots of a work item (whole warps of columns).
+struct BoxShape {
+  int Lx, G, Ly;
+  int P, reps, slots;
+};
+constexpr int BOX_TPB = 1024;
+constexpr int box_replicas(int S) { return S <= 8 ? 4 : 2; }  // most replicas of a word
+// Words after which the uniforms start a generator call again.
+constexpr int box_period(int S) { return S % 4 == 0 ? 1 : (S % 2 == 0 ? 2 : 4); }
+
+// Shared memory of a block in words: the threshold table (256-byte aligned; its
+// memory also takes the sums of the energies and then the word ranges'
+// energies), NH half-sweep tables of Q calls, the colour words at column stride
+// CS.
+struct BoxTabShape {
+  int Q, NH, CS, thr_words;
+  size_t words;
+};
+__host__ __device__ inline BoxTabShape boxtab_shape(int WR, int S, const BoxShape& b) {
+  BoxTabShape sh;
+  const int U = box_period(S), columns = b.slots / b.reps;
+  const int wpp = ((WR + U - 1) / U + b.P - 1) / b.P * U;
+  sh.Q = (WR * S + 3) / 4;
+  sh.CS = columns;
+  for (int cs = columns; b.P > 1 && cs < columns + 4; ++cs) {  // the P ranges on different banks, if they can be
+    const int m = (wpp * cs) % 32;
+    if (m % (32 / b.P) == 0 && ((m / (32 / b.P)) & 1)) {
+      sh.CS = cs;
+      break;
+    }
+  }
+  sh.thr_words = 128 * WR * S > b.P * b.slots ? 128 * WR * S : (b.P * b.slots + 3) / 4 * 4;
+  const size_t fixed = 64 + (size_t)sh.thr_words + 2 * (size_t)WR * sh.CS;
+  const long long room = (224ll * 1024 - 4ll * (long long)fixed) / (16ll * sh.Q);
+  sh.NH = room >= 20 ? 20 : (room < 2 ? 2 : (int)(room & ~1ll));
+  sh.words = fixed + 4 * (size_t)sh.NH * sh.Q;
+  return sh;
+}
+
 }  // namespace pa

@@ -93,3 +93,26 @@ def test_chosen_gauss_chain_shape_bit_exact(N, is_open, R0, split):
     assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.energies(), c.energies())
     assert np.array_equal(g.spins(), c.spins())
+
+
+# (Lx, Ly, Lz, periodic mask, R0): general boxes whose words hold 4, 6, 8, 9, 12,
+# 15 and 16 sites of a colour (uniforms that start a call again after 1, 2 and 4
+# words), with 1, 2 and 4 replicas a thread.
+@pytest.mark.parametrize("gaussian", [False, True])
+@pytest.mark.parametrize("Lx,Ly,Lz,mask,R0", [(8, 6, 5, 3, 20001), (8, 6, 5, 3, 1999), (4, 4, 3, 3, 30001),
+                                              (4, 8, 8, 3, 5003), (6, 4, 3, 3, 20003), (8, 4, 3, 3, 9001),
+                                              (6, 8, 5, 3, 8009), (8, 8, 8, 3, 7001), (2, 3, 2, 0, 40001),
+                                              (32, 2, 3, 1, 2503)])
+def test_chosen_box_shape_bit_exact(Lx, Ly, Lz, mask, R0, gaussian):
+    J = inputs.gaussian_couplings_lattice(Lx, Ly, Lz, 6) if gaussian else inputs.couplings_lattice(Lx, Ly, Lz, 6, 3)
+    cap = R0 + 4000
+    g = pa.Run(J, Lx, 3, R0, 41, R_cap=cap, gaussian=gaussian, Ls=(Lx, Ly, Lz), periodic_mask=mask)
+    assert pa.pa_sweep_shape(g._h)[0] == 1024
+    c = (o.GaussRun if gaussian else o.Run)(J, 3, Lx, Ly, Lz, mask, R0=R0, R_cap=cap, seed=41)
+    for beta, sweeps in ((1e-6, 1), (0.4, 1), (0.9, 0), (1.5, 1), (2.5, 0), (5.0, 0), (12.0, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+        assert g.observables()["R"] == c.state().R, beta
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.energies().astype(np.int64), c.energies().astype(np.int64))
+    assert np.array_equal(g.spins(), c.spins())
