@@ -354,11 +354,15 @@ __device__ __forceinline__ int64_t block_exscan_i64(int64_t v, int64_t* s_warp, 
 // Inverse-CDF walk of one Poisson piece (mean am, P(0) = p0) for uniform u:
 // P_k = (P_{k-1} am) / k, C_k = C_{k-1} + P_k, stop at the first k with
 // u < C_k (or at POISSON_KMAX).  The division by k is the exact integer one
-// of div_small_rn, the same double as a correctly rounded division.
+// of div_small_rn, the same double as a correctly rounded division; u and C are
+// not negative, so they compare as their bits do (at_least).
+__device__ __forceinline__ bool at_least(double u, double C) {
+  return __double_as_longlong(u) >= __double_as_longlong(C);
+}
 __device__ __forceinline__ int poisson_piece(double u, double am, double p0) {
   int k = 0;
   double P = p0, C = p0;
-  while (u >= C && k < POISSON_KMAX) {
+  while (at_least(u, C) && k < POISSON_KMAX) {
     k = k + 1;
     P = div_small_rn(__dmul_rn(P, am), (uint32_t)k);
     C = __dadd_rn(C, P);
@@ -366,15 +370,10 @@ __device__ __forceinline__ int poisson_piece(double u, double am, double p0) {
   return k;
 }
 
-__device__ __forceinline__ int64_t pieces_sum(const RunDev& R, int64_t j, int64_t first, int64_t stride, int64_t m,
-                                              double am, double p0) {
-  const uint32_t stp = (uint32_t)R.step;
-  int64_t c = 0;
-  for (int64_t piece = first; piece < m; piece += stride) {
-    const u32x4 r = philox_seeded(R.seed, (uint32_t)piece, (uint32_t)j, stp, TAG_RESAMPLE);
-    c += poisson_piece(u53(r.a, r.b), am, p0);
-  }
-  return c;
+// Copies of one piece of replica j from its own mean.
+__device__ __forceinline__ int piece_copies(const RunDev& R, int64_t j, int64_t piece, double am, double p0) {
+  const u32x4 r = philox_seeded(R.seed, (uint32_t)piece, (uint32_t)j, (uint32_t)R.step, TAG_RESAMPLE);
+  return poisson_piece(u53(r.a, r.b), am, p0);
 }
 
 // The same walk from a bin's table: with U the 53-bit integer of the
@@ -393,7 +392,7 @@ __device__ __forceinline__ int poisson_piece_tab(uint64_t U, const uint64_t* __r
   if (k < POISSON_TAB) return k;
   const double u = __dmul_rn((double)U, 0x1.0p-53);
   k = POISSON_TAB - 1;
-  while (u >= C && k < POISSON_KMAX) {
+  while (at_least(u, C) && k < POISSON_KMAX) {
     k = k + 1;
     P = div_small_rn(__dmul_rn(P, am), (uint32_t)k);
     C = __dadd_rn(C, P);
@@ -401,30 +400,17 @@ __device__ __forceinline__ int poisson_piece_tab(uint64_t U, const uint64_t* __r
   return k;
 }
 
-__device__ __forceinline__ int64_t pieces_sum_tab(const RunDev& R, int64_t j, int64_t first, int64_t stride,
-                                                  int64_t m, int b) {
-  const uint32_t stp = (uint32_t)R.step;
-  const uint64_t* thr = R.bin_thr + (size_t)b * POISSON_TAB;
-  int64_t c = 0;
-  for (int64_t piece = first; piece < m; piece += stride) {
-    const u32x4 r = philox_seeded(R.seed, (uint32_t)piece, (uint32_t)j, stp, TAG_RESAMPLE);
-    const uint64_t U = ((((uint64_t)r.a) << 32) | (uint64_t)r.b) >> 11;
-    c += poisson_piece_tab(U, thr, R.bin_end[2 * b], R.bin_end[2 * b + 1], R.bin_am[b]);
-  }
-  return c;
+// Copies of one piece of replica j from the tables of its bin b.
+__device__ __forceinline__ int piece_copies_tab(const RunDev& R, int64_t j, int64_t piece, int b) {
+  const u32x4 r = philox_seeded(R.seed, (uint32_t)piece, (uint32_t)j, (uint32_t)R.step, TAG_RESAMPLE);
+  const uint64_t U = ((((uint64_t)r.a) << 32) | (uint64_t)r.b) >> 11;
+  return poisson_piece_tab(U, R.bin_thr + (size_t)b * POISSON_TAB, R.bin_end[2 * b], R.bin_end[2 * b + 1],
+                           R.bin_am[b]);
 }
 
-// Poisson pieces of replica j: from the per-bin tables (+-1 couplings) or
-// from the replica's own weight (Gaussian couplings; same arithmetic as the
-// per-bin tables of k_prepare).
+// Poisson pieces of replica j of a Gaussian run from its own weight (the
+// arithmetic of the per-bin tables of k_prepare).
 __device__ __forceinline__ void replica_poisson(RunDev& R, int64_t j, int64_t* m, double* am, double* p0) {
-  if (R.model == 0) {
-    const int b = (R.E[R.cur][j] + R.Nb) >> 1;
-    *m = R.bin_m[b];
-    *am = R.bin_am[b];
-    *p0 = R.bin_p0[b];
-    return;
-  }
   double a = __ddiv_rn(__dmul_rn((double)R.Rt_next, R.w_rep[j]), R.Qp_staged);
   // w_j <= Q' makes a <= R_target (up to rounding); anything else (a stale or
   // unset weight) draws nothing and flags the run instead of sampling an
@@ -444,72 +430,82 @@ __device__ __forceinline__ void replica_poisson(RunDev& R, int64_t j, int64_t* m
   *p0 = dexp_np(-a1);
 }
 
-// Replicas whose mean needs more pieces than this are sampled by the whole
-// block (pieces split over the threads, counts summed): after a large
-// temperature step a few low-energy replicas carry most of the weight.
-constexpr int64_t HEAVY_PIECES = 8;
+// A replica whose mean is above this, or that needs several pieces, is left to
+// the second pass of k_copies.
+constexpr double LONG_MEAN = 4.0;
 
+// Last i in [0, CHUNK) with off[i] <= t (off does not decrease): of entries of
+// which some are empty, the one that holds t.
+template <class T>
+__device__ __forceinline__ int holder(const T* __restrict__ off, T t) {
+  int i = 0;
+#pragma unroll
+  for (int step = CHUNK / 2; step >= 1; step >>= 1)
+    if (off[i + step] <= t) i += step;
+  return i;
+}
+
+// Copy counts of a chunk of replicas.  A draw is a walk of about as many
+// dependent FP64 steps as copies (each instruction holds a sub-partition for 64
+// cycles), so after a large temperature step a warp waits for its heaviest
+// replica, and families of heavy replicas lie side by side.  So the first pass
+// draws only the short walks; the pieces of all other replicas of the chunk are
+// laid out one after the other and drawn by the block's threads in turn.
+// L = 10, 20000 Gaussian replicas, the first 13 of 40 steps to beta = 4: 59 us a
+// launch with the heavy replicas one by one and the middling ones in their own
+// threads, 27 so; 1.2e6 +-1 replicas at steps of 0.2 in beta 124 -> 85.  (The
+// bound of the first pass hardly matters: 2, 4 and 7 are alike within 1 %.)
 __global__ void __launch_bounds__(CHUNK) k_copies(RunDev* __restrict__ runs, const Work* __restrict__ table) {
   __shared__ int64_t s_warp[CHUNK / 32];
-  __shared__ int32_t s_heavy[CHUNK];
-  __shared__ int s_nheavy;
+  __shared__ int64_t s_off[CHUNK];           // first piece of each replica in the second pass
+  __shared__ unsigned long long s_cnt[CHUNK];
+  __shared__ double s_am[CHUNK], s_p0[CHUNK];  // Gaussian runs
+  __shared__ int32_t s_bin[CHUNK];             // +-1 runs
   const Work wk = table[blockIdx.x];
   RunDev& R = runs[wk.run];
   if (R.skip) return;
-  const int64_t j = (int64_t)wk.first + threadIdx.x;
+  const int tid = threadIdx.x;
+  const int64_t j = (int64_t)wk.first + tid;
   const int64_t Rold = R.R;
   if ((int64_t)wk.first >= Rold) {
-    if (threadIdx.x == 0) R.chunk_sum[wk.first / CHUNK] = 0;
+    if (tid == 0) R.chunk_sum[wk.first / CHUNK] = 0;
     return;
   }
-  if (threadIdx.x == 0) s_nheavy = 0;
-  __syncthreads();
-  int64_t c = 0;
+  int64_t c = 0, later = 0;  // copies; pieces of the second pass
   if (j < Rold) {
-    int64_t m;
-    double am, p0;
-    if (R.model == 0) {  // +-1 couplings: the bin's tables
+    if (R.model == 0) {
       const int b = (R.E[R.cur][j] + R.Nb) >> 1;
-      m = R.bin_m[b];
-      if (m > HEAVY_PIECES) {
-        s_heavy[atomicAdd(&s_nheavy, 1)] = (int32_t)(j - wk.first);
-      } else {
-        c = pieces_sum_tab(R, j, 0, 1, m, b);
-        R.copies[j] = (int32_t)c;
-      }
+      const int64_t m = R.bin_m[b];
+      s_bin[tid] = b;
+      if (m > 1 || R.bin_am[b] > LONG_MEAN) later = m;
+      else c = piece_copies_tab(R, j, 0, b);
     } else {
+      int64_t m;
+      double am, p0;
       replica_poisson(R, j, &m, &am, &p0);
-      if (m > HEAVY_PIECES) {
-        s_heavy[atomicAdd(&s_nheavy, 1)] = (int32_t)(j - wk.first);
-      } else {
-        c = pieces_sum(R, j, 0, 1, m, am, p0);
-        R.copies[j] = (int32_t)c;
-      }
+      s_am[tid] = am;
+      s_p0[tid] = p0;
+      if (m > 1 || am > LONG_MEAN) later = m;
+      else c = piece_copies(R, j, 0, am, p0);
     }
   }
-  __syncthreads();
-  const int nh = s_nheavy;
-  for (int h = 0; h < nh; ++h) {
-    const int64_t jh = (int64_t)wk.first + s_heavy[h];
-    int64_t mh;
-    double amh, p0h;
-    int64_t part;
-    if (R.model == 0) {
-      const int bh = (R.E[R.cur][jh] + R.Nb) >> 1;
-      part = pieces_sum_tab(R, jh, threadIdx.x, CHUNK, R.bin_m[bh], bh);
-    } else {
-      replica_poisson(R, jh, &mh, &amh, &p0h);
-      part = pieces_sum(R, jh, threadIdx.x, CHUNK, mh, amh, p0h);
-    }
-    const int64_t tot = block_sum_i64(part, s_warp);
-    if (threadIdx.x == 0) {
-      R.copies[jh] = (int32_t)(tot > 0x7FFFFFFF ? 0x7FFFFFFF : tot);
-      c += tot;  // thread 0 carries the heavy totals into the chunk sum
+  if (__syncthreads_or(later > 0)) {
+    int64_t pieces;
+    s_cnt[tid] = 0ull;
+    s_off[tid] = block_exscan_i64(later, s_warp, &pieces);
+    __syncthreads();
+    for (int64_t t = tid; t < pieces; t += CHUNK) {
+      const int h = holder(s_off, t);
+      const int64_t piece = t - s_off[h], jh = (int64_t)wk.first + h;
+      const int k = R.model == 0 ? piece_copies_tab(R, jh, piece, s_bin[h]) : piece_copies(R, jh, piece, s_am[h], s_p0[h]);
+      atomicAdd(&s_cnt[h], (unsigned long long)k);
     }
     __syncthreads();
+    if (later > 0) c = (int64_t)s_cnt[tid];
   }
+  if (j < Rold) R.copies[j] = (int32_t)(c > 0x7FFFFFFF ? 0x7FFFFFFF : c);
   const int64_t tot = block_sum_i64(c, s_warp);
-  if (threadIdx.x == 0) R.chunk_sum[wk.first / CHUNK] = tot;
+  if (tid == 0) R.chunk_sum[wk.first / CHUNK] = tot;
 }
 
 __global__ void __launch_bounds__(CHUNK) k_scan(RunDev* __restrict__ runs, const int32_t* __restrict__ ids) {
@@ -538,8 +534,13 @@ __global__ void __launch_bounds__(CHUNK) k_scan(RunDev* __restrict__ runs, const
   }
 }
 
+// Source of every new slot.  The block's threads take the new slots of the
+// chunk in turn and look their replica up in the offsets: with a thread writing
+// the copies of its own replica a chunk took as long as its heaviest one (279
+// us at worst in a batch of 1.2e6 replicas at steps of 0.2 in beta, 60 so).
 __global__ void __launch_bounds__(CHUNK) k_scatter(RunDev* __restrict__ runs, const Work* __restrict__ table) {
   __shared__ int64_t s_warp[CHUNK / 32];
+  __shared__ int64_t s_off[CHUNK];
   const Work wk = table[blockIdx.x];
   RunDev& R = runs[wk.run];
   if (R.skip) return;
@@ -548,9 +549,10 @@ __global__ void __launch_bounds__(CHUNK) k_scatter(RunDev* __restrict__ runs, co
   const int64_t j = (int64_t)wk.first + threadIdx.x;
   const int64_t c = (j < Rold) ? R.copies[j] : 0;
   int64_t tot;
-  const int64_t ex = block_exscan_i64(c, s_warp, &tot);
-  const int64_t off = R.chunk_off[wk.first / CHUNK] + ex;
-  for (int64_t q = 0; q < c; ++q) R.src[off + q] = (int32_t)j;
+  s_off[threadIdx.x] = block_exscan_i64(c, s_warp, &tot);
+  __syncthreads();
+  int32_t* __restrict__ src = R.src + R.chunk_off[wk.first / CHUNK];
+  for (int64_t q = threadIdx.x; q < tot; q += CHUNK) src[q] = wk.first + holder(s_off, q);
 }
 
 // Commit the step (or, after a device-detected error, leave the state as it was).
