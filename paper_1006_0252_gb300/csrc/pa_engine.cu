@@ -785,6 +785,8 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
   std::vector<Work> ct;
   for (int r = 0; r < n_runs; ++r)
     for (int64_t f = 0; f < E.h[r].R_cap; f += CHUNK) ct.push_back({r, (int32_t)f});
+  E.small = E.model == 0;
+  for (const RunDev& d : E.h) E.small = E.small && d.R_cap <= SMALL_RUN;
   E.n_copy_work = (int)ct.size();
   E.d_copy_table = (Work*)E.dalloc(sizeof(Work) * ct.size());
   if (!E.d_copy_table) return fail(PA_ERR_OOM, "work table allocation refused");
@@ -839,7 +841,6 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
   return PA_OK;
 }
 
-// Enqueue one annealing step for all runs of the engine.
 // Reweighting factors, Q', ln Q and the Poisson means of the coming step
 // (staged, not committed).
 int engine_prep(Engine& E, bool ovr, double beta, int theta, int64_t Rt) {
@@ -855,14 +856,21 @@ int engine_prep(Engine& E, bool ovr, double beta, int theta, int64_t Rt) {
   return PA_OK;
 }
 
-static int engine_step(Engine& E, bool ovr, double beta, int theta, int64_t Rt) {
-  NvtxRange step_range("pa_step");
-  int pst;
+// Resampling of one annealing step (staged, not committed).  The stages of
+// larger runs are a launch each; small ones take one for all of them, which
+// also commits the step before where asked.
+static int engine_resample(Engine& E, bool commit_first, bool ovr, double beta, int theta, int64_t Rt) {
+  if (E.small) {
+    NvtxRange r("reweight+copies+sources (k_resample)");
+    PA_CUDA(launch_resample(E.d_runs, nullptr, E.n, commit_first, ovr, beta, theta, Rt, E.st));
+    E.launches += 1;
+    return PA_OK;
+  }
   {
     NvtxRange r("reweight+Q (k_prepare)");
-    pst = engine_prep(E, ovr, beta, theta, Rt);
+    const int pst = engine_prep(E, ovr, beta, theta, Rt);
+    if (pst != PA_OK) return pst;
   }
-  if (pst != PA_OK) return pst;
   {
     NvtxRange r("copy counts (k_copies)");
     PA_CUDA(launch_copies(E.d_runs, E.d_copy_table, E.n_copy_work, E.st));
@@ -875,6 +883,18 @@ static int engine_step(Engine& E, bool ovr, double beta, int theta, int64_t Rt) 
     NvtxRange r("replica sources (k_scatter)");
     PA_CUDA(launch_scatter(E.d_runs, E.d_copy_table, E.n_copy_work, E.st));
   }
+  E.launches += 4;
+  return PA_OK;
+}
+
+// Enqueue one annealing step for all runs of the engine.  In a schedule
+// (after, before: a step precedes, follows) small runs commit a step at the
+// start of the next.
+static int engine_step(Engine& E, bool ovr, double beta, int theta, int64_t Rt, bool after = false,
+                       bool before = false) {
+  NvtxRange step_range("pa_step");
+  const int pst = engine_resample(E, E.small && after, ovr, beta, theta, Rt);
+  if (pst != PA_OK) return pst;
   NvtxRange sweep_range("gather+sweeps+measure (k_sweep*)");
   for (auto& c : E.cls) {
     cudaEvent_t a = nullptr, b = nullptr;
@@ -894,11 +914,12 @@ static int engine_step(Engine& E, bool ovr, double beta, int theta, int64_t Rt) 
       (E.capturing ? E.graph_ev : E.prof_ev).push_back({a, b});
     }
   }
-  {
+  E.launches += (int64_t)E.cls.size();
+  if (!(E.small && before)) {
     NvtxRange r("commit (k_commit)");
     PA_CUDA(launch_commit(E.d_runs, nullptr, E.n, E.st));
+    E.launches += 1;
   }
-  E.launches += 5 + (int64_t)E.cls.size();
   E.host_steps += 1;
   return PA_OK;
 }
@@ -1005,7 +1026,7 @@ int engine_run_schedule(Engine& E, int n_steps, const double* betas, int per_run
   E.harvest_graph_timing();
   if (!use_graph) {
     for (int k = 0; k < n_steps; ++k) {
-      int st = engine_step(E, false, 0.0, 0, 0);
+      int st = engine_step(E, false, 0.0, 0, 0, k > 0, k + 1 < n_steps);
       if (st != PA_OK) return st;
     }
     return PA_OK;
@@ -1019,7 +1040,7 @@ int engine_run_schedule(Engine& E, int n_steps, const double* betas, int per_run
     const int64_t saved = E.host_steps, saved_launches = E.launches, saved_seen = E.prof_seen;
     E.capturing = true;
     E.prof_seen = 0;
-    for (int k = 0; k < n_steps && st == PA_OK; ++k) st = engine_step(E, false, 0.0, 0, 0);
+    for (int k = 0; k < n_steps && st == PA_OK; ++k) st = engine_step(E, false, 0.0, 0, 0, k > 0, k + 1 < n_steps);
     E.capturing = false;
     E.graph_kernels = E.launches - saved_launches;
     E.host_steps = saved;

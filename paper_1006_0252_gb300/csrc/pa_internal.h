@@ -18,6 +18,7 @@ constexpr uint32_t TAG_BOOT = 0x4D000000u;
 constexpr int POISSON_KMAX = 512;  // longest inverse-CDF walk of one piece (mean <= 32)
 constexpr int POISSON_TAB = 8;     // tabulated inverse-CDF steps per energy bin (+-1 couplings)
 constexpr int CHUNK = 256;         // slots per block in the resampling kernels
+constexpr int SMALL_RUN = 2048;    // largest population capacity resampled by one block
 
 // Error codes (mirrors pa.h).
 constexpr int OK = 0, ERR_INVALID = 1, ERR_OOM = 2, ERR_CAPACITY = 3, ERR_EXTINCT = 4,

@@ -133,6 +133,30 @@ __device__ __forceinline__ void commit_energy_sums(RunDev& R) {
   }
 }
 
+// Commit the step whose population has been measured (or, after a
+// device-detected error, leave the state as it was).
+__device__ __forceinline__ void commit_step(RunDev& R) {
+  if (R.skip || R.error) return;
+  R.cur ^= 1;
+  R.R = R.R_next;
+  R.beta = R.beta_next;
+  R.mbF = R.mbF_staged;
+  R.lnQ_last = R.lnQ_staged;
+  R.Qp_last = R.Qp_staged;
+  R.step += 1;
+  R.sweeps += R.theta_next;
+  commit_energy_sums(R);
+  const int64_t k = R.step;
+  if (k <= R.max_steps) {
+    R.rec_beta[k] = R.beta;
+    R.rec_lnQ[k] = R.lnQ_last;
+    R.rec_mbF[k] = R.mbF;
+    R.rec_R[k] = R.R;
+    R.rec_sumE[k] = R.sumE;
+    R.rec_sumE2[k] = R.sumE2;
+  }
+}
+
 __global__ void k_init_finish(RunDev* __restrict__ runs, const int32_t* __restrict__ ids, int n) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
@@ -153,19 +177,18 @@ constexpr int PREP_THREADS = 256;
 constexpr int PREP_WIN = 2048;  // bins of one shared-memory window of the Q' sum
 
 // Every FP64 instruction holds an SM sub-partition for about 64 cycles on
-// this GPU, so the kernel keeps the FP64 chains short and side by side: the
+// this GPU, so the block keeps the FP64 chains short and side by side: the
 // per-bin work is spread over the block, the Q' tree reads its terms from
 // shared memory and visits only the occupied range of bins, and ln Q and the
 // thresholds are computed by threads without bins while the others build the
-// Poisson tables.
-__global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ runs,
-                                                          const int32_t* __restrict__ ids, int use_override,
-                                                          double beta_o, int theta_o, int64_t Rt_o) {
+// Poisson tables.  Returns false (in all threads) where the run has no step to
+// take.
+template <int NT>
+__device__ __forceinline__ bool prepare_block(RunDev& R, int use_override, double beta_o, int theta_o, int64_t Rt_o) {
   __shared__ int s_ok, s_bmin, s_bmax, s_theta, s_nocc;
   __shared__ double s_bn, s_Qp;
   __shared__ long long s_Rt;
   __shared__ double s_term[PREP_WIN];
-  RunDev& R = runs[ids ? ids[blockIdx.x] : blockIdx.x];
   const int tid = threadIdx.x;
   if (tid == 0) {
     int ok = 1;
@@ -199,7 +222,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
     s_nocc = 0;
   }
   __syncthreads();
-  if (!s_ok) return;
+  if (!s_ok) return false;
   const double bn = s_bn;
   const int64_t Rt = s_Rt;
   const double dbeta = __dsub_rn(bn, R.beta);
@@ -210,7 +233,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
   // occupied bins, compacted so the FP64 work below spreads evenly over the
   // block; the first and last occupied bins
   int32_t* __restrict__ occ = R.occ;
-  for (int b = tid; b < nbins; b += PREP_THREADS)
+  for (int b = tid; b < nbins; b += NT)
     if (h[b] != 0u) {
       atomicMin(&s_bmin, b);
       atomicMax(&s_bmax, b);
@@ -220,7 +243,7 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
   const int bmin = s_bmin, bmax = s_bmax;
   const int nocc = s_nocc;
   // reweighting factors of the occupied bins, w_b = exp(-dbeta (E_b - E_min))
-  for (int i = tid; i < nocc; i += PREP_THREADS) {
+  for (int i = tid; i < nocc; i += NT) {
     const int b = occ[i];
     w[b] = dexp_np(-__dmul_rn(dbeta, (double)(2 * (b - bmin))));
   }
@@ -232,9 +255,9 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
   double acc = 0.0;
   for (int lo = bmin & ~31; lo <= bmax; lo += PREP_WIN) {
     const int span = min(PREP_WIN, bmax + 1 - lo);
-    for (int t = tid; t < span; t += PREP_THREADS) s_term[t] = 0.0;
+    for (int t = tid; t < span; t += NT) s_term[t] = 0.0;
     __syncthreads();
-    for (int i = tid; i < nocc; i += PREP_THREADS) {
+    for (int i = tid; i < nocc; i += NT) {
       const int b = occ[i];
       if (b >= lo && b < lo + span) s_term[b - lo] = __dmul_rn((double)h[b], w[b]);
     }
@@ -251,8 +274,8 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
   __syncthreads();
   const double Qp = s_Qp;
   // ln Q, the staged -beta F~ and the thresholds by the last threads, which
-  // have no bin while nocc < PREP_THREADS - 8
-  if (tid == PREP_THREADS - 1) {
+  // have no bin while nocc < NT - 8
+  if (tid == NT - 1) {
     const int64_t Emin = 2 * (int64_t)bmin - R.Nb;
     const double lnQ = __dsub_rn(__dsub_rn(log(Qp), log((double)R.R)), __dmul_rn(dbeta, (double)Emin));
     R.lnQ_staged = lnQ;
@@ -266,15 +289,15 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
     R.sumE2_next = 0ull;
     R.skip = 0;
   }
-  if (tid >= PREP_THREADS - 9 && tid < PREP_THREADS - 1) {
-    const int d = tid - (PREP_THREADS - 9);
+  if (tid >= NT - 9 && tid < NT - 1) {
+    const int d = tid - (NT - 9);
     R.thr[d] = (d == 0 || d == 7) ? 0u : metropolis_threshold(bn, 2 * d);
   }
   // Poisson means a_b = R_target w_b / Q' = (R/R~) tau_j (Eq. (1)), split in
   // m = ceil(a/32) pieces when a > 32 (a / 32 and a / 1 are exact, so they
   // are taken as a product and as a itself).
   const double Rtd = (double)Rt;
-  for (int i = tid; i < nocc; i += PREP_THREADS) {
+  for (int i = tid; i < nocc; i += NT) {
     const int b = occ[i];
     const double a = __ddiv_rn(__dmul_rn(Rtd, w[b]), Qp);
     int64_t m = 1;
@@ -303,7 +326,14 @@ __global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ r
     R.bin_end[2 * b + 1] = C;
   }
   uint32_t* hn = R.hist[R.cur ^ 1];
-  for (int b = tid; b < nbins; b += PREP_THREADS) hn[b] = 0u;
+  for (int b = tid; b < nbins; b += NT) hn[b] = 0u;
+  return true;
+}
+
+__global__ void __launch_bounds__(PREP_THREADS) k_prepare(RunDev* __restrict__ runs,
+                                                          const int32_t* __restrict__ ids, int use_override,
+                                                          double beta_o, int theta_o, int64_t Rt_o) {
+  prepare_block<PREP_THREADS>(runs[ids ? ids[blockIdx.x] : blockIdx.x], use_override, beta_o, theta_o, Rt_o);
 }
 
 // ---------------------------------------------------------------------------
@@ -380,8 +410,7 @@ __device__ __forceinline__ int piece_copies(const RunDev& R, int64_t j, int64_t 
 // uniform, the walk stops at the first k with U < thr[k]; the thresholds do
 // not decrease, so that k is the number of thresholds U reaches.  Past the
 // table the walk goes on from the stored state, step by step as above.
-__device__ __forceinline__ int poisson_piece_tab(uint64_t U, const uint64_t* __restrict__ thr, double P, double C,
-                                                 double am) {
+__device__ __forceinline__ int poisson_piece_tab(uint64_t U, const uint64_t* thr, double P, double C, double am) {
   const ulonglong2* t2 = reinterpret_cast<const ulonglong2*>(thr);
   int k = 0;
 #pragma unroll
@@ -434,13 +463,13 @@ __device__ __forceinline__ void replica_poisson(RunDev& R, int64_t j, int64_t* m
 // the second pass of k_copies.
 constexpr double LONG_MEAN = 4.0;
 
-// Last i in [0, CHUNK) with off[i] <= t (off does not decrease): of entries of
+// Last i in [0, N) with off[i] <= t (off does not decrease): of entries of
 // which some are empty, the one that holds t.
-template <class T>
-__device__ __forceinline__ int holder(const T* __restrict__ off, T t) {
+template <int N>
+__device__ __forceinline__ int holder(const int64_t* off, int64_t t) {
   int i = 0;
 #pragma unroll
-  for (int step = CHUNK / 2; step >= 1; step >>= 1)
+  for (int step = N / 2; step >= 1; step >>= 1)
     if (off[i + step] <= t) i += step;
   return i;
 }
@@ -495,7 +524,7 @@ __global__ void __launch_bounds__(CHUNK) k_copies(RunDev* __restrict__ runs, con
     s_off[tid] = block_exscan_i64(later, s_warp, &pieces);
     __syncthreads();
     for (int64_t t = tid; t < pieces; t += CHUNK) {
-      const int h = holder(s_off, t);
+      const int h = holder<CHUNK>(s_off, t);
       const int64_t piece = t - s_off[h], jh = (int64_t)wk.first + h;
       const int k = R.model == 0 ? piece_copies_tab(R, jh, piece, s_bin[h]) : piece_copies(R, jh, piece, s_am[h], s_p0[h]);
       atomicAdd(&s_cnt[h], (unsigned long long)k);
@@ -506,6 +535,19 @@ __global__ void __launch_bounds__(CHUNK) k_copies(RunDev* __restrict__ runs, con
   if (j < Rold) R.copies[j] = (int32_t)(c > 0x7FFFFFFF ? 0x7FFFFFFF : c);
   const int64_t tot = block_sum_i64(c, s_warp);
   if (tid == 0) R.chunk_sum[wk.first / CHUNK] = tot;
+}
+
+// The population after resampling; a run that dies out or outgrows its buffers
+// stays as it is.
+__device__ __forceinline__ void set_population(RunDev& R, int64_t total) {
+  R.R_next = total;
+  if (total == 0) {
+    R.error = ERR_EXTINCT;
+    R.skip = 1;
+  } else if (total > R.R_cap) {
+    R.error = ERR_CAPACITY;
+    R.skip = 1;
+  }
 }
 
 __global__ void __launch_bounds__(CHUNK) k_scan(RunDev* __restrict__ runs, const int32_t* __restrict__ ids) {
@@ -522,16 +564,7 @@ __global__ void __launch_bounds__(CHUNK) k_scan(RunDev* __restrict__ runs, const
     if (i < nch) R.chunk_off[i] = running + ex;
     running += tot;
   }
-  if (threadIdx.x == 0) {
-    R.R_next = running;
-    if (running == 0) {
-      R.error = ERR_EXTINCT;
-      R.skip = 1;
-    } else if (running > R.R_cap) {
-      R.error = ERR_CAPACITY;
-      R.skip = 1;
-    }
-  }
+  if (threadIdx.x == 0) set_population(R, running);
 }
 
 // Source of every new slot.  The block's threads take the new slots of the
@@ -552,33 +585,73 @@ __global__ void __launch_bounds__(CHUNK) k_scatter(RunDev* __restrict__ runs, co
   s_off[threadIdx.x] = block_exscan_i64(c, s_warp, &tot);
   __syncthreads();
   int32_t* __restrict__ src = R.src + R.chunk_off[wk.first / CHUNK];
-  for (int64_t q = threadIdx.x; q < tot; q += CHUNK) src[q] = wk.first + holder(s_off, q);
+  for (int64_t q = threadIdx.x; q < tot; q += CHUNK) src[q] = wk.first + holder<CHUNK>(s_off, q);
 }
 
-// Commit the step (or, after a device-detected error, leave the state as it was).
+// The whole resampling of a +-1 run of at most SMALL_RUN replicas by one block:
+// k_prepare, k_copies and k_scatter without the launches in between.  A run of
+// 1000 replicas at L = 4 took 30.7 us a step with six launches (of which 12.5
+// the sweep) in a graph, 24.5 with this one and the sweep.
+constexpr int SMALL_THREADS = 1024;
+__global__ void __launch_bounds__(SMALL_THREADS) k_resample(RunDev* __restrict__ runs, const int32_t* __restrict__ ids,
+                                                            int commit_first, int use_override, double beta_o,
+                                                            int theta_o, int64_t Rt_o) {
+  constexpr int NT = SMALL_THREADS;
+  __shared__ int64_t s_warp[NT / 32];
+  __shared__ int64_t s_off[NT];
+  __shared__ unsigned long long s_cnt[NT];
+  __shared__ int32_t s_bin[NT];
+  RunDev& R = runs[ids ? ids[blockIdx.x] : blockIdx.x];
+  if (commit_first) {
+    if (threadIdx.x == 0) commit_step(R);
+    __syncthreads();
+  }
+  if (!prepare_block<NT>(R, use_override, beta_o, theta_o, Rt_o)) return;
+  __syncthreads();  // the bins' tables in place
+  const int tid = threadIdx.x;
+  const int64_t Rold = R.R, cap = R.R_cap;
+  const int32_t* E = R.E[R.cur];
+  int64_t running = 0;
+  for (int64_t base = 0; base < Rold; base += NT) {
+    const int64_t j = base + tid;
+    int64_t c = 0, later = 0;
+    if (j < Rold) {
+      const int b = (E[j] + R.Nb) >> 1;
+      const int64_t m = R.bin_m[b];
+      s_bin[tid] = b;
+      if (m > 1 || R.bin_am[b] > LONG_MEAN) later = m;
+      else c = piece_copies_tab(R, j, 0, b);
+    }
+    if (__syncthreads_or(later > 0)) {
+      int64_t pieces;
+      s_cnt[tid] = 0ull;
+      s_off[tid] = block_exscan_i64(later, s_warp, &pieces);
+      __syncthreads();
+      for (int64_t t = tid; t < pieces; t += NT) {
+        const int h = holder<NT>(s_off, t);
+        atomicAdd(&s_cnt[h], (unsigned long long)piece_copies_tab(R, base + h, t - s_off[h], s_bin[h]));
+      }
+      __syncthreads();
+      if (later > 0) c = (int64_t)s_cnt[tid];
+    }
+    const int32_t kept = (int32_t)(c > 0x7FFFFFFF ? 0x7FFFFFFF : c);
+    if (j < Rold) R.copies[j] = kept;
+    int64_t tot;
+    const int64_t ex = block_exscan_i64(c, s_warp, &tot);
+    s_off[tid] = ex;
+    __syncthreads();
+    // a run past its capacity is not swept: the slots it has room for are enough
+    const int64_t room = cap - running;
+    for (int64_t q = tid; q < tot && q < room; q += NT) R.src[running + q] = (int32_t)(base + holder<NT>(s_off, q));
+    running += tot;
+    __syncthreads();  // the offsets are no longer read
+  }
+  if (tid == 0) set_population(R, running);
+}
+
 __global__ void k_commit(RunDev* __restrict__ runs, const int32_t* __restrict__ ids, int n) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  RunDev& R = runs[ids ? ids[t] : t];
-  if (R.skip || R.error) return;
-  R.cur ^= 1;
-  R.R = R.R_next;
-  R.beta = R.beta_next;
-  R.mbF = R.mbF_staged;
-  R.lnQ_last = R.lnQ_staged;
-  R.Qp_last = R.Qp_staged;
-  R.step += 1;
-  R.sweeps += R.theta_next;
-  commit_energy_sums(R);
-  const int64_t k = R.step;
-  if (k <= R.max_steps) {
-    R.rec_beta[k] = R.beta;
-    R.rec_lnQ[k] = R.lnQ_last;
-    R.rec_mbF[k] = R.mbF;
-    R.rec_R[k] = R.R;
-    R.rec_sumE[k] = R.sumE;
-    R.rec_sumE2[k] = R.sumE2;
-  }
+  if (t < n) commit_step(runs[ids ? ids[t] : t]);
 }
 
 // ---------------------------------------------------------------------------
@@ -901,6 +974,11 @@ cudaError_t launch_init_finish(RunDev* runs, const int32_t* ids, int n, cudaStre
 cudaError_t launch_prepare(RunDev* runs, const int32_t* ids, int n, bool ovr, double beta, int theta,
                            int64_t Rt, cudaStream_t st) {
   k_prepare<<<n, PREP_THREADS, 0, st>>>(runs, ids, ovr ? 1 : 0, beta, theta, Rt);
+  return cudaGetLastError();
+}
+cudaError_t launch_resample(RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr, double beta,
+                            int theta, int64_t Rt, cudaStream_t st) {
+  k_resample<<<n, SMALL_THREADS, 0, st>>>(runs, ids, commit_first ? 1 : 0, ovr ? 1 : 0, beta, theta, Rt);
   return cudaGetLastError();
 }
 cudaError_t launch_copies(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {

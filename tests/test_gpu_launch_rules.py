@@ -116,3 +116,45 @@ def test_chosen_box_shape_bit_exact(Lx, Ly, Lz, mask, R0, gaussian):
     assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.energies().astype(np.int64), c.energies().astype(np.int64))
     assert np.array_equal(g.spins(), c.spins())
+
+
+# Populations resampled by one block (capacity up to 2048: passes of 1024
+# replicas) and by one block per 256 replicas; heavy replicas, a step that
+# changes nothing, and the state after a step that outgrows the capacity.
+@pytest.mark.parametrize("R0,cap", [(40, 400), (1024, 1500), (1025, 2048), (1600, 2048), (1600, 2049), (5121, 8000)])
+def test_resampling_paths_bit_exact(R0, cap):
+    J = inputs.couplings_3d(4, 3, 9)
+    g = pa.Run(J, 4, 3, R0, 43, R_cap=cap)
+    c = o.Run(J, 3, 4, 4, 4, 7, R0=R0, R_cap=cap, seed=43)
+    for beta in (0.2, 0.2, 1.6, 5.0):
+        Rprev = c.state().R
+        g.step(beta, 1)
+        c.step(beta, 1, R0)
+        assert np.array_equal(g.copies(Rprev), c.copies(Rprev)), beta
+        assert g.observables()["R"] == c.state().R, beta
+        assert np.array_equal(g.energies(), c.energies()), beta
+    assert np.array_equal(g.spins(), c.spins())
+    E = g.energies()
+    with pytest.raises(pa.PAError) as e:
+        g.step(5.1, 1, R_target=40 * cap)
+        g.sync()
+    assert e.value.code == pa.PA_ERR_CAPACITY
+    assert np.array_equal(pa.pa_copy_energies(g._h, cap), E)
+
+
+# A schedule of small runs commits a step at the start of the next: the same states as steps
+# committed one by one, with and without a graph.
+@pytest.mark.parametrize("gaussian,R0", [(False, 900), (False, 5000), (True, 900)])
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_schedule_commits_every_step(gaussian, R0, use_graph):
+    J = inputs.gaussian_couplings_3d(4, 3, 9) if gaussian else inputs.couplings_3d(4, 3, 9)
+    betas = np.array([0.1, 0.3, 0.3, 0.7])
+    a, b = (pa.Run(J, 4, 3, R0, 47, gaussian=gaussian) for _ in range(2))
+    a.run_schedule(betas, np.full(4, 2), use_graph=use_graph)
+    a.sync()
+    for beta in betas:
+        b.step(float(beta), 2)
+    assert a.observables() == b.observables()
+    ta, tb = a.trajectory(), b.trajectory()
+    assert all(np.array_equal(ta[k], tb[k]) for k in tb)
+    assert np.array_equal(a.spins(), b.spins())
