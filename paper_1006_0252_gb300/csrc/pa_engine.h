@@ -42,7 +42,9 @@ cudaError_t launch_weighted(int G, int M, const double* x, const double* A, cons
 cudaError_t launch_weighted_pairs(int G, int M, const double* x1, const double* x2, const double* A,
                                   const double* R1, const double* R2, double* mean, double* fbar, cudaStream_t st);
 cudaError_t launch_bootstrap(int M, const double* x, const double* A, const double* Rw, int B, uint64_t seed,
-                             double* bmean, double* bfbar, cudaStream_t st, int GK = 1);
+                             double* bmean, double* bfbar, double* tab, cudaStream_t st, int GK = 1);
+// Doubles of the weight tables of a bootstrap of GK groups of M runs.
+inline size_t boot_table_size(int M, int64_t GK) { return (size_t)GK * (3 * (size_t)M + 1); }
 bool sweep1d_split_ok(int split);
 cudaError_t launch_sweep1d(int tpb, int split, int rp, RunDev* runs, const Work* table, int nwork, int W, int WR,
                            cudaStream_t st, bool init, int min_smem);

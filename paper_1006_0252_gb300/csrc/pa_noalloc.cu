@@ -80,7 +80,8 @@ extern "C" int pa_bootstrap_noalloc(int M, const double* x_dev, const double* A_
   cudaStream_t st = (cudaStream_t)stream;
   // every one of the 2B scratch entries read below is written first by this
   // call, so nothing has to be cleared
-  if (pa::launch_bootstrap(M, x_dev, A_dev, R_dev, B, seed, scratch, scratch + PA_BOOTSTRAP_NOALLOC_MAX_B, st) !=
+  if (pa::launch_bootstrap(M, x_dev, A_dev, R_dev, B, seed, scratch, scratch + PA_BOOTSTRAP_NOALLOC_MAX_B, nullptr,
+                           st) !=
       cudaSuccess)
     return PA_ERR_CUDA;
   k_boot_std<<<1, 256, 0, st>>>(scratch, B, out_dev);

@@ -158,3 +158,20 @@ def test_schedule_commits_every_step(gaussian, R0, use_graph):
     ta, tb = a.trajectory(), b.trajectory()
     assert all(np.array_equal(ta[k], tb[k]) for k in tb)
     assert np.array_equal(a.spins(), b.spins())
+
+
+# Bootstrap with tabulated weights: one run, a lane's worth and more of them,
+# population factors and the observable given or not, and weights so far apart
+# that most resamples miss the runs that carry them (1e-200 of the largest).
+@pytest.mark.parametrize("M,B", [(1, 2), (2, 33), (33, 129), (200, 64)])
+@pytest.mark.parametrize("spread", [0.9, 3000.0])
+def test_bootstrap_weights(M, B, spread):
+    rng = np.random.default_rng(M)
+    x, A = rng.normal(2500.0, spread, M), rng.normal(-600.0, 4.0, M)
+    R = rng.integers(20000, 80000, M).astype(np.float64)
+    for args in ((x, A, R), (x, A, None), (x, None, R), (x, None, None)):
+        g, want = pa.pa_bootstrap(*args, B=B, seed=9), o.bootstrap(*args, B=B, seed=9)
+        # values of ~3e3 agree to a few units of 2^-53 a draw; their spread may
+        # cancel to zero where every resample is the same
+        for a, b in zip(g, want):
+            assert abs(a - b) <= 1e-9 * abs(b) + 1e-10, (M, B, spread, a, b)
