@@ -792,16 +792,39 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sum or maximum of v over a block of NT threads, in every thread; s_part: one
+// value a warp.
+template <int NT, bool MAX>
+__device__ __forceinline__ double block_fold(double v, double* s_part) {
+  v = MAX ? warp_max(v) : warp_sum(v);
+  if constexpr (NT > 32) {
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = s_part[0];
+#pragma unroll
+    for (int w = 1; w < NT / 32; ++w) v = MAX ? fmax(v, s_part[w]) : v + s_part[w];
+    __syncthreads();  // s_part may be written again
+  }
+  return v;
+}
+
 // PAIRS: Sec. 4, Eq. (11) -- an observable of two independent runs
 // (the overlap) is averaged over M pairs with weights e^{-beta (F~1 + F~2)}
 // (R1 R2 e^{...} with the population factors of Eq. (6)), and fbar is
 // ln[(1/M) sum_r e^{x1_r + x2_r}].  Otherwise x2 and Rw2 are unused.
-template <bool PAIRS>
-__global__ void __launch_bounds__(32) k_weighted(int M, const double* __restrict__ x, const double* __restrict__ x2,
+//
+// One block of NT threads per group.  A logarithm or an exponential is some 25
+// dependent FP64 instructions of 64 cycles, so a lone group is bound by how
+// many of them a thread does in turn: M = 200 takes 52 us (pairs) and 33 with a
+// warp, 16 and 14 with 256 threads, which keep their first value instead of
+// computing it again.
+template <bool PAIRS, int NT>
+__global__ void __launch_bounds__(NT) k_weighted(int M, const double* __restrict__ x, const double* __restrict__ x2,
                                                  const double* __restrict__ A, const double* __restrict__ Rw,
                                                  const double* __restrict__ Rw2, double* __restrict__ mean,
                                                  double* __restrict__ fbar) {
-  const int g = blockIdx.x, lane = threadIdx.x;
+  __shared__ double s_part[NT / 32];
+  const int g = blockIdx.x, t = threadIdx.x;
   const double* xg = x + (int64_t)g * M;
   const double* x2g = PAIRS ? x2 + (int64_t)g * M : nullptr;
   const double* Ag = A ? A + (int64_t)g * M : nullptr;
@@ -814,49 +837,56 @@ __global__ void __launch_bounds__(32) k_weighted(int M, const double* __restrict
     if (PAIRS && R2g) y = y + log(R2g[r]);
     return y;
   };
-  double mu = -INFINITY, mux = -INFINITY;
-  for (int r = lane; r < M; r += 32) {
-    mu = fmax(mu, yr(r));
+  double mu = -INFINITY, mux = -INFINITY, y0 = 0.0;
+  for (int r = t; r < M; r += NT) {
+    const double y = yr(r);
+    if (r == t) y0 = y;
+    mu = fmax(mu, y);
     mux = fmax(mux, xr(r));
   }
-  mu = warp_max(mu);
-  mux = warp_max(mux);
+  mu = block_fold<NT, true>(mu, s_part);
+  mux = block_fold<NT, true>(mux, s_part);
   double S = 0.0, SA = 0.0, Sx = 0.0;
-  for (int r = lane; r < M; r += 32) {
-    const double e = exp(yr(r) - mu);
+  for (int r = t; r < M; r += NT) {
+    const double e = exp((r == t ? y0 : yr(r)) - mu);
     S += e;
     if (Ag) SA += e * Ag[r];
     Sx += exp(xr(r) - mux);
   }
-  S = warp_sum(S);
-  SA = warp_sum(SA);
-  Sx = warp_sum(Sx);
-  if (lane == 0) {
+  S = block_fold<NT, false>(S, s_part);
+  SA = block_fold<NT, false>(SA, s_part);
+  Sx = block_fold<NT, false>(Sx, s_part);
+  if (t == 0) {
     mean[g] = Ag ? SA / S : 0.0;
     fbar[g] = mux + log(Sx) - log((double)M);
   }
 }
 
-// Weights of the runs of each group for k_bootstrap, one warp per group: with y
+// Weights of the runs of each group for k_bootstrap, one block per group: with y
 // = x + ln R, tab[gk] = {e^{y_k - max y}, e^{y_k - max y} A_k, e^{x_k - max x}} for
 // the M runs, then max x.  HAS_A, HAS_R: whether A and Rw are given.
+constexpr int BOOT_WEIGHT_THREADS = 256;  // M = 200, one group: 24 us with a warp, 9 so
 template <bool HAS_A, bool HAS_R>
-__global__ void __launch_bounds__(32) k_boot_weights(int M, const double* __restrict__ x, const double* __restrict__ A,
-                                                     const double* __restrict__ Rw, double* __restrict__ tab) {
-  const int gk = blockIdx.x, lane = threadIdx.x;
+__global__ void __launch_bounds__(BOOT_WEIGHT_THREADS) k_boot_weights(int M, const double* __restrict__ x,
+                                                                      const double* __restrict__ A,
+                                                                      const double* __restrict__ Rw,
+                                                                      double* __restrict__ tab) {
+  constexpr int NT = BOOT_WEIGHT_THREADS;
+  __shared__ double s_part[NT / 32];
+  const int gk = blockIdx.x, first = threadIdx.x;
   const double* xg = x + (int64_t)gk * M;
   double* t = tab + (int64_t)gk * (3 * (int64_t)M + 1);
   double mu = -INFINITY, mux = -INFINITY;
-  for (int k = lane; k < M; k += 32) {
+  for (int k = first; k < M; k += NT) {
     double y = xg[k];
     if constexpr (HAS_R) y += log(Rw[(int64_t)gk * M + k]);
     t[k] = y;
     mu = fmax(mu, y);
     mux = fmax(mux, xg[k]);
   }
-  mu = warp_max(mu);
-  mux = warp_max(mux);
-  for (int k = lane; k < M; k += 32) {  // the lane's own y
+  mu = block_fold<NT, true>(mu, s_part);
+  mux = block_fold<NT, true>(mux, s_part);
+  for (int k = first; k < M; k += NT) {  // the thread's own y
     const double e = exp(t[k] - mu);
     t[k] = e;
     if constexpr (HAS_A) t[(int64_t)M + k] = e * A[(int64_t)gk * M + k];
@@ -864,40 +894,50 @@ __global__ void __launch_bounds__(32) k_boot_weights(int M, const double* __rest
     if constexpr (HAS_R) t[2 * (int64_t)M + k] = exp(xg[k] - mux);
     else t[2 * (int64_t)M + k] = e;  // without population factors y = x
   }
-  if (lane == 0) t[3 * (int64_t)M] = mux;
+  if (first == 0) t[3 * (int64_t)M] = mux;
 }
 
 // Sec. 3 bootstrap: resample b draws index floor(word0 * M / 2^32) of
-// Philox(ctr = (b, i, 0, TAG_BOOT)); one thread per resample.  GK groups of M
-// values each (x, A, Rw laid out [GK][M]) are resampled with the same draws;
+// Philox(ctr = (b, i, 0, TAG_BOOT)); LANES threads per resample take its draws
+// in turn.  GK groups of M values each (x, A, Rw laid out [GK][M]) are resampled with the same draws;
 // the results are laid out [GK][B].
 //
 // tab: the weights of k_boot_weights (nullptr: none).  With them a draw is its
 // generator call, three loads and three FP64 additions; without, two
 // exponentials and two logarithms, some 25 FP64 instructions of 64 cycles each
-// (M = 200, B = 1000: 785 us, with tables 46 and 22 for the weights).  A
+// (M = 200, B = 1000: 785 us with one thread a resample, 46 with tables, 11
+// with eight threads, which spread 1000 resamples over more than 8 SMs).  A
 // resample that misses the runs that carry the weight (all of its weights below
-// 1e-200 of the largest) is summed against its own largest value all the same.
+// 1e-200 of the largest) is summed by its first thread against its own largest
+// value all the same.
+template <int LANES>
 __global__ void k_bootstrap(int M, const double* __restrict__ x, const double* __restrict__ A,
                             const double* __restrict__ Rw, const double* __restrict__ tab, int B, uint64_t seed,
                             int GK, double* __restrict__ bmean, double* __restrict__ bfbar) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
+  const int at = (blockIdx.x * blockDim.x + threadIdx.x) / LANES, lane = threadIdx.x % LANES;
+  const int b = min(at, B - 1);  // the threads past the last resample draw it again and write nothing
   for (int gk = blockIdx.y; gk < GK; gk += gridDim.y) {
     double S = 0.0, SA = 0.0, Sx = 0.0, mux = -INFINITY;
     bool direct = true;
     if (tab) {
       const double* t = tab + (int64_t)gk * (3 * (int64_t)M + 1);
-      for (int i = 0; i < M; ++i) {
+      for (int i = lane; i < M; i += LANES) {
         const u32x4 r = philox_seeded(seed, (uint32_t)b, (uint32_t)i, 0u, TAG_BOOT);
         const int k = (int)(((uint64_t)r.a * (uint64_t)M) >> 32);
         S += t[k];
         SA += t[(int64_t)M + k];
         Sx += t[2 * (int64_t)M + k];
       }
+#pragma unroll
+      for (int sh = LANES / 2; sh >= 1; sh >>= 1) {
+        S += __shfl_xor_sync(0xFFFFFFFFu, S, sh);
+        SA += __shfl_xor_sync(0xFFFFFFFFu, SA, sh);
+        Sx += __shfl_xor_sync(0xFFFFFFFFu, Sx, sh);
+      }
       mux = t[3 * (int64_t)M];
       direct = S < 1e-200 || Sx < 1e-200;
     }
+    if (lane != 0 || at >= B) continue;
     if (direct) {
       const double* xg = x + (int64_t)gk * M;
       const double* Ag = A ? A + (int64_t)gk * M : nullptr;
@@ -1107,28 +1147,39 @@ cudaError_t launch_variance(int G, int M, const double* x, double* var, cudaStre
   return cudaGetLastError();
 }
 
+// A block of 256 threads a group where the groups leave SMs idle, a warp a
+// group else (and where a warp holds the group).
+template <bool PAIRS>
+static cudaError_t launch_weighted_t(int G, int M, const double* x1, const double* x2, const double* A,
+                                     const double* R1, const double* R2, double* mean, double* fbar, cudaStream_t st) {
+  if (M > 32 && G <= 608) k_weighted<PAIRS, 256><<<G, 256, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
+  else k_weighted<PAIRS, 32><<<G, 32, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
+  return cudaGetLastError();
+}
 cudaError_t launch_weighted(int G, int M, const double* x, const double* A, const double* Rw, double* mean,
                             double* fbar, cudaStream_t st) {
-  k_weighted<false><<<G, 32, 0, st>>>(M, x, nullptr, A, Rw, nullptr, mean, fbar);
-  return cudaGetLastError();
+  return launch_weighted_t<false>(G, M, x, nullptr, A, Rw, nullptr, mean, fbar, st);
 }
 cudaError_t launch_weighted_pairs(int G, int M, const double* x1, const double* x2, const double* A,
                                   const double* R1, const double* R2, double* mean, double* fbar, cudaStream_t st) {
-  k_weighted<true><<<G, 32, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
-  return cudaGetLastError();
+  return launch_weighted_t<true>(G, M, x1, x2, A, R1, R2, mean, fbar, st);
 }
 cudaError_t launch_bootstrap(int M, const double* x, const double* A, const double* Rw, int B, uint64_t seed,
                              double* bmean, double* bfbar, double* tab, cudaStream_t st, int GK) {
-  if (tab) {
-    if (A && Rw) k_boot_weights<true, true><<<GK, 32, 0, st>>>(M, x, A, Rw, tab);
-    else if (A) k_boot_weights<true, false><<<GK, 32, 0, st>>>(M, x, A, Rw, tab);
-    else if (Rw) k_boot_weights<false, true><<<GK, 32, 0, st>>>(M, x, A, Rw, tab);
-    else k_boot_weights<false, false><<<GK, 32, 0, st>>>(M, x, A, Rw, tab);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+  const unsigned groups = (unsigned)std::min(GK, 65535);
+  if (!tab) {
+    k_bootstrap<1><<<dim3((B + 127) / 128, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
+    return cudaGetLastError();
   }
-  const dim3 grid((B + 127) / 128, (unsigned)std::min(GK, 65535));
-  k_bootstrap<<<grid, 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
+  if (A && Rw) k_boot_weights<true, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+  else if (A) k_boot_weights<true, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+  else if (Rw) k_boot_weights<false, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+  else k_boot_weights<false, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  constexpr int LANES = 8, PER_BLOCK = 128 / LANES;
+  k_bootstrap<LANES><<<dim3((B + PER_BLOCK - 1) / PER_BLOCK, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK,
+                                                                                    bmean, bfbar);
   return cudaGetLastError();
 }
 

@@ -175,3 +175,17 @@ def test_bootstrap_weights(M, B, spread):
         # cancel to zero where every resample is the same
         for a, b in zip(g, want):
             assert abs(a - b) <= 1e-9 * abs(b) + 1e-10, (M, B, spread, a, b)
+
+
+# Weighted averages by a warp (up to 32 runs) and by a block of 256 threads.
+@pytest.mark.parametrize("M", [32, 33, 256, 257, 1000])
+def test_weighted_average_sizes(M):
+    rng = np.random.default_rng(M)
+    x, x2, A = rng.normal(2500.0, 0.9, M), rng.normal(2500.0, 0.9, M), rng.normal(-600.0, 4.0, M)
+    R = rng.integers(20000, 80000, M).astype(np.float64)
+    for Rw in (R, None):
+        # sums of M terms in FP64, relative to their own size: 1e-12
+        for got, want in ((pa.pa_weighted_average(x, A, Rw), o.weighted_average(x, A, Rw)),
+                          (pa.pa_weighted_average_pairs(x, x2, A, Rw, Rw),
+                           o.weighted_average(x + x2, A, None if Rw is None else Rw * Rw))):
+            assert all(abs(a - b) <= 1e-12 * abs(b) for a, b in zip(got, want)), (M, got, want)
