@@ -939,10 +939,12 @@ int engine_init_population(Engine& E) {
 
 int engine_fetch(Engine& E, std::vector<RunDev>& out) {
   PA_CUDA(cudaSetDevice(E.device));
+  out.resize(E.n);
+  // on the engine's own stream: one wait, where a synchronisation and a copy
+  // on the default stream were two
+  PA_CUDA(cudaMemcpyAsync(out.data(), E.d_runs, sizeof(RunDev) * E.n, cudaMemcpyDeviceToHost, E.st));
   PA_CUDA(cudaStreamSynchronize(E.st));
   E.harvest_graph_timing();
-  out.resize(E.n);
-  PA_CUDA(cudaMemcpy(out.data(), E.d_runs, sizeof(RunDev) * E.n, cudaMemcpyDeviceToHost));
   return PA_OK;
 }
 
