@@ -4,7 +4,7 @@
 // reads and writes it there, so a whole schedule runs without host round
 // trips (and can be captured in one CUDA graph).
 #pragma once
-#include <cuda_runtime_api.h>
+#include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace pa {
@@ -128,6 +128,27 @@ struct Sweep3dLaunch {
   int min_smem;
   cudaStream_t st;
 };
+
+// Launch of a kernel that begins with cudaGridDependencySynchronize(): its
+// blocks may take their place on the SMs before the kernel ahead of it in the
+// stream has finished (where that one triggers, as soon as all of its blocks
+// have begun), and wait there for its end.  The two kernels of a step of a small
+// run (1000 replicas, L = 4): 24.2 -> 23.4 us a step.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t st,
+                                    A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
 
 // Gaussian threshold-table kernel (pa_gauss3d_tab.cuh): the finest split of an
 // edge (whole rows, pairs of them where a row's uniforms end within a generator

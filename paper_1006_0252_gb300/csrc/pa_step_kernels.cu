@@ -602,6 +602,8 @@ __global__ void __launch_bounds__(SMALL_THREADS) k_resample(RunDev* __restrict__
   __shared__ unsigned long long s_cnt[NT];
   __shared__ int32_t s_bin[NT];
   RunDev& R = runs[ids ? ids[blockIdx.x] : blockIdx.x];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   if (commit_first) {
     if (threadIdx.x == 0) commit_step(R);
     __syncthreads();
@@ -1072,8 +1074,8 @@ cudaError_t launch_prepare(RunDev* runs, const int32_t* ids, int n, bool ovr, do
 }
 cudaError_t launch_resample(RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr, double beta,
                             int theta, int64_t Rt, cudaStream_t st) {
-  k_resample<<<n, SMALL_THREADS, 0, st>>>(runs, ids, commit_first ? 1 : 0, ovr ? 1 : 0, beta, theta, Rt);
-  return cudaGetLastError();
+  return launch_dependent(k_resample, n, SMALL_THREADS, (size_t)0, st, runs, ids, commit_first ? 1 : 0, ovr ? 1 : 0,
+                          beta, theta, Rt);
 }
 cudaError_t launch_copies(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
   k_copies<<<nwork, CHUNK, 0, st>>>(runs, table);

@@ -271,6 +271,8 @@ __global__ void __launch_bounds__(TPB) k_sweep3d(RunDev* __restrict__ runs, cons
   uint4* s_bond = reinterpret_cast<uint4*>(smem + SH::TAB_WORDS);
   ColourWord<RP>* s_spin = reinterpret_cast<ColourWord<RP>*>(smem + SH::TAB_WORDS + SH::BOND_WORDS);  // [2][WR][CS]
   const Work wk = table[blockIdx.x / SH::BPI];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   RunDev& R = runs[wk.run];
   if (R.skip) return;
   const int64_t Rn = R.R_next;
@@ -490,8 +492,7 @@ cudaError_t sweep3d_p(const Sweep3dLaunch& a) {
       return cudaFuncSetAttribute((const void*)k_sweep3d<L, TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   sm);
     }
-    k_sweep3d<L, TPB, P, RP><<<a.nwork * SH::BPI, TPB, sm, a.st>>>(a.runs, a.table);
-    return cudaGetLastError();
+    return launch_dependent(k_sweep3d<L, TPB, P, RP>, a.nwork * SH::BPI, TPB, (size_t)sm, a.st, a.runs, a.table);
   }
 }
 
