@@ -163,6 +163,7 @@ struct LatticeClass {
   std::vector<int32_t> runs;
   Work* d_table = nullptr;
   int nwork = 0;
+  double sites = 0.0;  // spins of all its replicas
   int item = 0;      // slots of a work item where they are chosen by the populations (spread_blocks), else 0
   // Slots of a work item: the block's threads where a power of two of them
   // shares a replica (split / rp blocks an item), else the block's replicas.
@@ -172,6 +173,17 @@ struct LatticeClass {
 // One launch shape of a class.
 struct LaunchShape {
   int tpb, split, rp;
+};
+
+// Streams on which the classes of a step are swept side by side: the blocks of
+// one class fill the SMs that the last blocks of another leave idle.
+struct ClassFan {
+  static constexpr size_t MOST = 8;  // classes at once
+  std::vector<cudaStream_t> st;
+  std::vector<cudaEvent_t> done;
+  cudaEvent_t fork = nullptr;
+  int ensure(size_t n);
+  void release();
 };
 
 struct Engine {
@@ -187,6 +199,7 @@ struct Engine {
   std::vector<int64_t> R0;
   RunDev* d_runs = nullptr;
   std::vector<LatticeClass> cls;
+  ClassFan fan;
   Work* d_copy_table = nullptr;
   int n_copy_work = 0;
   int max_bins = 0;
@@ -269,6 +282,7 @@ struct Engine {
     }
     prof_ev.clear();
     drop_graph();
+    fan.release();
     for (auto& s : slabs) {
       if (ff) ff(s.p, s.n, (void*)st, actx);
       else cudaFreeAsync(s.p, st);
@@ -301,6 +315,7 @@ std::vector<LaunchShape> launch_shapes(const LatticeClass& c);
 bool split_supported(const LatticeClass& c, int split);
 bool tpb_supported(const LatticeClass& c, int tpb);
 int launch_class_on(RunDev* runs, cudaStream_t st, const LatticeClass& c, const Work* table, int nwork, bool init);
+int launch_classes(RunDev* runs, cudaStream_t st, const std::vector<LatticeClass>& cls, ClassFan& fan, bool graph);
 int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork, bool init);
 int prepare_class_launch(RunDev* runs, cudaStream_t st, const LatticeClass& c);
 int build_class_table(Engine& E, LatticeClass& c);

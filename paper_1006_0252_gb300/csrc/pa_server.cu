@@ -60,6 +60,7 @@ struct pa_server {
   DevBuf ids_buf, copy_buf, init_ids_buf;
   int n_copy = 0;
   std::vector<LatticeClass> cls;
+  ClassFan fan;
   std::vector<DevBuf> cls_buf, init_buf;
   std::chrono::steady_clock::time_point t0;
 
@@ -227,6 +228,7 @@ void pa_server_destroy(pa_server* S) {
   if (!S) return;
   cudaSetDevice(S->device);
   cudaStreamSynchronize(S->st);
+  S->fan.release();
   for (int sl = 0; sl < S->max_runs; ++sl) S->dfree(S->slot_mem[sl].p, S->slot_mem[sl].n);
   S->dfree(S->ids_buf.p, S->ids_buf.n);
   S->dfree(S->copy_buf.p, S->copy_buf.n);
@@ -341,11 +343,8 @@ int pa_server_tick(pa_server* S, int steps, int32_t* n_active, int32_t* n_queued
     PA_CUDA(launch_copies(S->d_runs, (const Work*)S->copy_buf.p, S->n_copy, S->st));
     PA_CUDA(launch_scan(S->d_runs, ids, na, S->st));
     PA_CUDA(launch_scatter(S->d_runs, (const Work*)S->copy_buf.p, S->n_copy, S->st));
-    for (auto& c : S->cls) {
-      if (c.nwork == 0) continue;
-      st = launch_class_on(S->d_runs, S->st, c, c.d_table, c.nwork, false);
-      if (st != PA_OK) return st;
-    }
+    st = launch_classes(S->d_runs, S->st, S->cls, S->fan, false);
+    if (st != PA_OK) return st;
     PA_CUDA(launch_commit(S->d_runs, ids, na, S->st));
   }
   // 3. retire finished (or failed) runs

@@ -189,3 +189,22 @@ def test_weighted_average_sizes(M):
                           (pa.pa_weighted_average_pairs(x, x2, A, Rw, Rw),
                            o.weighted_average(x + x2, A, None if Rw is None else Rw * Rw))):
             assert all(abs(a - b) <= 1e-12 * abs(b) for a, b in zip(got, want)), (M, got, want)
+
+
+# Classes swept side by side, in a graph and (from 2^20 spins outside the
+# largest class) launch by launch: every run ends as it does alone.
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_classes_side_by_side(use_graph):
+    betas = np.array([0.2, 0.5, 0.9])
+    sizes = [(8, 3001), (6, 6001), (8, 2999), (4, 3000)]
+    specs = [inputs.RunSpec(3, L, 0, 50 + i, R0, betas, 2) for i, (L, R0) in enumerate(sizes)]
+    b = pa.Batch(specs)
+    b.run(betas, thetas=2, use_graph=use_graph)
+    assert not b.sync().any()
+    res = b.results()
+    for r, (L, R0) in enumerate(sizes):
+        g = pa.Run(specs[r].couplings(), L, 3, R0, 50 + r)
+        g.run_schedule(betas, np.full(3, 2))
+        ob = g.observables()
+        assert res["R"][r] == ob["R"] and res["sumE"][r] == ob["sumE"] and res["sumE2"][r] == ob["sumE2"], r
+        assert np.array_equal(b.spins(r, ob["R"]), g.spins()), r
