@@ -45,13 +45,13 @@ TIME_EVERY = 8  # sweep launches timed with CUDA events: every 8th
 # DRAM bytes (read + write) per sweep launch from one ncu capture of this
 # kernel source (dram__bytes_read.sum + dram__bytes_write.sum); reported only
 # while the kernel source is the one that was captured.
-SWEEP_TRAFFIC = {"sha256_16": "e6c85eeaf62e4f52", "bytes": 5563477}
+SWEEP_TRAFFIC = {"sha256_16": "7c50a8d87ed4f3e4", "bytes": 4337920}
 
 
 def sweep_traffic():
     import hashlib
     h = hashlib.sha256()
-    for f in ("pa_sweep3d.cuh", "pa_lattice3d.cuh"):
+    for f in ("pa_sweep3d.cuh", "pa_colour3d.cuh", "pa_lattice3d.cuh"):
         with open(os.path.join(ROOT, "paper_1006_0252_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return SWEEP_TRAFFIC["bytes"] if h.hexdigest()[:16] == SWEEP_TRAFFIC["sha256_16"] else None

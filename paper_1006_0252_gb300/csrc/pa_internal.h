@@ -115,7 +115,7 @@ struct Work {
   int32_t first;
 };
 
-// A launch of the +-1 cubic sweep kernel: tpb threads per block, split of them
+// A launch of a cubic sweep kernel: tpb threads per block, split of them
 // sharing the rp replicas of a column; nwork work items (nwork <= 0 only
 // prepares the kernel for launches); at least min_smem bytes of shared memory
 // a block.
