@@ -9,8 +9,9 @@
 // site and pattern 2^32 - t, where the site flips iff its uniform u < t (t =
 // 2^32 for dE <= 0, whose entry is 0): adding the uniform carries exactly when
 // it rejects, as in the Gaussian cubic kernel (pa_gauss3d_tab.cuh).  t = 0 has
-// no entry; it takes that of t = 1, and in a block with such an entry the
-// uniforms that are 0 are decided again (reject_zero).
+// no entry; it takes that of t = 1.  So every thread keeps the minimum of its
+// uniforms of a half sweep, and in a block with such an entry a minimum of 0
+// sends it to decide_zeros.
 //
 // Words are split by colour as in pa_colour3d.cuh, with the geometry known only
 // at run time: the S = k Lx / 2 colour-c sites of a word by rank m = j Lx/2 +
@@ -23,15 +24,18 @@
 //
 // P threads (lanes of one warp) share a column of replicas on ranges of words.
 //
-// What bounds it: instruction issue at full blocks (19 instructions a flip at
-// four sites a word), in small populations the 15-20 us of tables, gather and
-// energies.  One launch, theta = 10, us at beta = 0.5, site at a time (pa_box.cu,
-// every box before) -> this kernel:
-//   8 x 6 x 5, +-1       20000 replicas 832 -> 109     1000 775 -> 29
-//   8 x 6 x 5, Gaussian  20000          903 -> 109
-//   6 x 8 x 8, +-1       30000         1311 -> 164
-//   8 x 8 x 8, Gaussian  10000         1765 -> 84      (open z)
+// What bounds it: instruction issue at full blocks (27 instructions a flip at
+// four sites a word: the generator 8.5, the walk and the patterns of a word shared
+// by 16 flips), in small populations the 15-20 us of tables, gather and energies.
+// One launch, theta = 10, us at beta = 0.5, site at a time (pa_box.cu, every box
+// before) -> this kernel:
+//   8 x 6 x 5, +-1       20000 replicas 832 -> 82      1000 775 -> 31
+//   8 x 6 x 5, Gaussian  20000          903 -> 82
+//   6 x 8 x 8, +-1       30000         1311 -> 130
+//   8 x 8 x 8, Gaussian  10000         1765 -> 70      (open z)
 //   6 x 6 x 7, Gaussian   3000          955 -> 64
+// (Uniforms of 0 looked for site by site under a flag took 46 instructions and
+// 109 us of the first: predicated off, they are issued all the same.)
 #pragma once
 #include "pa_gauss.cuh"
 #include "pa_lattice3d.cuh"
@@ -110,18 +114,37 @@ __device__ __forceinline__ void box_anti(const int32_t* __restrict__ gJ, int pla
   a[3] = acc + j0 + j1;
 }
 
-// Whether the site at bit b of the pattern words rejects the uniform 0: a rise
-// of threshold 0.
-static __device__ __noinline__ bool reject_zero(const RunDev& R, int plane, int site, int odd, uint32_t pattern,
-                                                float beta_f) {
-  const int c = site >= plane, at = site - c * plane;
-  const int32_t* gJ = R.gJ + (size_t)c * 6 * plane + at;
-  int32_t acc = 0;
-  for (int bit = 0; bit < 6; ++bit)
-    if ((pattern >> bit) & 1u) acc += gJ[(bit < 2 ? bit ^ odd : bit) * plane];
-  const int32_t dE = 4 * acc - 2 * R.gS[site];
-  if (dE <= 0) return false;
-  return (R.model == 1 ? gauss_threshold(dE, beta_f) : R.thr[dE >> 1]) == 0u;
+// Words w0 .. w1-1 of a column after a colour-c half sweep at sweep T: sites whose
+// uniform was 0 were flipped (no entry makes 0 carry), and those that rise with
+// threshold 0 go back.  Their neighbours have the other colour and are as they
+// were.  Slow: a uniform is 0 once in 2^32 draws.  (Inline: a call here would
+// cost registers in the sweep, 5 us of 34 in a launch of 1000 replicas.)
+__device__ __forceinline__ void decide_zeros(const RunDev& R, uint32_t* own, const uint32_t* oth, int CS, int S,
+                                             int field, int c, int w0, int w1, int reps, int64_t slot, int ncol,
+                                             uint32_t T, float beta_f) {
+  const int plane = R.Wr * S, H = R.bx / 2;
+#pragma unroll 1
+  for (int w = w0; w < w1; ++w)
+#pragma unroll 1
+    for (int m = 0; m < S; ++m)
+#pragma unroll 1
+      for (int k = 0; k < reps; ++k) {
+        const int at = w * S + m;
+        const uint32_t call = (uint32_t)at >> 2, s_k = (uint32_t)(slot + (int64_t)k * ncol);
+        if (pick(philox_seeded(R.seed, call, s_k, T, TAG_SWEEP + (uint32_t)c), at & 3) != 0u) continue;
+        const uint32_t bit = 1u << (field * k + m);
+        const uint32_t s = (own[w * CS] & bit) ? 0u : 1u;  // before the flip
+        int32_t acc = 0;
+        for (int d = 0; d < 6; ++d) {
+          const int32_t J = R.gJ[(c * 6 + d) * plane + at];
+          if (J == 0) continue;
+          const int code = R.box_code[(c * 7 + 1 + d) * plane + at], p = code & 31;  // the neighbour's packed place
+          const int rank = p / R.bx * H + p % R.bx / 2;
+          if (((oth[(code >> 5) * CS] >> (field * k + rank)) & 1u) != s) acc += J;
+        }
+        const int32_t dE = 4 * acc - 2 * R.gS[c * plane + at];
+        if (dE > 0 && (R.model == 1 ? gauss_threshold(dE, beta_f) : R.thr[dE >> 1]) == 0u) own[w * CS] ^= bit;
+      }
 }
 
 // Sec. 2: gather of the resampled population, theta checkerboard sweeps at
@@ -240,6 +263,7 @@ __global__ void __launch_bounds__(BOX_TPB) k_sweep_boxtab(RunDev* __restrict__ r
       }
       uint32_t* own = col + c * WR * CS;
       const uint32_t* oth = col + (1 - c) * WR * CS;
+      uint32_t low = ~0u;  // the minimum of the half sweep's uniforms
       uint32_t carry[RP][4];
 #pragma unroll
       for (int k = 0; k < RP; ++k) carry[k][0] = carry[k][1] = carry[k][2] = carry[k][3] = 0u;
@@ -260,7 +284,7 @@ __global__ void __launch_bounds__(BOX_TPB) k_sweep_boxtab(RunDev* __restrict__ r
 #pragma unroll
             for (int k = 0; k < RP; ++k) {
               if (k >= reps) break;
-              uint32_t ge = 0u, zeros = 0u;
+              uint32_t ge = 0u;
               uint32_t held[4];
 #pragma unroll
               for (int i = 0; i < 4; ++i) held[i] = carry[k][i];
@@ -283,26 +307,16 @@ __global__ void __launch_bounds__(BOX_TPB) k_sweep_boxtab(RunDev* __restrict__ r
                     for (int i = 0; i < 4; ++i) carry[k][i] = u[i];
                   }
                 }
+                low = __vimin3_u32(__vimin3_u32(low, u[0], u[1]), u[2], u[3]);
                 static_for<0, 4>([&](auto jc) {
                   constexpr int i = 3 - decltype(jc)::value, m = 4 * q + i - A;
                   if constexpr (m >= 0 && m < S) {
                     const int b = T * k + m;
                     const uint32_t addr = __byte_perm(pat.f[b & 7], base, (uint32_t)(b >> 3) | 0x7650u);
                     ge = shift_in_carry(ge, u[i], load_shared<m * 256>(addr));
-                    if (never) zeros |= (u[i] == 0u ? 1u : 0u) << m;
                   }
                 });
               });
-              if (zeros != 0u) {
-                for (uint32_t rest = zeros; rest != 0u; rest &= rest - 1u) {
-                  const int m = __ffs((int)rest) - 1, b = T * k + m;
-                  uint32_t p = 0u;
-                  for (int d = 0; d < 6; ++d) p |= ((x[d] >> b) & 1u) << d;
-                  const int odd = (int)(bw.odd_x(c, y, g) >> b) & 1;
-                  const bool rej = reject_zero(R, plane, c * plane + w * S + m, odd, p, beta_f);
-                  ge = (ge & ~(1u << m)) | (rej ? 1u << m : 0u);
-                }
-              }
               stay &= ~(((~ge) & ((1u << S) - 1u)) << (T * k));
             }
             own[w * CS] = s ^ (B::ALL & ~stay);
@@ -313,6 +327,8 @@ __global__ void __launch_bounds__(BOX_TPB) k_sweep_boxtab(RunDev* __restrict__ r
           }
         });
       }
+      if (never && low == 0u)
+        decide_zeros(R, own, oth, CS, S, T, c, w0, w1, reps, first + r, ncol, T0 + (uint32_t)((h0 + j) >> 1), beta_f);
       __syncwarp();  // the next half sweep reads what the other threads of the column wrote
     }
   }

@@ -449,8 +449,8 @@ static int box_most(const LatticeClass& c, int P, int reps) {
 // thread of that kernel: the finest split that keeps the even share of an SM's
 // replicas in one block, as many replicas a word as it holds, fewer where that
 // would leave the block fewer than eight warps.  8 x 6 x 5, 20000 replicas, us a
-// launch for (split, replicas): (16, 4) 109, (32, 4) 120, (8, 4) 134, (16, 2)
-// 137, (16, 1) 169; 1000 replicas (32, 2) 29, (16, 1) 31, (16, 4) 47; 6 x 6 x 7,
+// launch for (split, replicas), while uniforms of 0 were looked for site by site:
+// (16, 4) 109, (32, 4) 120, (8, 4) 134, (16, 2) 137, (16, 1) 169; 1000 replicas (32, 2) 29, (16, 1) 31, (16, 4) 47; 6 x 6 x 7,
 // 3000 replicas (16, 1) 64, (16, 2) 70, (8, 1) 87, (16, 4) 110.
 static bool set_box_table(LatticeClass& c, int64_t replicas) {
   const int U = box_period(c.bsites), groups = (c.Wr + U - 1) / U;

@@ -29,13 +29,13 @@
 // (pa_sweep1d.cu), with two compares a site where that one needs one.  One
 // launch, us, with packed words, one thread a replica and a threshold looked up
 // per site and pattern -> now:
-//   N = 256, theta = 50   2e5 replicas 1961 -> 1675   20000 413 -> 220   1000 301 -> 57
-//   N = 512, theta = 10   5e4 258 -> 193
+//   N = 256, theta = 50   2e5 replicas 1961 -> 1584   20000 413 -> 210   1000 301 -> 55
+//   N = 512, theta = 10   5e4 258 -> 182
 //   N = 64,  theta = 10   1e5 102 -> 61
-//   N = 4096, theta = 10  5000 1050 -> 290
-// (2e5: (threads a block, split, replicas a thread) = (128, 8, 2) 1675,
-// (128, 4, 2) 1639, (128, 2, 2) 1705, (64, 1, 1) 1882; smaller populations
-// want the finest split.)
+//   N = 4096, theta = 10  5000 1050 -> 283
+// (2e5, with the maxima for thresholds of 0 still in the loop: (threads a block,
+// split, replicas a thread) = (128, 8, 2) 1675, (128, 4, 2) 1639, (128, 2, 2)
+// 1705, (64, 1, 1) 1882; smaller populations want the finest split.)
 #include "pa_gauss.cuh"
 #include "pa_lattice3d.cuh"
 #include "pa_patterns.cuh"
@@ -141,12 +141,14 @@ __device__ __forceinline__ GchainWord gchain_word(const T* __restrict__ own, con
 // own[w CS], the other colour's at oth[w CS]).  The uniforms of word w are
 // calls 4w .. 4w+3 of the colour; the calls are taken from the last, so that
 // the outcomes are shifted in from the highest rank.
-template <int C, int RP>
+// NEVER: the table has a threshold 0 (a parameter: predicated off, the maxima
+// would still take an issue slot a site).
+template <int C, int RP, bool NEVER>
 __device__ __forceinline__ void half_sweep_gauss1d(ColourWord<RP>* __restrict__ own,
                                                    const ColourWord<RP>* __restrict__ oth, int CS,
                                                    const uint4* __restrict__ thr, int WR, int last, int w0, int w1,
                                                    const uint4* __restrict__ half, const SweepKey (&key)[RP],
-                                                   const RoundKeys& rk, bool never) {
+                                                   const RoundKeys& rk) {
 #pragma unroll 1
   for (int w = w0; w < w1; ++w) {
     const GchainWord g = gchain_word<C>(own, oth, CS, w, WR, last);
@@ -158,7 +160,7 @@ __device__ __forceinline__ void half_sweep_gauss1d(ColourWord<RP>* __restrict__ 
 #pragma unroll
       for (int k = 0; k < RP; ++k) {
         u32x4 v = philox_sweep(half[GCHAIN_CALLS * w + q], key[k], rk);
-        if (never) v = {max(v.a, 1u), max(v.b, 1u), max(v.c, 1u), max(v.d, 1u)};
+        if constexpr (NEVER) v = {max(v.a, 1u), max(v.b, 1u), max(v.c, 1u), max(v.d, 1u)};
         ga[k] = shift_in_carry(ga[k], v.d, a.w);
         gb[k] = shift_in_carry(gb[k], v.d, b.w);
         ga[k] = shift_in_carry(ga[k], v.c, a.z);
@@ -305,12 +307,17 @@ __global__ void __launch_bounds__(TPB) k_sweep_gauss1d(RunDev* __restrict__ runs
 #pragma unroll
       for (int k = 0; k < RP; ++k)
         key[k] = sweep_key((uint32_t)(slot + k * NC), T0 + (uint32_t)((h0 + j) >> 1), rk);
-      if (live)
-        half_sweep_gauss1d<0, RP>(col, col + WR * CS, CS, s_thr, WR, last, w0, w1, half, key, rk, never);
-      __syncwarp();  // colour-1 words read what the other threads of the column wrote
-      if (live)
-        half_sweep_gauss1d<1, RP>(col + WR * CS, col, CS, s_thr + GCHAIN_ENTRY * WR, WR, last, w0, w1,
-                                  half + GCHAIN_CALLS * WR, key, rk, never);
+      const auto sweep = [&](auto nc) {
+        constexpr bool NEVER = decltype(nc)::value;
+        if (live)
+          half_sweep_gauss1d<0, RP, NEVER>(col, col + WR * CS, CS, s_thr, WR, last, w0, w1, half, key, rk);
+        __syncwarp();  // colour-1 words read what the other threads of the column wrote
+        if (live)
+          half_sweep_gauss1d<1, RP, NEVER>(col + WR * CS, col, CS, s_thr + GCHAIN_ENTRY * WR, WR, last, w0, w1,
+                                           half + GCHAIN_CALLS * WR, key, rk);
+      };
+      if (never) sweep(std::true_type());
+      else sweep(std::false_type());
       __syncwarp();
     }
   }

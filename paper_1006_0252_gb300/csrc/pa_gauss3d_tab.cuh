@@ -34,17 +34,16 @@
 // one byte permute per site yields the address of its entry.
 //
 // What bounds it: instruction issue and the multiply pipe, as the +-1 sweep
-// (pa_sweep3d.cuh).  At L = 8 a flip takes 17.1 instructions (10.8 of them the
+// (pa_sweep3d.cuh).  At L = 8 a flip takes 16.1 instructions (9.8 of them the
 // generator and the walk, 3.9 the patterns and table addresses, 1.1 the loads,
 // 1.3 the compare and its collection) where packed words and a compare into a
-// predicate took 20.8; ten sweeps of 1e5 replicas take 362 us of a launch, 255
-// of them the generator, and the tables, the gather and the energies 44.  One
-// launch, theta = 10, us (packed words, or one thread a replica and an
-// exponential per site at L = 10 -> now):
-//   L = 8   1e5 replicas 572 -> 404    2000 190 -> 29
-//   L = 10  80000 2400 -> 782    20000 794 -> 214    2000 648 -> 97
-//   L = 6   50000  199 -> 105     3000 168 -> 34
-//   L = 4   60000   80 -> 50      2000  39 -> 17
+// predicate took 20.8; of a launch of 1e5 replicas the generator takes 250 us and
+// the tables, the gather and the energies 44.  One launch, theta = 10, us (packed
+// words, or one thread a replica and an exponential per site at L = 10 -> now):
+//   L = 8   1e5 replicas 572 -> 376    2000 190 -> 29
+//   L = 10  80000 2400 -> 780    20000 794 -> 213    2000 648 -> 97
+//   L = 6   50000  199 -> 99      3000 168 -> 34
+//   L = 4   60000   80 -> 47      2000  39 -> 17
 // (populations that leave SMs idle gain most: the finest split spreads them.)
 // Not kept: the seed's round keys forced into uniform registers (same
 // instruction count), blocks of 512 threads (10-40 % slower; one block of 1024
@@ -140,8 +139,10 @@ __device__ __forceinline__ int fill_thresholds(uint32_t* __restrict__ s_thr, con
   return never;
 }
 
-// The word updates of one half sweep, as walk_rows calls them.
-template <int L, int RP>
+// The word updates of one half sweep, as walk_rows calls them.  NEVER: the table
+// has a threshold 0 (a parameter, not a branch: predicated off, the maxima still
+// take an issue slot a site).
+template <int L, int RP, bool NEVER>
 struct TabUpdate {
   using GEO = Geo3<L>;
   using HF = Half<GEO>;
@@ -149,7 +150,6 @@ struct TabUpdate {
   const uint4* half;  // its first call's entry
   const SweepKey (&key)[RP];
   const RoundKeys& rk;
-  bool never;  // the table has a threshold 0
   uint32_t carry[RP][4];
 
   template <int K, int A, int GP>
@@ -191,11 +191,9 @@ struct TabUpdate {
             for (int i = 0; i < 4; ++i) carry[k][i] = u[i];
           }
         }
-        if constexpr (!FOLD) {
-          if (never) {
+        if constexpr (NEVER) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) u[i] = max(u[i], 1u);
-          }
+          for (int i = 0; i < 4; ++i) u[i] = max(u[i], 1u);
         }
         static_for<0, 4>([&](auto jc) {
           constexpr int i = 3 - decltype(jc)::value, m = 4 * q + i - A;
@@ -377,9 +375,15 @@ __global__ void __launch_bounds__(TPB) k_sweep_gtab3d(RunDev* __restrict__ runs,
           key[k] = sweep_key((uint32_t)(first + k * ncol + r), T0 + (uint32_t)((h0 + j) >> 1), rk);
       }
       if (live) {
-        TabUpdate<L, RP> upd{thr0 + (uint32_t)(c * WR * S * 4 * E), half_table<GEO, P>(s_tab, j) + part + w0 * S / 4,
-                             key, rk, never, {}};
-        walk_rows<GEO, CS, RPP>(col, c, y0, upd);
+        const uint32_t thr = thr0 + (uint32_t)(c * WR * S * 4 * E);
+        const uint4* half = half_table<GEO, P>(s_tab, j) + part + w0 * S / 4;
+        if (!gtab_folded<L>() && never) {
+          TabUpdate<L, RP, !gtab_folded<L>()> upd{thr, half, key, rk, {}};
+          walk_rows<GEO, CS, RPP>(col, c, y0, upd);
+        } else {
+          TabUpdate<L, RP, false> upd{thr, half, key, rk, {}};
+          walk_rows<GEO, CS, RPP>(col, c, y0, upd);
+        }
       }
       // the next half sweep reads the words the other threads of the column wrote
       if constexpr (!pow2(P)) __syncthreads();

@@ -208,3 +208,29 @@ def test_classes_side_by_side(use_graph):
         ob = g.observables()
         assert res["R"][r] == ob["R"] and res["sumE"][r] == ob["sumE"] and res["sumE2"][r] == ob["sumE2"], r
         assert np.array_equal(b.spins(r, ob["R"]), g.spins()), r
+
+
+# Uniforms of exactly 0 (found by search: seed, slot, sweep, colour, call) at
+# thresholds of 0: such a site must stay, where any other threshold lets it go.
+@pytest.mark.parametrize("seed,slot,T,c,q", [(699, 356, 1, 0, 5), (3247, 1167, 3, 0, 8), (3332, 1187, 1, 1, 19),
+                                             (3760, 1084, 0, 0, 22), (3878, 231, 3, 0, 2), (3932, 1324, 4, 1, 3)])
+def test_uniform_zero_against_threshold_zero(seed, slot, T, c, q):
+    R0, beta = 1600, 200.0  # e^{-beta dE} is below 2^-32 for every rise of +-1 and almost every Gaussian one
+    made = []
+    for g in (False, True):
+        J = inputs.gaussian_couplings_lattice(8, 6, 5, 3) if g else inputs.couplings_lattice(8, 6, 5, 3, 1)
+        made.append((J, g, (8, 6, 5), 3))
+    made += [(inputs.gaussian_couplings_3d(L, 3, 1), True, (L, L, L), 7) for L in (6, 8, 10)]
+    made += [(inputs.couplings_3d(8, 3, 1), False, (8, 8, 8), 7)]
+    for J, g, (Lx, Ly, Lz), mask in made:
+        a = pa.Run(J, Lx, 3, R0, seed, R_cap=3000, gaussian=g, Ls=(Lx, Ly, Lz), periodic_mask=mask)
+        b = (o.GaussRun if g else o.Run)(J, 3, Lx, Ly, Lz, mask, R0=R0, R_cap=3000, seed=seed)
+        a.step(beta, 6)
+        b.step(beta, 6, R0)
+        assert a.observables()["R"] > slot
+        assert np.array_equal(a.spins(), b.spins()), (Lx, Ly, Lz, g)
+    J = inputs.gaussian_couplings_chain(256, 3, 1, open_chain=False)
+    a, b = pa.Run(J, 256, 1, R0, seed, R_cap=3000, gaussian=True), o.GaussRun(J, 1, 256, R0=R0, R_cap=3000, seed=seed)
+    a.step(beta, 6)
+    b.step(beta, 6, R0)
+    assert np.array_equal(a.spins(), b.spins())
