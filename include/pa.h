@@ -87,10 +87,11 @@ typedef struct pa_opts {
   int32_t threads_per_replica; /* threads sharing a replica's sweep: cubic lattices 1, 2, 4 or 8 for
                                   +-1 couplings, 1, 2 or 4 for Gaussian ones (ranges of whole rows;
                                   PA_ERR_INVALID where the rows do not split so; the library
-                                  itself also takes 3, 5, 6, 7 or 12, and lets a thread sweep two
+                                  itself also takes 3, 5, 6, 7, 8 or 12, and lets a thread sweep two
                                   replicas side by side in large populations); +-1 chains 1, 2,
                                   4 or 8 (ranges of ceil(words / P) words); Gaussian chains and
-                                  general boxes 1; 0 = library default */
+                                  general boxes 1 (the library itself up to 8 and 32, where no
+                                  block size is asked for); 0 = library default */
 } pa_opts;
 
 /* Observables after the last committed step (Sec. 2: measured after the
