@@ -20,9 +20,6 @@
 
 namespace pa {
 
-// Largest dynamic shared memory of a block (227 KB less the static part).
-constexpr size_t BOX_SMEM_MAX = 227 * 1024 - 256;
-
 template <int TPB>
 __device__ __forceinline__ uint32_t col_bit(const uint32_t* __restrict__ col, int code) {
   return (col[(code >> 5) * TPB] >> (code & 31)) & 1u;
@@ -213,9 +210,9 @@ template <int TPB>
 static cudaError_t launch_box_t(int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
                                 bool init) {
   const size_t sm = box_smem_bytes(WR, S, TPB);
-  if (sm > BOX_SMEM_MAX) return nwork > 0 ? cudaErrorInvalidValue : cudaSuccess;
+  if (sm > SMEM_LIMIT) return nwork > 0 ? cudaErrorInvalidValue : cudaSuccess;
   if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_box<TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_sweep_box<TPB>);
     if (e != cudaSuccess) return e;
   }
   if (nwork <= 0) return cudaSuccess;

@@ -397,7 +397,7 @@ cudaError_t launch_boxtab_s(const BoxShape& box, RunDev* runs, const Work* table
   const size_t sm = sizeof(uint32_t) * boxtab_shape(WR, S, box).words;
   if (nwork <= 0) {
     if (sm <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute((const void*)k_sweep_boxtab<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    return allow_shared(k_sweep_boxtab<S>);
   }
   k_sweep_boxtab<S><<<nwork, BOX_TPB, sm, st>>>(runs, table, box);
   return cudaGetLastError();

@@ -66,7 +66,6 @@ void clear_last_error() { g_err.clear(); }
 // Largest general box: its per-site tables (28 words per site pair) stay in
 // shared memory next to the spin columns.
 constexpr int MAX_BOX_SITES = 2048;
-constexpr size_t SMEM_LIMIT = 227 * 1024 - 256;
 
 // General Lx x Ly x Lz box (periodic axis d where bit d of mask is set),
 // either coupling model; J is int8 (model 0) or int32 fixed point (model 1)
@@ -760,8 +759,8 @@ int launch_class(Engine& E, const LatticeClass& c, const Work* table, int nwork,
   return launch_class_on(E.d_runs, E.st, c, table, nwork, init);
 }
 
-// Set the dynamic shared-memory limits of the class's launch shape, outside
-// any stream capture (again wherever the shape changes).
+// Allow the kernels of the class's launch shape the shared memory they take,
+// outside any stream capture (again wherever the shape changes).
 int prepare_class_launch(RunDev* runs, cudaStream_t st, const LatticeClass& c) {
   int s = launch_class_on(runs, st, c, nullptr, 0, false);
   return s == PA_OK ? launch_class_on(runs, st, c, nullptr, 0, true) : s;

@@ -411,7 +411,7 @@ static cudaError_t launch_g1d_p(RunDev* runs, const Work* table, int nwork, int 
     const size_t sm = need > (size_t)min_smem ? need : (size_t)min_smem;
     if (nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
-      return cudaFuncSetAttribute(k_sweep_gauss1d<TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      return allow_shared(k_sweep_gauss1d<TPB, P, RP>);
     }
     k_sweep_gauss1d<TPB, P, RP><<<nwork * (P / RP), TPB, sm, st>>>(runs, table);
     return cudaGetLastError();
@@ -425,7 +425,7 @@ static cudaError_t launch_g1d_t(int split, int rp, RunDev* runs, const Work* tab
     const size_t sm = sizeof(uint32_t) * (size_t)WR * TPB;
     if (nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
-      return cudaFuncSetAttribute(k_init_gauss1d<TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      return allow_shared(k_init_gauss1d<TPB>);
     }
     k_init_gauss1d<TPB><<<nwork, TPB, sm, st>>>(runs, table);
     return cudaGetLastError();

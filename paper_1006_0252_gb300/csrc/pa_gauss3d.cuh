@@ -405,8 +405,7 @@ cudaError_t launch_gauss3d_p(const Sweep3dLaunch& a) {
   } else {
     const size_t sm = sizeof(uint32_t) * GaussShape<L, TPB, P>::SMEM_WORDS;
     if (sm > 48 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute((const void*)k_sweep_gauss3d<L, TPB, P>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      cudaError_t e = allow_shared(k_sweep_gauss3d<L, TPB, P>);
       if (e != cudaSuccess) return e;
     }
     if (a.nwork <= 0) return cudaSuccess;
@@ -420,8 +419,7 @@ cudaError_t launch_gauss3d_init(const Sweep3dLaunch& a) {
   using GEO = Geo3<L>;
   const size_t sm = 4 * (gauss_tables_words<L>() + (size_t)GEO::WR * TPB);
   if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_init_gauss3d<L, TPB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = allow_shared(k_init_gauss3d<L, TPB>);
     if (e != cudaSuccess) return e;
   }
   if (a.nwork <= 0) return cudaSuccess;

@@ -274,7 +274,7 @@ struct GTabShape {
   static_assert(GEO::WR * Half<GEO>::S * 64 <= TAB, "the energy table takes the threshold table's memory");
   static_assert(P * NR <= TAB, "the row ranges' energies take the threshold table's memory at the end");
   static_assert(NR <= TPB, "one thread records a replica");
-  static_assert(4 * SMEM_WORDS <= 227 * 1024, "shared memory of a block");
+  static_assert(4 * SMEM_WORDS <= SMEM_LIMIT, "shared memory of a block");
 };
 
 // Sec. 2 with the Gaussian couplings of Sec. 4: gather of the resampled
@@ -470,8 +470,7 @@ cudaError_t launch_gtab3d_p(const Sweep3dLaunch& a) {
     const size_t sm = sizeof(uint32_t) * SH::SMEM_WORDS;
     if (a.nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
-      return cudaFuncSetAttribute((const void*)k_sweep_gtab3d<L, TPB, P, RP>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      return allow_shared(k_sweep_gtab3d<L, TPB, P, RP>);
     }
     k_sweep_gtab3d<L, TPB, P, RP><<<a.nwork, TPB, sm, a.st>>>(a.runs, a.table, a.slots);
     return cudaGetLastError();

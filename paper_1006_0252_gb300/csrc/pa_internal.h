@@ -129,6 +129,21 @@ struct Sweep3dLaunch {
   cudaStream_t st;
 };
 
+// Dynamic shared memory a block of this library may ask for: the 227 KB that an SM
+// gives one block, less room for a kernel's static arrays.
+constexpr size_t SMEM_LIMIT = 227 * 1024 - 256;
+
+// Let a kernel's launches take more than 48 KB of dynamic shared memory.  The
+// attribute belongs to the kernel on the device, so to every handle of the
+// process, while a block's need depends on the lattice and the population: it
+// only ever takes this one value, which no launch exceeds.  (Set to the need of
+// the class at hand, the limit failed the launches of every handle made before
+// that needs more.)
+template <class K>
+inline cudaError_t allow_shared(K* kernel) {
+  return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT);
+}
+
 // Launch of a kernel that begins with cudaGridDependencySynchronize(): its
 // blocks may take their place on the SMs before the kernel ahead of it in the
 // stream has finished (where that one triggers, as soon as all of its blocks

@@ -385,8 +385,8 @@ __global__ void __launch_bounds__(TPB) k_init1d(RunDev* __restrict__ runs,
   measure_store(R, 0, slot, live, E);
 }
 
-// One launch over nwork work items (with nwork <= 0 only the dynamic shared
-// memory limit is raised, outside any stream capture).
+// One launch over nwork work items (with nwork <= 0 the kernel is only
+// allowed its shared memory, outside any stream capture).
 template <int TPB, int P, int RP>
 static cudaError_t launch_sweep1d_p(RunDev* runs, const Work* table, int nwork, int WR, cudaStream_t st,
                                     int min_smem) {
@@ -397,7 +397,7 @@ static cudaError_t launch_sweep1d_p(RunDev* runs, const Work* table, int nwork, 
     const size_t sm = need > (size_t)min_smem ? need : (size_t)min_smem;
     if (nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
-      return cudaFuncSetAttribute(k_sweep1d<TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      return allow_shared(k_sweep1d<TPB, P, RP>);
     }
     k_sweep1d<TPB, P, RP><<<nwork * (P / RP), TPB, sm, st>>>(runs, table);
     return cudaGetLastError();
@@ -426,7 +426,7 @@ static cudaError_t launch1d_t(RunDev* runs, const Work* table, int nwork, int W,
   const size_t sm = sizeof(uint32_t) * (4 * (size_t)W + (size_t)WR * TPB);
   if (nwork <= 0) {
     if (sm <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(k_init1d<TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    return allow_shared(k_init1d<TPB>);
   }
   k_init1d<TPB><<<nwork, TPB, sm, st>>>(runs, table);
   return cudaGetLastError();

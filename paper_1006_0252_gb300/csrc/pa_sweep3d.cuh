@@ -476,8 +476,8 @@ inline size_t init3d_smem() {
   return sizeof(uint32_t) * (6 * GEO::W + GEO::WR * TPB);
 }
 
-// One launch over nwork work items (with nwork <= 0 only the dynamic shared
-// memory limit is raised, outside any stream capture).
+// One launch over nwork work items (with nwork <= 0 the kernel is only
+// allowed its shared memory, outside any stream capture).
 template <int L, int TPB, int P, int RP>
 cudaError_t sweep3d_p(const Sweep3dLaunch& a) {
   if constexpr (!rows_split<Geo3<L>>(P)) {
@@ -489,8 +489,7 @@ cudaError_t sweep3d_p(const Sweep3dLaunch& a) {
     const int need = (int)(sizeof(uint32_t) * SH::SMEM_WORDS), sm = need > a.min_smem ? need : a.min_smem;
     if (a.nwork <= 0) {
       if (sm <= 48 * 1024) return cudaSuccess;
-      return cudaFuncSetAttribute((const void*)k_sweep3d<L, TPB, P, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  sm);
+      return allow_shared(k_sweep3d<L, TPB, P, RP>);
     }
     return launch_dependent(k_sweep3d<L, TPB, P, RP>, a.nwork * SH::BPI, TPB, (size_t)sm, a.st, a.runs, a.table);
   }
@@ -500,8 +499,7 @@ template <int L, int TPB>
 cudaError_t launch_init3d_t(int slots, RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
   const size_t sm = init3d_smem<L, TPB>();
   if (sm > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute((const void*)k_init3d<L, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const cudaError_t e = allow_shared(k_init3d<L, TPB>);
     if (e != cudaSuccess) return e;
   }
   if (nwork <= 0) return cudaSuccess;
