@@ -549,9 +549,12 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   } else if (gauss_chain(c) && tpb_opt == 0) {
     c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : (c.Wr >= 2 ? 2 : 1));
   }
-  if (tpb_opt && tpb_supported(c, tpb_opt)) c.tpb = tpb_opt;
+  // The blocks of 512 and 1024 threads of the threshold-table kernel, where it has a
+  // shape with the split asked for (not for L = 10 with one thread a replica).
+  const bool table = gauss_cubic(c) && (gtab_shape_ok(c.L, c.split, 1) || gtab_shape_ok(c.L, c.split, 2));
+  if (tpb_opt && tpb_supported(c, tpb_opt) && (tpb_opt < 512 || table)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
-  else if (gauss_cubic(c) && gtab_finest(c.L) > 0) c.tpb = 1024;
+  else if (table) c.tpb = 1024;
   else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * NUM_SMS ? 256 : 128;  // 5 threads a replica: 25 or 51 of
                                                                                   // them a block
   else if (c.split > 1) c.tpb = 128;

@@ -234,3 +234,20 @@ def test_uniform_zero_against_threshold_zero(seed, slot, T, c, q):
     a.step(beta, 6)
     b.step(beta, 6, R0)
     assert np.array_equal(a.spins(), b.spins())
+
+
+# Gaussian cubic lattices with every number of threads per replica that their
+# rows split into, in every block size: what the threshold tables have no shape
+# for (L = 10 with one thread a replica) runs in a smaller block.
+@pytest.mark.parametrize("L,split", [(4, 1), (4, 2), (4, 4), (6, 1), (8, 1), (8, 2), (8, 4), (10, 1), (12, 1), (12, 2)])
+@pytest.mark.parametrize("tpb", [0, 128, 512, 1024])
+def test_gauss_cubic_asked_shape_bit_exact(L, split, tpb):
+    J = inputs.gaussian_couplings_3d(L, 4, 1)
+    g = pa.Run(J, L, 3, 301, 53, gaussian=True, threads_per_block=tpb, threads_per_replica=split)
+    assert pa.pa_sweep_shape(g._h)[1] == split
+    c = o.GaussRun(J, 3, L, L, L, 7, R0=301, seed=53)
+    for beta in (0.4, 1.5):
+        g.step(beta, 1)
+        c.step(beta, 1, 301)
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.spins(), c.spins())
