@@ -495,28 +495,38 @@ static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
   return best;
 }
 
+// Share of a work item (table_item), and the shared memory that keeps a launch's
+// blocks even over the SMs; alone: no other class is swept side by side.
+//
 // While a launch's blocks fit the SMs at once, the SM that gets the most of
-// them sets its time, and the hardware does not deal them out evenly: 296
-// blocks of 256 threads, two an SM, ran 1.44 times as long wherever three
-// fitted one.  So a block asks for as much shared memory as leaves an SM no
-// room for more than its even share of the blocks that hold replicas (a
-// population stays within three standard deviations, sqrt(R0), of its target;
-// a larger one only takes longer).  With more blocks than that it changes
-// nothing.
-void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0) {
+// them sets its time, and where they nearly fill `most` of them on every SM the
+// hardware gives some SMs one more.  Then a block asks for so much shared
+// memory that most + 1 of them do not fit an SM, and no more.  One launch of 40
+// steps, theta = 10, ms without and with it, at 0.95-0.98 of most x SMs:
+// L = 8, 7000 replicas 2.66 / 2.30; L = 16, 7000 14.1 / 11.2; L = 10, 30000 15.4 /
+// 11.0; chain of 4096, 7000 11.6 / 9.3; Gaussian chain of 256, 9400 2.33 / 2.14.
+// Up to 0.9 of them, and with at most one block an SM, it changes nothing (90 sizes of
+// ten lattices), but would shut out the blocks of whatever else runs: eight
+// chains of 256 spins, 2000 replicas each, stepped from eight threads took 4.55 ms with it, 2.42
+// without, and the classes of one step are side by side on purpose (three chains
+// of 2000 replicas 3.41 / 2.59).
+// (The population stays within three standard deviations, sqrt(R0), of its
+// target; a larger one only takes longer.)
+void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone) {
   constexpr int SM_SMEM = 228 * 1024, BLOCK_RESERVED = 1024;
   c.min_smem = 0;
   c.item = gauss_table(c) || box_table(c) ? table_item(c, R0) : 0;
-  if (!sweeps_pairs(c)) return;
+  if (!sweeps_pairs(c) || !alone) return;
   const int64_t per_block = c.tpb / c.split * c.rp;
   int64_t blocks = 0;
   for (int64_t r : R0) blocks += (r + (int64_t)(3.0 * std::sqrt((double)r)) + per_block - 1) / per_block;
-  const int64_t most = std::max<int64_t>(1, (blocks + NUM_SMS - 1) / NUM_SMS);
-  c.min_smem = std::max<int>(0, std::min<int>((int)SMEM_LIMIT, (int)(SM_SMEM / most) / 128 * 128 - BLOCK_RESERVED));
+  const int64_t most = (blocks + NUM_SMS - 1) / NUM_SMS;
+  if (most < 2 || 10 * blocks < 9 * most * NUM_SMS) return;
+  c.min_smem = std::max<int>(0, (int)(SM_SMEM / (most + 1)) / 128 * 128 + 128 - BLOCK_RESERVED);
 }
 
-// Launch shape of a class before any autotuning; R0: the target populations
-// of its runs.  Gaussian cubic sweeps of L <= 10 take the threshold-table
+// Launch shape of a class before any autotuning (spread_blocks follows); R0: the
+// target populations of its runs.  Gaussian cubic sweeps of L <= 10 take the threshold-table
 // kernel on its finest split, of L = 12 four threads per replica, which keeps
 // enough warps resident to hide the latency of the generator's dependent
 // multiplies; chains up to 8 on ranges of words; other classes 1.
@@ -527,10 +537,7 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   for (int64_t r : R0) replicas += r;
   c.sites = (double)replicas * (c.dim == 1 ? c.L : (c.bx > 0 ? (double)c.bx * c.by * c.bz : (double)c.L * c.L * c.L));
   c.tpb = 0;
-  if (c.bx > 0 && tpb_opt == 0 && split_opt == 0 && set_box_table(c, replicas)) {
-    spread_blocks(c, R0);
-    return;
-  }
+  if (c.bx > 0 && tpb_opt == 0 && split_opt == 0 && set_box_table(c, replicas)) return;
   if (split_opt > 0) {
     c.split = split_supported(c, split_opt) ? split_opt : 1;
   } else if (pm_cubic(c)) {
@@ -580,7 +587,6 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
         (gtab_shape_ok(c.L, c.split, 2) && replicas * c.split > from * NUM_SMS))
       c.rp = 2;
   }
-  spread_blocks(c, R0);
 }
 
 // Every launch shape the sweep kernel of a class has.
@@ -896,6 +902,7 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
     std::vector<int64_t> R0;
     for (int32_t r : c.runs) R0.push_back(E.R0[r]);
     set_default_launch(c, tpb_opt, split_opt, R0);
+    spread_blocks(c, R0, E.cls.size() == 1);
     if (split_opt > 1 && c.split != split_opt)
       return fail(PA_ERR_INVALID, "%d threads per replica do not split the rows of this lattice or block", split_opt);
     st = build_class_table(E, c);

@@ -310,7 +310,7 @@ int setup_run(char* base, const Geometry& g, const pa_run_spec& s, int64_t cap, 
               cudaStream_t st, RunDev* out);
 int default_tpb(int dim, int L);
 void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0);
-void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0);
+void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone);
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c);
 bool split_supported(const LatticeClass& c, int split);
 bool tpb_supported(const LatticeClass& c, int tpb);

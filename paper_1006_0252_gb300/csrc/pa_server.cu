@@ -127,11 +127,13 @@ static int server_rebuild_tables(pa_server* S) {
     }
     S->cls[k].runs.push_back(sl);
   }
+  const int used = (int)std::count_if(S->cls.begin(), S->cls.end(), [](const LatticeClass& c) { return !c.runs.empty(); });
   for (size_t k = 0; k < S->cls.size(); ++k) {
     LatticeClass& c = S->cls[k];
     std::vector<int64_t> R0;
     for (int32_t sl : c.runs) R0.push_back(S->h[sl].R);
     set_default_launch(c, S->tpb_opt, S->split_opt, R0);  // the shape follows the runs that are active
+    spread_blocks(c, R0, used == 1);
     if (!c.runs.empty()) {
       const int st = prepare_class_launch(S->d_runs, S->st, c);
       if (st != PA_OK) return st;

@@ -1,0 +1,84 @@
+"""The host rules that choose a launch shape, called in the built library (no
+GPU): a small program is compiled against the engine's header."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1006_0252_gb300 import build
+
+# Prints, for a class given as (kind, size, alone, R0 ...): threads a block,
+# threads a replica, replicas a thread, shared memory asked for, slots of an item.
+PROGRAM = r"""
+#include "pa_engine.h"
+int main(int n, char** a) {
+  LatticeClass c;
+  const std::string kind = a[1];
+  c.model = kind[0] == 'g';
+  c.dim = kind.back() == 'c' ? 1 : 3;
+  c.L = atoi(a[2]);
+  c.Wr = (c.L + 31) / 32;
+  c.W = (c.Wr + 3) / 4 * 4;
+  std::vector<int64_t> R0;
+  for (int i = 4; i < n; ++i) R0.push_back(atoll(a[i]));
+  set_default_launch(c, 0, 0, R0);
+  spread_blocks(c, R0, atoi(a[3]) != 0);
+  printf("%d %d %d %d %d\n", c.tpb, c.split, c.rp, c.min_smem, c.item);
+}
+"""
+SM_SMEM, BLOCK_RESERVED, NUM_SMS = 228 * 1024, 1024, 152
+
+
+@pytest.fixture(scope="module")
+def shape(tmp_path_factory):
+    lib = build.build_library()
+    d = tmp_path_factory.mktemp("shape")
+    src, exe = d / "shape.cu", d / "shape"
+    src.write_text(PROGRAM)
+    where = os.path.dirname(lib)
+    p = subprocess.run([build.nvcc(), *build.ARCH, "-std=c++17", "--expt-relaxed-constexpr", "-I", build.CSRC, "-I",
+                        build.INCLUDE, str(src), "-o", str(exe), "-L", where, "-l:" + os.path.basename(lib), "-Xlinker",
+                        "-rpath=" + where], capture_output=True, text=True)
+    assert p.returncode == 0, p.stderr
+
+    def call(kind, size, *R0, alone=True):
+        out = subprocess.run([str(exe), kind, str(size), str(int(alone)), *map(str, R0)], capture_output=True, text=True)
+        assert out.returncode == 0, out.stderr
+        return dict(zip(("tpb", "split", "rp", "min_smem", "item"), map(int, out.stdout.split())))
+
+    return call
+
+
+# (kind, size): pm / gpm cubic, c / gc chains.
+SPREAD = [("pm", 4), ("pm", 6), ("pm", 8), ("pm", 10), ("pm", 12), ("pm", 14), ("pm", 16), ("c", 256), ("c", 4096),
+          ("gc", 256)]
+
+
+def _blocks(sh, R0):
+    per = sh["tpb"] // sh["split"] * sh["rp"]
+    return -(-(R0 + int(3 * R0 ** 0.5)) // per)
+
+
+@pytest.mark.parametrize("kind,size", SPREAD)
+def test_no_shared_memory_is_held_where_it_evens_nothing(shape, kind, size):
+    """At most one block an SM, or blocks that leave a tenth of their places
+    free: nothing that would keep the blocks of other handles out."""
+    for R0 in (100, 300, 1000, 1500, 2000, 2300, 3400, 5600, 8000, 16000):
+        sh = shape(kind, size, R0)
+        blocks = _blocks(sh, R0)
+        most = -(-blocks // NUM_SMS)
+        if most == 1 or blocks < 0.9 * most * NUM_SMS:
+            assert sh["min_smem"] == 0, (R0, sh)
+
+
+@pytest.mark.parametrize("kind,size", SPREAD)
+def test_shared_memory_keeps_one_block_more_out(shape, kind, size):
+    for R0 in range(3000, 16000, 700):
+        sh = shape(kind, size, R0)
+        blocks = _blocks(sh, R0)
+        most = -(-blocks // NUM_SMS)
+        if most > 1 and blocks >= 0.9 * most * NUM_SMS:
+            held = sh["min_smem"] + BLOCK_RESERVED
+            assert most * held <= SM_SMEM < (most + 1) * held, (R0, sh)
+        # classes of one step share the SMs
+        assert shape(kind, size, R0, alone=False)["min_smem"] == 0
