@@ -2,6 +2,8 @@
 // advanced together by one Engine, their schedules captured as CUDA graphs,
 // and the Sec. 3 estimators over groups of runs computed on the device.
 #include <algorithm>
+#include <numeric>
+
 #include "pa_engine.h"
 
 extern "C" {
@@ -297,7 +299,7 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
     LaunchShape pick = {c.tpb, c.split, c.rp};
     LatticeClass trial = c;
     std::vector<int64_t> R0;
-    for (int32_t r : c.runs) R0.push_back(E.R0[r]);
+    for (int32_t r : c.runs) R0.push_back(E.most[r]);
     for (const LaunchShape& cand : launch_shapes(c)) {
       if (cand.split == 1 && cand.tpb == 256) continue;
       trial.tpb = cand.tpb;
@@ -325,8 +327,10 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
         pick = cand;
       }
     }
+    c.tuned = true;
+    c.shaped = c.spread = std::accumulate(R0.begin(), R0.end(), (int64_t)0);
     if (pick.tpb != c.tpb || pick.split != c.split || pick.rp != c.rp) {
-      E.dfree(c.d_table, sizeof(Work) * std::max(c.nwork, 1));
+      E.dfree(c.d_table, sizeof(Work) * std::max(c.room, 1));
       c.tpb = pick.tpb;
       c.split = pick.split;
       c.rp = pick.rp;

@@ -775,15 +775,87 @@ int prepare_class_launch(RunDev* runs, cudaStream_t st, const LatticeClass& c) {
   return s == PA_OK ? launch_class_on(runs, st, c, nullptr, 0, true) : s;
 }
 
-int build_class_table(Engine& E, LatticeClass& c) {
+static std::vector<Work> class_items(const Engine& E, const LatticeClass& c) {
   std::vector<Work> t;
   for (int32_t r : c.runs)
     for (int64_t f = 0; f < E.h[r].R_cap; f += c.slots()) t.push_back({r, (int32_t)f});
-  c.nwork = (int)t.size();
+  return t;
+}
+
+int build_class_table(Engine& E, LatticeClass& c) {
+  const std::vector<Work> t = class_items(E, c);
+  c.nwork = c.room = (int)t.size();
   c.d_table = (Work*)E.dalloc(sizeof(Work) * std::max<size_t>(t.size(), 1));
   if (!c.d_table) return fail(PA_ERR_OOM, "work table allocation refused");
   if (!t.empty()) PA_CUDA(cudaMemcpyAsync(c.d_table, t.data(), sizeof(Work) * t.size(), cudaMemcpyHostToDevice, E.st));
   PA_CUDA(cudaStreamSynchronize(E.st));
+  return PA_OK;
+}
+
+// Launch shapes for the population targets of the coming steps (one per run)
+// where these are above those that the shapes were chosen for.  A shape for 1000
+// replicas is a poor one for 1e5: work items of a few slots, each of which builds
+// the tables of a whole block, one replica a thread, blocks that hold shared memory
+// to spread few of them evenly.  40 steps of theta = 10 at the larger target, ms, with the
+// first shape and so: Gaussian L = 6, 1000 -> 50000 replicas 40.9 / 5.2; Gaussian L = 8,
+// 1000 -> 1e5 79.0 / 16.8; +-1 L = 8, 1000 -> 1e5 29.5 / 15.1; +-1 chain of 256, 1000 -> 1e5
+// 21.4 / 7.4; 8 x 6 x 5 box, 1000 -> 3000 3.9 / 2.2.
+// The even spread follows every larger target; the shape is chosen again from
+// half as many replicas more on.  A change waits for the stream once and captures
+// the schedule anew.  Nothing is allocated (larger work items need fewer entries;
+// where the table has no room the shape stays), and while the caller captures the
+// stream all stays as it is.
+static int refit_classes(Engine& E, const std::vector<int64_t>& targets) {
+  const auto target = [&](int r) { return std::min<int64_t>(targets[r], E.h[r].R_cap); };
+  bool more = false;
+  for (int r = 0; r < E.n; ++r) more = more || target(r) > E.most[r];
+  if (!more) return PA_OK;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  PA_CUDA(cudaStreamIsCapturing(E.st, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return PA_OK;
+  for (int r = 0; r < E.n; ++r) E.most[r] = std::max(E.most[r], target(r));
+  const bool alone = E.cls.size() == 1;
+  for (auto& c : E.cls) {
+    std::vector<int64_t> R;
+    int64_t sum = 0;
+    for (int32_t r : c.runs) {
+      R.push_back(E.most[r]);
+      sum += E.most[r];
+    }
+    if (sum == c.spread) continue;
+    LatticeClass n = c;
+    std::vector<Work> t;
+    if (2 * sum > 3 * c.shaped) {
+      if (!c.tuned) set_default_launch(n, E.tpb_opt, E.split_opt, R);
+      else n.sites *= (double)sum / (double)c.shaped;
+      spread_blocks(n, R, alone);
+      t = class_items(E, n);
+      if ((int)t.size() > c.room) {
+        n = c;
+        t.clear();
+      }
+      n.shaped = sum;
+    }
+    if (t.empty()) {
+      spread_blocks(n, R, alone);
+      n.item = c.item;
+    }
+    n.spread = sum;
+    const bool items = n.slots() != c.slots();
+    if (items || n.tpb != c.tpb || n.split != c.split || n.rp != c.rp || n.min_smem != c.min_smem) {
+      PA_CUDA(cudaStreamSynchronize(E.st));
+      E.harvest_graph_timing();
+      E.drop_graph();
+      const int s = prepare_class_launch(E.d_runs, E.st, n);
+      if (s != PA_OK) return s;
+      if (items) {
+        n.nwork = (int)t.size();
+        PA_CUDA(cudaMemcpyAsync(n.d_table, t.data(), sizeof(Work) * t.size(), cudaMemcpyHostToDevice, E.st));
+        PA_CUDA(cudaStreamSynchronize(E.st));
+      }
+    }
+    c = n;
+  }
   return PA_OK;
 }
 
@@ -834,6 +906,9 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
     if (cap > 0x7FFFFF00LL) return fail(PA_ERR_INVALID, "R_cap too large");
     E.R0[r] = s.R0;
   }
+  E.most = E.R0;
+  E.tpb_opt = tpb_opt;
+  E.split_opt = split_opt;
   if (E.st == nullptr) {
     // a private stream: graph capture needs a non-default stream
     PA_CUDA(cudaStreamCreateWithFlags(&E.st, cudaStreamNonBlocking));
@@ -903,6 +978,8 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
     for (int32_t r : c.runs) R0.push_back(E.R0[r]);
     set_default_launch(c, tpb_opt, split_opt, R0);
     spread_blocks(c, R0, E.cls.size() == 1);
+    for (int64_t r : R0) c.shaped += r;
+    c.spread = c.shaped;
     if (split_opt > 1 && c.split != split_opt)
       return fail(PA_ERR_INVALID, "%d threads per replica do not split the rows of this lattice or block", split_opt);
     st = build_class_table(E, c);
@@ -1111,6 +1188,13 @@ int engine_run_schedule(Engine& E, int n_steps, const double* betas, int per_run
   // read the timing of a replay still pending)
   PA_CUDA(cudaStreamSynchronize(E.st));
   E.harvest_graph_timing();
+  if (R_targets) {
+    std::vector<int64_t> most(E.n, 0);
+    for (int r = 0; r < E.n; ++r)
+      for (int k = 0; k < n_steps; ++k) most[r] = std::max(most[r], R_targets[per_run ? (size_t)r * n_steps + k : (size_t)k]);
+    const int st = refit_classes(E, most);
+    if (st != PA_OK) return st;
+  }
   if (!use_graph) {
     for (int k = 0; k < n_steps; ++k) {
       int st = engine_step(E, false, 0.0, 0, 0, k > 0, k + 1 < n_steps);
@@ -1419,7 +1503,8 @@ int pa_step_target(pa_run* run, double beta_next, int sweeps, int64_t R_target) 
   if (!(beta_next >= run->e.host_beta[0]) || !std::isfinite(beta_next))
     return fail(PA_ERR_INVALID, "beta must not decrease (%g after %g)", beta_next, run->e.host_beta[0]);
   PA_CUDA(cudaSetDevice(run->e.device));
-  int st = engine_step(run->e, true, beta_next, sweeps, R_target);
+  int st = refit_classes(run->e, {R_target});
+  if (st == PA_OK) st = engine_step(run->e, true, beta_next, sweeps, R_target);
   if (st != PA_OK) return st;
   run->e.host_beta[0] = beta_next;
   return PA_OK;

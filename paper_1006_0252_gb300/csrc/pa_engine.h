@@ -162,8 +162,10 @@ struct LatticeClass {
   int min_smem = 0;  // shared memory of a sweep block that keeps the blocks even over the SMs (spread_blocks)
   std::vector<int32_t> runs;
   Work* d_table = nullptr;
-  int nwork = 0;
-  double sites = 0.0;  // spins of all its replicas
+  int nwork = 0, room = 0;         // work items; those its table has room for
+  double sites = 0.0;              // spins of all its replicas
+  bool tuned = false;              // the shape was measured, not chosen
+  int64_t shaped = 0, spread = 0;  // target populations that the shape was chosen, the blocks spread for (sums)
   int item = 0;      // slots of a work item where they are chosen by the populations (spread_blocks), else 0
   // Slots of a work item: the block's threads where a power of two of them
   // shares a replica (split / rp blocks an item), else the block's replicas.
@@ -197,6 +199,8 @@ struct Engine {
   int n = 0;
   std::vector<RunDev> h;           // host copies of the static part
   std::vector<int64_t> R0;
+  std::vector<int64_t> most;       // largest population target of each run so far
+  int tpb_opt = 0, split_opt = 0;  // the launch shape asked for (pa_opts)
   RunDev* d_runs = nullptr;
   std::vector<LatticeClass> cls;
   ClassFan fan;
