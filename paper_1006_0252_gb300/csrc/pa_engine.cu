@@ -936,7 +936,10 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
   for (int r = 0; r < n_runs; ++r)
     for (int64_t f = 0; f < E.h[r].R_cap; f += CHUNK) ct.push_back({r, (int32_t)f});
   E.small = E.model == 0;
-  for (const RunDev& d : E.h) E.small = E.small && d.R_cap <= SMALL_RUN;
+  int64_t largest = 0;
+  for (const RunDev& d : E.h) largest = std::max(largest, d.R_cap);
+  E.small = E.small && largest <= SMALL_RUN;
+  E.small_threads = largest <= 512 || n_runs > NUM_SMS ? 256 : 1024;
   E.n_copy_work = (int)ct.size();
   E.d_copy_table = (Work*)E.dalloc(sizeof(Work) * ct.size());
   if (!E.d_copy_table) return fail(PA_ERR_OOM, "work table allocation refused");
@@ -1019,7 +1022,7 @@ int engine_prep(Engine& E, bool ovr, double beta, int theta, int64_t Rt) {
 static int engine_resample(Engine& E, bool commit_first, bool ovr, double beta, int theta, int64_t Rt) {
   if (E.small) {
     NvtxRange r("reweight+copies+sources (k_resample)");
-    PA_CUDA(launch_resample(E.d_runs, nullptr, E.n, commit_first, ovr, beta, theta, Rt, E.st));
+    PA_CUDA(launch_resample(E.small_threads, E.d_runs, nullptr, E.n, commit_first, ovr, beta, theta, Rt, E.st));
     E.launches += 1;
     return PA_OK;
   }

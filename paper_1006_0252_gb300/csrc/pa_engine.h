@@ -28,8 +28,8 @@ cudaError_t launch_init_state(RunDev* runs, const int32_t* ids, int n, int max_b
 cudaError_t launch_init_finish(RunDev* runs, const int32_t* ids, int n, cudaStream_t st);
 cudaError_t launch_prepare(RunDev* runs, const int32_t* ids, int n, bool ovr, double beta, int theta,
                            int64_t Rt, cudaStream_t st);
-cudaError_t launch_resample(RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr, double beta,
-                            int theta, int64_t Rt, cudaStream_t st);
+cudaError_t launch_resample(int threads, RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr,
+                            double beta, int theta, int64_t Rt, cudaStream_t st);
 cudaError_t launch_copies(RunDev* runs, const Work* table, int nwork, cudaStream_t st);
 cudaError_t launch_scan(RunDev* runs, const int32_t* ids, int n, cudaStream_t st);
 cudaError_t launch_scatter(RunDev* runs, const Work* table, int nwork, cudaStream_t st);
@@ -219,6 +219,7 @@ struct Engine {
   bool capturing = false;
   int model = 0;  // all runs of an engine share one coupling model
   bool small = false;  // +-1 runs of at most SMALL_RUN replicas: resampled by one block each
+  int small_threads = 1024;  // of such a block (k_resample)
   // measurement hooks
   bool prof = false;
   int prof_stride = 1;       // time every prof_stride-th sweep launch

@@ -592,11 +592,17 @@ __global__ void __launch_bounds__(CHUNK) k_scatter(RunDev* __restrict__ runs, co
 // k_prepare, k_copies and k_scatter without the launches in between.  A run of
 // 1000 replicas at L = 4 took 30.7 us a step with six launches (of which 12.5
 // the sweep) in a graph, 24.5 with this one and the sweep.
-constexpr int SMALL_THREADS = 1024;
-__global__ void __launch_bounds__(SMALL_THREADS) k_resample(RunDev* __restrict__ runs, const int32_t* __restrict__ ids,
-                                                            int commit_first, int use_override, double beta_o,
-                                                            int theta_o, int64_t Rt_o) {
-  constexpr int NT = SMALL_THREADS;
+//
+// Blocks of 256 threads for populations of up to 512 slots, which leave most of a
+// larger block idle, and for more runs than SMs, where several blocks of an SM hide
+// one another's waits; else of 1024, which take fewer passes.  Batches of L = 4, 40
+// steps, ms with the launches apart / blocks of 1024 / of 256: 1 run of 1000 replicas
+// 1.24 / 0.93 / 1.03; 100 of 1000 4.47 / 3.36 / 3.50; 300 of 1000 11.0 / 8.70 / 8.35; 1000 of
+// 100 9.84 / 10.7 / 8.90; 3000 of 30 21.0 / 26.7 / 21.0.
+template <int NT>
+__global__ void __launch_bounds__(NT) k_resample(RunDev* __restrict__ runs, const int32_t* __restrict__ ids,
+                                                 int commit_first, int use_override, double beta_o, int theta_o,
+                                                 int64_t Rt_o) {
   __shared__ int64_t s_warp[NT / 32];
   __shared__ int64_t s_off[NT];
   __shared__ unsigned long long s_cnt[NT];
@@ -1072,10 +1078,10 @@ cudaError_t launch_prepare(RunDev* runs, const int32_t* ids, int n, bool ovr, do
   k_prepare<<<n, PREP_THREADS, 0, st>>>(runs, ids, ovr ? 1 : 0, beta, theta, Rt);
   return cudaGetLastError();
 }
-cudaError_t launch_resample(RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr, double beta,
-                            int theta, int64_t Rt, cudaStream_t st) {
-  return launch_dependent(k_resample, n, SMALL_THREADS, (size_t)0, st, runs, ids, commit_first ? 1 : 0, ovr ? 1 : 0,
-                          beta, theta, Rt);
+cudaError_t launch_resample(int threads, RunDev* runs, const int32_t* ids, int n, bool commit_first, bool ovr,
+                            double beta, int theta, int64_t Rt, cudaStream_t st) {
+  return launch_dependent(threads == 256 ? k_resample<256> : k_resample<1024>, n, threads, (size_t)0, st, runs, ids,
+                          commit_first ? 1 : 0, ovr ? 1 : 0, beta, theta, Rt);
 }
 cudaError_t launch_copies(RunDev* runs, const Work* table, int nwork, cudaStream_t st) {
   k_copies<<<nwork, CHUNK, 0, st>>>(runs, table);

@@ -1,6 +1,8 @@
 """Launch shapes the library chooses by itself (GPU): the +-1 cubic and chain
 sweeps and the Gaussian cubic sweep with one and with two replicas per thread
 against the oracle."""
+import time
+
 import numpy as np
 import pytest
 
@@ -251,3 +253,41 @@ def test_gauss_cubic_asked_shape_bit_exact(L, split, tpb):
         c.step(beta, 1, 301)
     assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.spins(), c.spins())
+
+
+# More runs than SMs: blocks of 256 threads, here with up to six passes over a population and
+# runs of a few replicas among them.
+def test_many_small_runs_bit_exact():
+    betas = np.array([0.2, 0.7, 2.5])
+    specs = [inputs.RunSpec(3, 4, r % 5, 100 + r, (40, 255, 256, 700, 1400)[r % 5], betas, 1) for r in range(160)]
+    b = pa.Batch(specs)
+    b.run(betas, thetas=1)
+    assert not b.sync().any()
+    res = b.results()
+    for r in (0, 1, 2, 3, 4, 77, 158, 159):
+        R0 = specs[r].R0
+        c = o.Run(specs[r].couplings(), 3, 4, 4, 4, 7, R0=R0, seed=100 + r)
+        for beta in betas:
+            c.step(float(beta), 1, R0)
+        assert res["R"][r] == c.state().R and res["sumE"][r] == c.state().sumE, r
+        assert np.array_equal(b.spins(r, c.state().R), c.spins()), r
+
+
+# ... and they take no longer than with the launches apart (capacities above
+# 2048), where blocks of 1024 threads took 1.15 times as long.
+def test_many_small_runs_take_no_longer():
+    betas = np.linspace(0.05, 4.0, 40)
+
+    def seconds(cap):
+        b = pa.Batch([inputs.RunSpec(3, 4, 0, 50 + r, 100, betas, 10, R_cap=cap) for r in range(3000)], max_steps=64)
+        times = []
+        for _ in range(5):
+            b.reset()
+            b.sync()
+            t = time.perf_counter()
+            b.run(betas, thetas=10)
+            b.sync()
+            times.append(time.perf_counter() - t)
+        return min(times)
+
+    assert seconds(2048) <= 1.05 * seconds(2049)
