@@ -424,7 +424,9 @@ int pa_batch_diagnostics(pa_batch* b, int M, int64_t count, double* E_bar,
  * and record).  Argument rules and errors as pa_batch_diagnostics, plus
  * 2 <= B <= 2^20; host arrays [n_runs / M][count], either may be NULL;
  * synchronises; scratch of 8 (3 M + 2 B + 2) n_runs/M count bytes from the
- * batch's allocator (PA_ERR_OOM if refused). */
+ * batch's allocator (PA_ERR_OOM if refused), and 8 (3 M + 1) n_runs/M count
+ * more for tabulated weights, without which, if refused, the call takes
+ * longer. */
 int pa_batch_bootstrap(pa_batch* b, int M, int64_t count, int B, uint64_t seed,
                        double* sd_E_bar, double* sd_minus_beta_Fbar);
 /* Sec. 4 overlap between runs of one batch, for n_pairs pairs at once:

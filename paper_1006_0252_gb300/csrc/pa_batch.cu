@@ -176,11 +176,16 @@ int pa_batch_bootstrap(pa_batch* b, int M, int64_t count, int B, uint64_t seed, 
   const int64_t GK = (int64_t)G * count;
   if (GK > INT32_MAX) return fail(PA_ERR_INVALID, "too many groups and records");
   const size_t nval = (size_t)GK * M, nres = (size_t)GK * B;
-  const size_t bytes = sizeof(double) * (3 * nval + 2 * nres + 2 * (size_t)GK + boot_table_size(M, GK));
-  double* buf = (double*)E.dalloc(bytes);
+  // with the weights' table where the allocator grants it, else without
+  size_t bytes = sizeof(double) * (3 * nval + 2 * nres + 2 * (size_t)GK);
+  const size_t table = sizeof(double) * boot_table_size(M, GK);
+  double* buf = (double*)E.dalloc(bytes + table);
+  const bool tabulated = buf != nullptr;
+  if (tabulated) bytes += table;
+  else buf = (double*)E.dalloc(bytes);
   if (!buf) return fail(PA_ERR_OOM, "bootstrap scratch of %zu bytes refused", bytes);
   double *x = buf, *A = x + nval, *Rw = A + nval, *bm = Rw + nval, *bf = bm + nres, *sm = bf + nres, *sf = sm + GK,
-         *tab = sf + GK;
+         *tab = tabulated ? sf + GK : nullptr;
   cudaError_t e = launch_gather_records(E.d_runs, M, (int)count, G, x, A, Rw, E.st);
   if (e == cudaSuccess) e = launch_bootstrap(M, x, A, Rw, B, seed, bm, bf, tab, E.st, (int)GK);
   if (e == cudaSuccess) e = launch_variance((int)GK, B, bm, sm, E.st, true);

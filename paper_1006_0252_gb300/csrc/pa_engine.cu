@@ -1784,10 +1784,16 @@ int pa_bootstrap(int M, const double* x, const double* A, const double* R, int B
   if (R && !all_positive(M, R)) return fail(PA_ERR_INVALID, "R weights must be positive");
   cudaStream_t st = nullptr;
   double* buf = nullptr;
+  bool table = true;  // of the weights, where there is memory for it
   int s = stage_inputs(M, x, A, R, &buf, st, 2 * (size_t)B + boot_table_size(M, 1));
+  if (s != PA_OK) {
+    cudaGetLastError();  // a refused allocation must not fail a later launch check
+    table = false;
+    s = stage_inputs(M, x, A, R, &buf, st, 2 * (size_t)B);
+  }
   if (s != PA_OK) return s;
   cudaError_t e = launch_bootstrap(M, buf, A ? buf + M : nullptr, R ? buf + 2 * M : nullptr, B, seed, buf + 3 * M,
-                                   buf + 3 * M + B, buf + 3 * M + 2 * (size_t)B, st);
+                                   buf + 3 * M + B, table ? buf + 3 * M + 2 * (size_t)B : nullptr, st);
   std::vector<double> bm(B), bf(B);
   if (e == cudaSuccess) e = cudaMemcpyAsync(bm.data(), buf + 3 * M, 8 * B, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(bf.data(), buf + 3 * M + B, 8 * B, cudaMemcpyDeviceToHost, st);
