@@ -1795,8 +1795,8 @@ int pa_bootstrap(int M, const double* x, const double* A, const double* R, int B
   cudaError_t e = launch_bootstrap(M, buf, A ? buf + M : nullptr, R ? buf + 2 * M : nullptr, B, seed, buf + 3 * M,
                                    buf + 3 * M + B, table ? buf + 3 * M + 2 * (size_t)B : nullptr, st);
   std::vector<double> bm(B), bf(B);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(bm.data(), buf + 3 * M, 8 * B, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(bf.data(), buf + 3 * M + B, 8 * B, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bm.data(), buf + 3 * M, 8 * (size_t)B, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(bf.data(), buf + 3 * M + B, 8 * (size_t)B, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   cudaFreeAsync(buf, st);
   if (e != cudaSuccess) return cuda_fail(e, "bootstrap");

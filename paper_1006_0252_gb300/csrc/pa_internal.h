@@ -178,6 +178,12 @@ constexpr bool gtab_shape_ok(int L, int split, int rp) {
   if (split == 1) return L <= 8 && rp == 1;
   return (L == 4 || L == 8) && (split == 2 || split == 4) && rp == 2;
 }
+// Resample of a thread of k_bootstrap, `lanes` threads each (the threads of a grid
+// of 2^31 - 1 resamples are more than 32 bits count).
+__host__ __device__ inline int64_t boot_resample(unsigned block, unsigned threads, unsigned thread, unsigned lanes) {
+  return (int64_t)block * (threads / lanes) + thread / lanes;
+}
+
 // Threshold-table kernel of general boxes (pa_boxtab.cuh): the geometry (extent
 // in x, words of a row, rows), P threads a column of `reps` replicas, `slots`
 // slots of a work item (whole warps of columns).

@@ -922,8 +922,8 @@ template <int LANES>
 __global__ void k_bootstrap(int M, const double* __restrict__ x, const double* __restrict__ A,
                             const double* __restrict__ Rw, const double* __restrict__ tab, int B, uint64_t seed,
                             int GK, double* __restrict__ bmean, double* __restrict__ bfbar) {
-  const int at = (blockIdx.x * blockDim.x + threadIdx.x) / LANES, lane = threadIdx.x % LANES;
-  const int b = min(at, B - 1);  // the threads past the last resample draw it again and write nothing
+  const int64_t at = boot_resample(blockIdx.x, blockDim.x, threadIdx.x, LANES);
+  const int lane = threadIdx.x % LANES, b = (int)min(at, (int64_t)B - 1);  // the threads past the last resample draw it again and write nothing
   for (int gk = blockIdx.y; gk < GK; gk += gridDim.y) {
     double S = 0.0, SA = 0.0, Sx = 0.0, mux = -INFINITY;
     bool direct = true;
@@ -1176,7 +1176,7 @@ cudaError_t launch_bootstrap(int M, const double* x, const double* A, const doub
                              double* bmean, double* bfbar, double* tab, cudaStream_t st, int GK) {
   const unsigned groups = (unsigned)std::min(GK, 65535);
   if (!tab) {
-    k_bootstrap<1><<<dim3((B + 127) / 128, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
+    k_bootstrap<1><<<dim3(((unsigned)B + 127) / 128, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
     return cudaGetLastError();
   }
   if (A && Rw) k_boot_weights<true, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
@@ -1186,8 +1186,8 @@ cudaError_t launch_bootstrap(int M, const double* x, const double* A, const doub
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   constexpr int LANES = 8, PER_BLOCK = 128 / LANES;
-  k_bootstrap<LANES><<<dim3((B + PER_BLOCK - 1) / PER_BLOCK, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK,
-                                                                                    bmean, bfbar);
+  k_bootstrap<LANES><<<dim3(((unsigned)B + PER_BLOCK - 1) / PER_BLOCK, groups), 128, 0, st>>>(M, x, A, Rw, tab, B,
+                                                                                              seed, GK, bmean, bfbar);
   return cudaGetLastError();
 }
 

@@ -14,6 +14,10 @@ PROGRAM = r"""
 int main(int n, char** a) {
   LatticeClass c;
   const std::string kind = a[1];
+  if (kind == "resample") {
+    printf("%lld 0 0 0 0\n", (long long)boot_resample(strtoul(a[2], 0, 10), 128, atoi(a[3]), 8));
+    return 0;
+  }
   c.model = kind[0] == 'g';
   c.dim = kind.back() == 'c' ? 1 : 3;
   c.L = atoi(a[2]);
@@ -82,3 +86,11 @@ def test_shared_memory_keeps_one_block_more_out(shape, kind, size):
             assert most * held <= SM_SMEM < (most + 1) * held, (R0, sh)
         # classes of one step share the SMs
         assert shape(kind, size, R0, alone=False)["min_smem"] == 0
+
+
+# Eight threads a resample, so a block of 128 threads takes 16: the thread's
+# number in the grid passes 2^32 from 2^29 resamples on.
+@pytest.mark.parametrize("block", [0, (1 << 25) - 1, 1 << 25, (1 << 27) - 1])
+def test_bootstrap_resample_of_a_thread(shape, block):
+    for thread in (0, 1):
+        assert shape("resample", block, alone=thread)["tpb"] == 16 * block
