@@ -414,7 +414,14 @@ static cudaError_t sweep3d_call(int L, const Sweep3dLaunch& a) {
   }
 }
 
-constexpr int NUM_SMS = 152;
+// Multiprocessors of a device (a GB300 has 152; read, since the same code runs
+// on parts with fewer enabled).
+int sm_count(int device) {
+  int n = 0;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) == cudaSuccess && n > 0) return n;
+  cudaGetLastError();
+  return LatticeClass().sms;
+}
 
 // Threads per replica of a +-1 cubic lattice before any autotuning: the most
 // that whole rows give, pairs of rows where a row's uniforms end within a
@@ -453,7 +460,7 @@ static int box_most(const LatticeClass& c, int P, int reps) {
 // 3000 replicas (16, 1) 64, (16, 2) 70, (8, 1) 87, (16, 4) 110.
 static bool set_box_table(LatticeClass& c, int64_t replicas) {
   const int U = box_period(c.bsites), groups = (c.Wr + U - 1) / U;
-  const int64_t share = (replicas + NUM_SMS - 1) / NUM_SMS;
+  const int64_t share = (replicas + c.sms - 1) / c.sms;
   int P = 1, reps = box_replicas(c.bsites);
   while (P < groups && P < 32) P *= 2;
   while (reps > 1 && (share + reps - 1) / reps * P < 256) reps /= 2;
@@ -473,7 +480,7 @@ static bool set_box_table(LatticeClass& c, int64_t replicas) {
 static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
   const int step = (c.split & (c.split - 1)) == 0 ? 32 / c.split * c.rp : 4 * c.rp;
   const int most = box_table(c) ? box_most(c, c.split, c.rp) : c.tpb / c.split * c.rp;
-  const int64_t resident = NUM_SMS * (c.tpb < 1024 && c.L < 8 ? 1024 / c.tpb : 1);
+  const int64_t resident = c.sms * (c.tpb < 1024 && c.L < 8 ? 1024 / c.tpb : 1);
   double sum = 0.0;
   for (int64_t r : R0) sum += (double)r;
   const double more = 1.0 + 3.0 / std::sqrt(std::max(1.0, sum));
@@ -520,8 +527,8 @@ void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone) 
   const int64_t per_block = c.tpb / c.split * c.rp;
   int64_t blocks = 0;
   for (int64_t r : R0) blocks += (r + (int64_t)(3.0 * std::sqrt((double)r)) + per_block - 1) / per_block;
-  const int64_t most = (blocks + NUM_SMS - 1) / NUM_SMS;
-  if (most < 2 || 10 * blocks < 9 * most * NUM_SMS) return;
+  const int64_t most = (blocks + c.sms - 1) / c.sms;
+  if (most < 2 || 10 * blocks < 9 * most * c.sms) return;
   c.min_smem = std::max<int>(0, (int)(SM_SMEM / (most + 1)) / 128 * 128 + 128 - BLOCK_RESERVED);
 }
 
@@ -562,8 +569,8 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   if (tpb_opt && tpb_supported(c, tpb_opt) && (tpb_opt < 512 || table)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
   else if (table) c.tpb = 1024;
-  else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * NUM_SMS ? 256 : 128;  // 5 threads a replica: 25 or 51 of
-                                                                                  // them a block
+  else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * c.sms ? 256 : 128;  // 5 threads a replica: 25 or 51 of
+                                                                               // them a block
   else if (c.split > 1) c.tpb = 128;
   else c.tpb = default_tpb(c.dim, c.L);
   if (c.tpb / c.split < 4 || (c.split > 1 && c.tpb < 64)) c.split = 1;
@@ -575,7 +582,7 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   // tables, not its threads, limit the blocks of an SM.  N = 4096, 5000
   // replicas, theta = 10: 394 us with one, 285 with two.)
   if (sweeps_pairs(c) && c.split > 1 &&
-      (replicas * c.split > (int64_t)900 * NUM_SMS || (gauss_chain(c) && c.Wr > 32)))
+      (replicas * c.split > (int64_t)900 * c.sms || (gauss_chain(c) && c.Wr > 32)))
     c.rp = 2;
   // The threshold-table kernel: from 600 threads an SM, from 400 where a word
   // holds few sites (L = 6, 10: 9, 10).  us of a launch with one and with two
@@ -584,7 +591,7 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   if (gauss_table(c)) {
     const int64_t from = c.L == 6 || c.L == 10 ? 400 : 600;
     if (!gtab_shape_ok(c.L, c.split, 1) ||
-        (gtab_shape_ok(c.L, c.split, 2) && replicas * c.split > from * NUM_SMS))
+        (gtab_shape_ok(c.L, c.split, 2) && replicas * c.split > from * c.sms))
       c.rp = 2;
   }
 }
@@ -939,7 +946,7 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
   int64_t largest = 0;
   for (const RunDev& d : E.h) largest = std::max(largest, d.R_cap);
   E.small = E.small && largest <= SMALL_RUN;
-  E.small_threads = largest <= 512 || n_runs > NUM_SMS ? 256 : 1024;
+  E.small_threads = largest <= 512 || n_runs > sm_count(E.device) ? 256 : 1024;
   E.n_copy_work = (int)ct.size();
   E.d_copy_table = (Work*)E.dalloc(sizeof(Work) * ct.size());
   if (!E.d_copy_table) return fail(PA_ERR_OOM, "work table allocation refused");
@@ -961,6 +968,7 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
       c.bz = gr.bz;
       c.bper = gr.bper;
       c.bsites = gr.bsites;
+      c.sms = sm_count(E.device);
       if (gr.bx > 0) {
         c.max_tpb = 32;
         for (int t = 256; t >= 32; t >>= 1)

@@ -156,6 +156,7 @@ struct LatticeClass {
   int bx = 0, by = 0, bz = 0, bsites = 0;  // general box (bx > 0)
   unsigned bper = 0;
   int max_tpb = 256;                        // largest block whose shared memory fits
+  int sms = 152;                            // multiprocessors of the device
   int tpb = 0;
   int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
   int rp = 1;        // +-1 lattices, chains, Gaussian threshold tables: replicas a thread sweeps side by side (1, 2)
@@ -314,6 +315,7 @@ size_t run_slab_bytes(const Geometry& g, int64_t cap, int max_steps);
 int setup_run(char* base, const Geometry& g, const pa_run_spec& s, int64_t cap, int max_steps,
               cudaStream_t st, RunDev* out);
 int default_tpb(int dim, int L);
+int sm_count(int device);
 void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0);
 void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone);
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c);

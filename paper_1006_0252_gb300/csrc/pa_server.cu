@@ -121,6 +121,7 @@ static int server_rebuild_tables(pa_server* S) {
       c.L = d.L;
       c.W = d.W;
       c.Wr = d.Wr;
+      c.sms = sm_count(S->device);
       S->cls.push_back(c);
       S->cls_buf.push_back(DevBuf());
       S->init_buf.push_back(DevBuf());

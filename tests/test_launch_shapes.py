@@ -21,6 +21,7 @@ int main(int n, char** a) {
   c.model = kind[0] == 'g';
   c.dim = kind.back() == 'c' ? 1 : 3;
   c.L = atoi(a[2]);
+  if (getenv("SMS")) c.sms = atoi(getenv("SMS"));
   c.Wr = (c.L + 31) / 32;
   c.W = (c.Wr + 3) / 4 * 4;
   std::vector<int64_t> R0;
@@ -45,8 +46,9 @@ def shape(tmp_path_factory):
                         "-rpath=" + where], capture_output=True, text=True)
     assert p.returncode == 0, p.stderr
 
-    def call(kind, size, *R0, alone=True):
-        out = subprocess.run([str(exe), kind, str(size), str(int(alone)), *map(str, R0)], capture_output=True, text=True)
+    def call(kind, size, *R0, alone=True, sms=NUM_SMS):
+        out = subprocess.run([str(exe), kind, str(size), str(int(alone)), *map(str, R0)], capture_output=True, text=True,
+                             env={**os.environ, "SMS": str(sms)})
         assert out.returncode == 0, out.stderr
         return dict(zip(("tpb", "split", "rp", "min_smem", "item"), map(int, out.stdout.split())))
 
@@ -56,6 +58,18 @@ def shape(tmp_path_factory):
 # (kind, size): pm / gpm cubic, c / gc chains.
 SPREAD = [("pm", 4), ("pm", 6), ("pm", 8), ("pm", 10), ("pm", 12), ("pm", 14), ("pm", 16), ("c", 256), ("c", 4096),
           ("gc", 256)]
+
+
+@pytest.mark.parametrize("sms", [132, 148, 152])
+def test_rules_follow_the_number_of_multiprocessors(shape, sms):
+    """As many replicas as fill sms blocks: one an SM, nothing to even out, on a
+    device that has that many; work items of the threshold tables fill one round."""
+    R0 = 16 * sms - 150
+    assert shape("pm", 8, R0, sms=sms)["min_smem"] == 0
+    assert shape("pm", 8, 2 * R0, sms=sms)["min_smem"] > 0
+    for R0 in range(900, 3000, 100):
+        item = shape("gpm", 8, R0, sms=sms)["item"]
+        assert -(-R0 // item) <= sms and (item <= 4 or -(-(R0 + 3 * R0 ** 0.5 + 1) // (item - 4)) > sms), (R0, item)
 
 
 def _blocks(sh, R0):
