@@ -512,7 +512,10 @@ static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
 // steps, theta = 10, ms without and with it, at 0.95-0.98 of most x SMs:
 // L = 8, 7000 replicas 2.66 / 2.30; L = 16, 7000 14.1 / 11.2; L = 10, 30000 15.4 /
 // 11.0; chain of 4096, 7000 11.6 / 9.3; Gaussian chain of 256, 9400 2.33 / 2.14.
-// Up to 0.9 of them, and with at most one block an SM, it changes nothing (90 sizes of
+// (Blocks of a capacity far above the population add to that, though they end at
+// once: from 0.7 of most x SMs, where the grid reaches most + 1 of them on every SM, 10-30 %;
+// L = 16, 2000 replicas 8.24 / 6.67.)
+// Elsewhere, above all with at most one block an SM, it changes nothing (90 sizes of
 // ten lattices), but would shut out the blocks of whatever else runs: eight
 // chains of 256 spins, 2000 replicas each, stepped from eight threads took 4.55 ms with it, 2.42
 // without, and the classes of one step are side by side on purpose (three chains
@@ -527,8 +530,10 @@ void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone) 
   const int64_t per_block = c.tpb / c.split * c.rp;
   int64_t blocks = 0;
   for (int64_t r : R0) blocks += (r + (int64_t)(3.0 * std::sqrt((double)r)) + per_block - 1) / per_block;
-  const int64_t most = (blocks + c.sms - 1) / c.sms;
-  if (most < 2 || 10 * blocks < 9 * most * c.sms) return;
+  const int64_t most = (blocks + c.sms - 1) / c.sms, grid = (c.capacity + per_block - 1) / per_block;
+  const bool full = most > 1 && 10 * blocks >= 9 * most * c.sms;
+  const bool spare = 10 * blocks >= 7 * most * c.sms && 10 * grid >= 9 * (most + 1) * c.sms;
+  if (!full && !spare) return;
   c.min_smem = std::max<int>(0, (int)(SM_SMEM / (most + 1)) / 128 * 128 + 128 - BLOCK_RESERVED);
 }
 
@@ -986,7 +991,10 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
   }
   for (auto& c : E.cls) {
     std::vector<int64_t> R0;
-    for (int32_t r : c.runs) R0.push_back(E.R0[r]);
+    for (int32_t r : c.runs) {
+      R0.push_back(E.R0[r]);
+      c.capacity += E.h[r].R_cap;
+    }
     set_default_launch(c, tpb_opt, split_opt, R0);
     spread_blocks(c, R0, E.cls.size() == 1);
     for (int64_t r : R0) c.shaped += r;

@@ -157,6 +157,7 @@ struct LatticeClass {
   unsigned bper = 0;
   int max_tpb = 256;                        // largest block whose shared memory fits
   int sms = 152;                            // multiprocessors of the device
+  int64_t capacity = 0;                     // slots of all its runs
   int tpb = 0;
   int split = 1;     // threads sharing a replica in the sweep kernel (1, 2, 4, 8; extra_split in pa_sweep3d.cuh)
   int rp = 1;        // +-1 lattices, chains, Gaussian threshold tables: replicas a thread sweeps side by side (1, 2)

@@ -132,7 +132,11 @@ static int server_rebuild_tables(pa_server* S) {
   for (size_t k = 0; k < S->cls.size(); ++k) {
     LatticeClass& c = S->cls[k];
     std::vector<int64_t> R0;
-    for (int32_t sl : c.runs) R0.push_back(S->h[sl].R);
+    c.capacity = 0;
+    for (int32_t sl : c.runs) {
+      R0.push_back(S->h[sl].R);
+      c.capacity += S->h[sl].R_cap;
+    }
     set_default_launch(c, S->tpb_opt, S->split_opt, R0);  // the shape follows the runs that are active
     spread_blocks(c, R0, used == 1);
     if (!c.runs.empty()) {

@@ -21,7 +21,8 @@ int main(int n, char** a) {
   c.model = kind[0] == 'g';
   c.dim = kind.back() == 'c' ? 1 : 3;
   c.L = atoi(a[2]);
-  if (getenv("SMS")) c.sms = atoi(getenv("SMS"));
+  c.sms = atoi(getenv("SMS"));
+  c.capacity = atoll(getenv("CAPACITY"));
   c.Wr = (c.L + 31) / 32;
   c.W = (c.Wr + 3) / 4 * 4;
   std::vector<int64_t> R0;
@@ -46,9 +47,9 @@ def shape(tmp_path_factory):
                         "-rpath=" + where], capture_output=True, text=True)
     assert p.returncode == 0, p.stderr
 
-    def call(kind, size, *R0, alone=True, sms=NUM_SMS):
+    def call(kind, size, *R0, alone=True, sms=NUM_SMS, capacity=0):
         out = subprocess.run([str(exe), kind, str(size), str(int(alone)), *map(str, R0)], capture_output=True, text=True,
-                             env={**os.environ, "SMS": str(sms)})
+                             env={**os.environ, "SMS": str(sms), "CAPACITY": str(capacity)})
         assert out.returncode == 0, out.stderr
         return dict(zip(("tpb", "split", "rp", "min_smem", "item"), map(int, out.stdout.split())))
 
@@ -97,6 +98,10 @@ def test_shared_memory_keeps_one_block_more_out(shape, kind, size):
         most = -(-blocks // NUM_SMS)
         if most > 1 and blocks >= 0.9 * most * NUM_SMS:
             held = sh["min_smem"] + BLOCK_RESERVED
+            assert most * held <= SM_SMEM < (most + 1) * held, (R0, sh)
+        # a capacity far above the population: from 0.7 of the places on
+        if blocks >= 0.7 * most * NUM_SMS:
+            held = shape(kind, size, R0, capacity=200 * R0)["min_smem"] + BLOCK_RESERVED
             assert most * held <= SM_SMEM < (most + 1) * held, (R0, sh)
         # classes of one step share the SMs
         assert shape(kind, size, R0, alone=False)["min_smem"] == 0
