@@ -1155,12 +1155,20 @@ cudaError_t launch_variance(int G, int M, const double* x, double* var, cudaStre
   return cudaGetLastError();
 }
 
-// A block of 256 threads a group where the groups leave SMs idle, a warp a
-// group else (and where a warp holds the group).
+// A block of 256 threads a group or a warp.  A block shortens the chain of a
+// thread but holds an SM's FP64 pipe with what its warps repeat (the folds, the
+// last logarithms), so the more groups an SM has, the longer they have to be for it;
+// terms: logarithms and exponentials of a group.  us, a warp / a block: 152 groups of 33
+// 14.7 / 12.6, of 1000 121 / 37; 304 of 64 14.5 / 16.7, of 100 22.8 / 18.8; 400 of 200 31.8 /
+// 33.0, of 400 53.5 / 49.4; 608 of 64 14.7 / 29.0, of 400 57.7 / 63.8, of 1000 135 / 129.
+static bool weighted_by_block(int G, int M, bool pairs) {
+  const int64_t terms = (int64_t)M * (pairs ? 2 : 1);
+  return M > 32 && (G <= 152 || (G <= 304 && terms >= 100) || (G <= 456 && terms >= 400) || (G <= 608 && terms >= 800));
+}
 template <bool PAIRS>
 static cudaError_t launch_weighted_t(int G, int M, const double* x1, const double* x2, const double* A,
                                      const double* R1, const double* R2, double* mean, double* fbar, cudaStream_t st) {
-  if (M > 32 && G <= 608) k_weighted<PAIRS, 256><<<G, 256, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
+  if (weighted_by_block(G, M, PAIRS)) k_weighted<PAIRS, 256><<<G, 256, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
   else k_weighted<PAIRS, 32><<<G, 32, 0, st>>>(M, x1, x2, A, R1, R2, mean, fbar);
   return cudaGetLastError();
 }
