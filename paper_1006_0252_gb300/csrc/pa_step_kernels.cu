@@ -1180,22 +1180,34 @@ cudaError_t launch_weighted_pairs(int G, int M, const double* x1, const double* 
                                   const double* R1, const double* R2, double* mean, double* fbar, cudaStream_t st) {
   return launch_weighted_t<true>(G, M, x1, x2, A, R1, R2, mean, fbar, st);
 }
+// A thread a resample, or eight.  Eight spread a few resamples over more SMs and
+// share a long one's draws, but leave lanes idle in resamples of fewer runs than
+// that and repeat their folds.  Up to three runs are summed directly: the table
+// saves less than its launch takes.  us of a call without population factors,
+// direct / table and eight threads / now: M = 2, B = 20000 104 / 130 / 106; M = 4, B = 20000
+// 108 / 128 / 105; M = 8, B = 1e5 402 / 461 / 342; a batch's 1600 groups of M = 1, B = 1000
+// 640 / 2156 / 622, its 4000 of M = 8 6759 / 5360 / 1067.
+template <int LANES>
+static void bootstrap_lanes(int M, const double* x, const double* A, const double* Rw, const double* tab, int B,
+                            uint64_t seed, int GK, double* bmean, double* bfbar, cudaStream_t st) {
+  constexpr unsigned PER_BLOCK = 128 / LANES;
+  const dim3 grid(((unsigned)B + PER_BLOCK - 1) / PER_BLOCK, (unsigned)std::min(GK, 65535));
+  k_bootstrap<LANES><<<grid, 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
+}
 cudaError_t launch_bootstrap(int M, const double* x, const double* A, const double* Rw, int B, uint64_t seed,
                              double* bmean, double* bfbar, double* tab, cudaStream_t st, int GK) {
-  const unsigned groups = (unsigned)std::min(GK, 65535);
-  if (!tab) {
-    k_bootstrap<1><<<dim3(((unsigned)B + 127) / 128, groups), 128, 0, st>>>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar);
-    return cudaGetLastError();
+  if (M <= 3) tab = nullptr;
+  if (tab) {
+    if (A && Rw) k_boot_weights<true, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+    else if (A) k_boot_weights<true, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+    else if (Rw) k_boot_weights<false, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+    else k_boot_weights<false, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
   }
-  if (A && Rw) k_boot_weights<true, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
-  else if (A) k_boot_weights<true, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
-  else if (Rw) k_boot_weights<false, true><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
-  else k_boot_weights<false, false><<<GK, BOOT_WEIGHT_THREADS, 0, st>>>(M, x, A, Rw, tab);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  constexpr int LANES = 8, PER_BLOCK = 128 / LANES;
-  k_bootstrap<LANES><<<dim3(((unsigned)B + PER_BLOCK - 1) / PER_BLOCK, groups), 128, 0, st>>>(M, x, A, Rw, tab, B,
-                                                                                              seed, GK, bmean, bfbar);
+  const bool shared = tab && (M >= 16 || (M >= 8 && (int64_t)GK * B <= 4096));
+  if (shared) bootstrap_lanes<8>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar, st);
+  else bootstrap_lanes<1>(M, x, A, Rw, tab, B, seed, GK, bmean, bfbar, st);
   return cudaGetLastError();
 }
 
