@@ -120,12 +120,21 @@ __device__ __forceinline__ void measure_box(RunDev& R, int nxt, int64_t slot, bo
   }
 }
 
-template <int TPB>
-__global__ void __launch_bounds__(TPB) k_sweep_box(RunDev* __restrict__ runs, const Work* __restrict__ table,
-                                                   int init, int slots) {
+// INIT: the initial state of work items of `slots` slots; a sweep's items are a
+// block's threads.
+//
+// One block an SM in the bounds: without it the compiler stays at 48 registers and
+// keeps values of the site loop in local memory, and with 80 shared memory limits the
+// blocks of an SM all the same.  16 x 16 x 8, 5000 replicas, 6 steps of theta = 10: 43.3 -> 30.1
+// ms (38.9 before the blocks of an item, which moved the spills); 8 x 6 x 5 in blocks of 64,
+// 1e5 replicas 12.0 -> 9.5.
+template <int TPB, bool INIT>
+__global__ void __launch_bounds__(TPB, 1) k_sweep_box(RunDev* __restrict__ runs, const Work* __restrict__ table,
+                                                   int slots) {
   extern __shared__ uint32_t smem[];
-  const int per = (slots + TPB - 1) / TPB;  // blocks of a work item
-  const int at = (int)(blockIdx.x % per) * TPB + threadIdx.x;
+  constexpr bool init = INIT;
+  const int per = INIT ? (slots + TPB - 1) / TPB : 1;  // blocks of a work item
+  const int at = (INIT ? (int)(blockIdx.x % per) * TPB : 0) + threadIdx.x;
   const Work wk = table[blockIdx.x / per];
   RunDev& R = runs[wk.run];
   if (!init && R.skip) return;
@@ -144,7 +153,7 @@ __global__ void __launch_bounds__(TPB) k_sweep_box(RunDev* __restrict__ runs, co
   for (int i = tid; i < 2 * plane; i += TPB) s_S[i] = R.gS[i];
   if (tid < 8) s_thr[tid] = R.thr[tid];
   const int64_t slot = (int64_t)wk.first + at;
-  const bool live = at < slots && slot < Rn;
+  const bool live = (!INIT || at < slots) && slot < Rn;
   const int cur = R.cur, nxt = init ? 0 : cur ^ 1;
   uint32_t* col = s_spin + tid;
   const uint32_t valid = R.bvalid;
@@ -206,27 +215,34 @@ size_t box_smem_bytes(int WR, int S, int tpb) {
   return sizeof(int32_t) * (28 * (size_t)WR * S + (size_t)WR * tpb);
 }
 
-template <int TPB>
-static cudaError_t launch_box_t(int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
-                                bool init) {
+template <int TPB, bool INIT>
+static cudaError_t launch_box_t(int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st) {
   const size_t sm = box_smem_bytes(WR, S, TPB);
-  if (sm > SMEM_LIMIT) return nwork > 0 ? cudaErrorInvalidValue : cudaSuccess;
+  if (sm > SMEM_LIMIT || (!INIT && slots != TPB)) return nwork > 0 ? cudaErrorInvalidValue : cudaSuccess;
   if (sm > 48 * 1024) {
-    cudaError_t e = allow_shared(k_sweep_box<TPB>);
+    cudaError_t e = allow_shared(k_sweep_box<TPB, INIT>);
     if (e != cudaSuccess) return e;
   }
   if (nwork <= 0) return cudaSuccess;
-  k_sweep_box<TPB><<<nwork * ((slots + TPB - 1) / TPB), TPB, sm, st>>>(runs, table, init ? 1 : 0, slots);
+  k_sweep_box<TPB, INIT><<<nwork * ((slots + TPB - 1) / TPB), TPB, sm, st>>>(runs, table, slots);
   return cudaGetLastError();
 }
 
 cudaError_t launch_box(int tpb, int slots, RunDev* runs, const Work* table, int nwork, int WR, int S, cudaStream_t st,
                        bool init) {
   switch (tpb) {
-    case 32: return launch_box_t<32>(slots, runs, table, nwork, WR, S, st, init);
-    case 64: return launch_box_t<64>(slots, runs, table, nwork, WR, S, st, init);
-    case 128: return launch_box_t<128>(slots, runs, table, nwork, WR, S, st, init);
-    case 256: return launch_box_t<256>(slots, runs, table, nwork, WR, S, st, init);
+    case 32:
+      return init ? launch_box_t<32, true>(slots, runs, table, nwork, WR, S, st)
+                  : launch_box_t<32, false>(slots, runs, table, nwork, WR, S, st);
+    case 64:
+      return init ? launch_box_t<64, true>(slots, runs, table, nwork, WR, S, st)
+                  : launch_box_t<64, false>(slots, runs, table, nwork, WR, S, st);
+    case 128:
+      return init ? launch_box_t<128, true>(slots, runs, table, nwork, WR, S, st)
+                  : launch_box_t<128, false>(slots, runs, table, nwork, WR, S, st);
+    case 256:
+      return init ? launch_box_t<256, true>(slots, runs, table, nwork, WR, S, st)
+                  : launch_box_t<256, false>(slots, runs, table, nwork, WR, S, st);
     default: return cudaErrorInvalidValue;
   }
 }
