@@ -458,7 +458,12 @@ static int box_most(const LatticeClass& c, int P, int reps) {
 // launch for (split, replicas), while uniforms of 0 were looked for site by site:
 // (16, 4) 109, (32, 4) 120, (8, 4) 134, (16, 2) 137, (16, 1) 169; 1000 replicas (32, 2) 29, (16, 1) 31, (16, 4) 47; 6 x 6 x 7,
 // 3000 replicas (16, 1) 64, (16, 2) 70, (8, 1) 87, (16, 4) 110.
+// Boxes of up to four sites take the site-at-a-time kernel unless the population
+// fills the chip: a step of theta = 10 takes less than a block's tables.  2 x 1 x 1, 12 steps,
+// us there / here: 300 replicas 300 / 411, 5000 421 / 496, 17000 510 / 509, 1e5 1204 / 644; 2 x 2 x 1
+// 5000 497 / 559, 1e5 916 / 719; 4 x 2 x 1 5000 594 / 547.
 static bool set_box_table(LatticeClass& c, int64_t replicas) {
+  if (c.bx * c.by * c.bz <= 4 && replicas < 20000) return false;
   const int U = box_period(c.bsites), groups = (c.Wr + U - 1) / U;
   const int64_t share = (replicas + c.sms - 1) / c.sms;
   int P = 1, reps = box_replicas(c.bsites);

@@ -291,3 +291,19 @@ def test_many_small_runs_take_no_longer():
         return min(times)
 
     assert seconds(2048) <= 1.05 * seconds(2049)
+
+
+# Boxes of up to four sites: site at a time in small populations.
+@pytest.mark.parametrize("Lx,Ly,Lz,R0,tpb", [(2, 1, 1, 5000, 64), (2, 2, 1, 19999, 64), (2, 2, 1, 20000, 1024),
+                                             (4, 2, 1, 5000, 1024)])
+@pytest.mark.parametrize("gaussian", [False, True])
+def test_tiny_box_shape_bit_exact(Lx, Ly, Lz, R0, tpb, gaussian):
+    J = inputs.gaussian_couplings_lattice(Lx, Ly, Lz, 6) if gaussian else inputs.couplings_lattice(Lx, Ly, Lz, 6, 3)
+    g = pa.Run(J, Lx, 3, R0, 41, R_cap=R0 + 4000, gaussian=gaussian, Ls=(Lx, Ly, Lz), periodic_mask=0)
+    assert pa.pa_sweep_shape(g._h)[0] == tpb
+    c = (o.GaussRun if gaussian else o.Run)(J, 3, Lx, Ly, Lz, 0, R0=R0, R_cap=R0 + 4000, seed=41)
+    for beta, sweeps in ((0.4, 1), (1.5, 2)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.spins(), c.spins())
