@@ -294,11 +294,11 @@ __global__ void __launch_bounds__(TPB) k_sweep_gauss1d(RunDev* __restrict__ runs
   for (int h0 = 0; h0 < nhalf; h0 += sh.NH) {
     if (h0 > 0) __syncthreads();  // the previous chunk's tables are no longer read
     const int nh = min(sh.NH, nhalf - h0);
-    for (int j = 0; j < nh; ++j) {
-      const uint32_t A1 = PHILOX_MUL1 * (T0 + (uint32_t)((h0 + j) >> 1));
-      for (int q = tid; q < Q; q += TPB)
-        s_tab[j * GCHAIN_CALLS * WR + GCHAIN_CALLS * (q >> 2) + (q & 3)] =
-            sweep_half_entry(sweep_call_entry((uint32_t)q, TAG_SWEEP + (uint32_t)(j & 1), rk), A1);
+    for (int i = tid; i < nh * Q; i += TPB) {
+      const int j = i / Q, q = i - j * Q;
+      s_tab[j * GCHAIN_CALLS * WR + GCHAIN_CALLS * (q >> 2) + (q & 3)] =
+          sweep_half_entry(sweep_call_entry((uint32_t)q, TAG_SWEEP + (uint32_t)(j & 1), rk),
+                           PHILOX_MUL1 * (T0 + (uint32_t)((h0 + j) >> 1)));
     }
     __syncthreads();
 #pragma unroll 1

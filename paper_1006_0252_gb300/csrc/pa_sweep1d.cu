@@ -295,7 +295,13 @@ __global__ void __launch_bounds__(TPB) k_sweep1d(RunDev* __restrict__ runs, cons
     for (int h0 = 0; h0 < nhalf; h0 += sh.NH) {
       if (h0 > 0) __syncthreads();  // the previous chunk's tables are no longer read
       const int nh = min(sh.NH, nhalf - h0);
-      for (int j = 0; j < nh; ++j) build(s_tab + j * sh.Q, j & 1, T0 + (uint32_t)((h0 + j) >> 1));
+      // over all entries at once: table by table, a chain of one word (four
+      // calls) left most threads idle for the length of the chunk
+      for (int i = tid; i < nh * sh.Q; i += TPB) {
+        const int j = i / sh.Q, q = i - j * sh.Q;
+        s_tab[i] = sweep_half_entry(sweep_call_entry((uint32_t)q, TAG_SWEEP + (uint32_t)(j & 1), rk),
+                                    PHILOX_MUL1 * (T0 + (uint32_t)((h0 + j) >> 1)));
+      }
       __syncthreads();
       if (live) {
 #pragma unroll 1
