@@ -439,6 +439,29 @@ static int pm_split(int L, int64_t replicas) {
   }
 }
 
+// Threads per replica of a chain: the finest split of its words (at most 8, of
+// one word a thread at least) spreads a small population, but ranges of ceil(words / P)
+// words leave threads idle where P does not divide the words (9 words of 8 threads: 16
+// places).  So from 460 threads an SM on, the split of the least places, each of
+// which takes a little longer in a coarser one.  (Gaussian chains of more than 32 words,
+// whose tables limit the blocks of an SM, from 2000: N = 1100, 20000 replicas 2948 at 8, 3181 at 4,
+// 100000 10313 / 9737.)  100000 replicas, theta = 10, 12 steps, us, at
+// 8 / 4 / 2 / 1 threads: N = 260 4058 / 3245 / 2974 / 2836, N = 352 4091 / 3255 / 3515 / 3382, N = 520
+// 5850 / 5111 / 5040 / 4991; 20000 replicas N = 260 1289 / 1122 / 1150 / 1285.
+static int chain_split(const LatticeClass& c, int finest, int64_t replicas) {
+  const auto cost = [&](int P) {
+    // us per place and replica, 8 threads 1; +-1 and Gaussian couplings
+    static const double pm[4] = {1.20, 1.15, 1.06, 1.0}, gauss[4] = {1.30, 1.10, 1.0, 1.0};
+    const int k = P == 1 ? 0 : (P == 2 ? 1 : (P == 4 ? 2 : 3));
+    return (double)((c.Wr + P - 1) / P * P) * (c.model == 1 ? gauss[k] : pm[k]);
+  };
+  const int64_t least = (c.model == 1 && c.Wr > 32 ? 2000 : 460) * (int64_t)c.sms;
+  int best = finest;
+  for (int P = finest / 2; P >= 1 && replicas * P >= least; P /= 2)
+    if (cost(P) < 0.95 * cost(best)) best = P;
+  return best;
+}
+
 // General boxes on their threshold-table kernel (blocks of BOX_TPB threads), and
 // the most slots a block of it takes: as many columns as it has threads for and
 // as fit shared memory, in whole warps (0: none fit).
@@ -569,9 +592,9 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
     // +-1 chains: the word ranges keep the uniform tables and the columns of
     // a block within shared memory at long chains (8 rather than 4 ranges of
     // 8 words: 25 against 33 us at 2000 replicas of 256 spins, 3 % at 20000)
-    c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : 1);
+    c.split = chain_split(c, c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : 1), replicas);
   } else if (gauss_chain(c) && tpb_opt == 0) {
-    c.split = c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : (c.Wr >= 2 ? 2 : 1));
+    c.split = chain_split(c, c.Wr >= 8 ? 8 : (c.Wr >= 4 ? 4 : (c.Wr >= 2 ? 2 : 1)), replicas);
   }
   // The blocks of 512 and 1024 threads of the threshold-table kernel, where it has a
   // shape with the split asked for (not for L = 10 with one thread a replica).
@@ -1527,7 +1550,7 @@ int pa_step_target(pa_run* run, double beta_next, int sweeps, int64_t R_target) 
   if (!(beta_next >= run->e.host_beta[0]) || !std::isfinite(beta_next))
     return fail(PA_ERR_INVALID, "beta must not decrease (%g after %g)", beta_next, run->e.host_beta[0]);
   PA_CUDA(cudaSetDevice(run->e.device));
-  int st = refit_classes(run->e, {R_target});
+  int st = R_target > run->e.most[0] ? refit_classes(run->e, {R_target}) : PA_OK;
   if (st == PA_OK) st = engine_step(run->e, true, beta_next, sweeps, R_target);
   if (st != PA_OK) return st;
   run->e.host_beta[0] = beta_next;

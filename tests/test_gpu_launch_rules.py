@@ -307,3 +307,32 @@ def test_tiny_box_shape_bit_exact(Lx, Ly, Lz, R0, tpb, gaussian):
         c.step(beta, sweeps, R0)
     assert g.observables()["sumE"] == c.state().sumE
     assert np.array_equal(g.spins(), c.spins())
+
+
+# Chains whose words the finest split leaves places idle for: coarser splits in large
+# populations (the last range short, one and two replicas a thread).
+@pytest.mark.parametrize("N,R0,split", [(130, 20000, 4), (130, 80001, 1), (190, 70001, 2), (260, 17400, 8),
+                                        (260, 17501, 4), (260, 70001, 1), (340, 36001, 4)])
+def test_coarser_chain_split_bit_exact(N, R0, split):
+    J = inputs.couplings_chain(N, 2, 9, open_chain=True)
+    J[N // 3] = 0
+    g, c = pa.Run(J, N, 1, R0, 59), o.Run(J, 1, N, R0=R0, seed=59)
+    assert pa.pa_sweep_shape(g._h)[1] == split
+    for beta, sweeps in ((0.1, 1), (1.5, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.spins(), c.spins())
+
+
+@pytest.mark.parametrize("N,R0,split", [(96, 18001, 2), (96, 70001, 1), (130, 40001, 2), (260, 18001, 4),
+                                        (260, 40001, 2), (1100, 17501, 8), (1100, 76001, 4)])
+def test_coarser_gauss_chain_split_bit_exact(N, R0, split):
+    J = inputs.gaussian_couplings_chain(N, 2, 9, open_chain=False)
+    g, c = pa.Run(J, N, 1, R0, 59, gaussian=True), o.GaussRun(J, 1, N, R0=R0, seed=59)
+    assert pa.pa_sweep_shape(g._h)[1] == split
+    for beta, sweeps in ((0.1, 1), (1.5, 1)):
+        g.step(beta, sweeps)
+        c.step(beta, sweeps, R0)
+    assert g.observables()["sumE"] == c.state().sumE
+    assert np.array_equal(g.spins(), c.spins())

@@ -113,3 +113,13 @@ def test_shared_memory_keeps_one_block_more_out(shape, kind, size):
 def test_bootstrap_resample_of_a_thread(shape, block):
     for thread in (0, 1):
         assert shape("resample", block, alone=thread)["tpb"] == 16 * block
+
+
+# Chains: the words' places of the split that a large population gets are within a
+# quarter of the words (the finest split of 9 words has 16).
+@pytest.mark.parametrize("kind", ["c", "gc"])
+def test_chain_splits_leave_few_places_idle(shape, kind):
+    for words in range(5, 60):
+        sh = shape(kind, 32 * words, 300000)
+        places = -(-words // sh["split"]) * sh["split"]
+        assert places <= 1.25 * words, (words, sh)
