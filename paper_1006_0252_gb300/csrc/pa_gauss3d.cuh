@@ -361,7 +361,10 @@ __global__ void __launch_bounds__(TPB) k_sweep_gauss3d(RunDev* __restrict__ runs
 }
 
 // Sec. 2: R0 independent uniformly random microstates at beta = 0 (keying as
-// k_init3d) and their fixed-point energies; one thread per slot of a work item.
+// k_init3d) and their fixed-point energies, one thread per slot.  The blocks are
+// those of the class table, but the i-th of a run takes the i-th TPB slots whatever a
+// work item holds: items of a few slots would have every block read the couplings
+// for a few replicas (L = 10, 300 replicas 72 us a reset, 46 so).
 template <int L, int TPB>
 __global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs, const Work* __restrict__ table,
                                                       int slots) {
@@ -373,12 +376,12 @@ __global__ void __launch_bounds__(TPB) k_init_gauss3d(RunDev* __restrict__ runs,
   uint32_t* s_spin = smem + gauss_tables_words<L>();
   const Work wk = table[blockIdx.x];
   RunDev& R = runs[wk.run];
-  const int64_t R0 = R.R;
-  if ((int64_t)wk.first >= R0) return;
+  const int64_t R0 = R.R, first = (int64_t)(wk.first / slots) * TPB;
+  if (first >= R0) return;
   const int tid = threadIdx.x;
   for (int i = tid; i < NJ; i += TPB) s_J[i] = R.gJ[i];
-  const int64_t slot = (int64_t)wk.first + tid;
-  const bool live = tid < slots && slot < R0;
+  const int64_t slot = first + tid;
+  const bool live = slot < R0;
   uint32_t* col = s_spin + tid;
   if (live) {
     for (int w4 = 0; w4 < W / 4; ++w4) {
@@ -427,11 +430,13 @@ cudaError_t launch_gauss3d_init(const Sweep3dLaunch& a) {
   return cudaGetLastError();
 }
 
-// The initial state in blocks of the smallest size that holds a work item.
+// The initial state in blocks of at least a work item's slots, of 128 threads or
+// more where the populations choose the items (threshold tables).
 template <int L>
 cudaError_t launch_gauss3d_init_any(const Sweep3dLaunch& a) {
-  if (a.slots <= 32) return launch_gauss3d_init<L, 32>(a);
-  if (a.slots <= 64) return launch_gauss3d_init<L, 64>(a);
+  const bool table = a.tpb >= 512;
+  if (a.slots <= 32 && !table) return launch_gauss3d_init<L, 32>(a);
+  if (a.slots <= 64 && !table) return launch_gauss3d_init<L, 64>(a);
   if (a.slots <= 128) return launch_gauss3d_init<L, 128>(a);
   if (a.slots <= 256) return launch_gauss3d_init<L, 256>(a);
   if constexpr (L <= 10) {
