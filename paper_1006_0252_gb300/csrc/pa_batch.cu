@@ -310,7 +310,7 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
       trial.tpb = cand.tpb;
       trial.split = cand.split;
       trial.rp = cand.rp;
-      spread_blocks(trial, R0, E.cls.size() == 1);
+      spread_blocks(trial, R0, spreads_alone(E.cls));
       trial.d_table = nullptr;
       int st = prepare_class_launch(E.d_runs, E.st, trial);
       if (st == PA_OK) st = build_class_table(E, trial);
@@ -339,7 +339,7 @@ int pa_batch_autotune(pa_batch* b, int32_t sweeps, int32_t* host_L, int32_t* hos
       c.tpb = pick.tpb;
       c.split = pick.split;
       c.rp = pick.rp;
-      spread_blocks(c, R0, E.cls.size() == 1);
+      spread_blocks(c, R0, spreads_alone(E.cls));
       int st = build_class_table(E, c);
       if (st != PA_OK) return st;
     }

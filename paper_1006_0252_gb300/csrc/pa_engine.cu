@@ -530,8 +530,14 @@ static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
   return best;
 }
 
+// Whether at most one of the classes of a step has blocks to spread: those of the
+// threshold tables hold an SM each, whatever the others ask for.
+bool spreads_alone(const std::vector<LatticeClass>& cls) {
+  return std::count_if(cls.begin(), cls.end(), sweeps_pairs) <= 1;
+}
+
 // Share of a work item (table_item), and the shared memory that keeps a launch's
-// blocks even over the SMs; alone: no other class is swept side by side.
+// blocks even over the SMs; alone: no other class to spread is swept side by side.
 //
 // While a launch's blocks fit the SMs at once, the SM that gets the most of
 // them sets its time, and where they nearly fill `most` of them on every SM the
@@ -540,14 +546,15 @@ static int table_item(const LatticeClass& c, const std::vector<int64_t>& R0) {
 // steps, theta = 10, ms without and with it, at 0.95-0.98 of most x SMs:
 // L = 8, 7000 replicas 2.66 / 2.30; L = 16, 7000 14.1 / 11.2; L = 10, 30000 15.4 /
 // 11.0; chain of 4096, 7000 11.6 / 9.3; Gaussian chain of 256, 9400 2.33 / 2.14.
-// (Blocks of a capacity far above the population add to that, though they end at
-// once: from 0.7 of most x SMs, where the grid reaches most + 1 of them on every SM, 10-30 %;
-// L = 16, 2000 replicas 8.24 / 6.67.)
+// The blocks of unused capacity add to that, though they end at once: from 0.7 of
+// most x SMs, where the grid reaches most + 1 of them on every SM (a capacity far above
+// the population: L = 16, 2000 replicas 8.24 / 6.67), or, with several runs, whose unused blocks lie
+// between the others, nearly most (12 steps of 7 runs of 500 replicas, L = 16, 3.03 / 2.32).
 // Elsewhere, above all with at most one block an SM, it changes nothing (90 sizes of
 // ten lattices), but would shut out the blocks of whatever else runs: eight
 // chains of 256 spins, 2000 replicas each, stepped from eight threads took 4.55 ms with it, 2.42
-// without, and the classes of one step are side by side on purpose (three chains
-// of 2000 replicas 3.41 / 2.59).
+// without, and the classes of one step are side by side on purpose (three chains of 2000
+// replicas in a batch 3.41 / 2.59, seven runs of L = 4 to 10 2.13 / 1.51).
 // (The population stays within three standard deviations, sqrt(R0), of its
 // target; a larger one only takes longer.)
 void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone) {
@@ -560,7 +567,8 @@ void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone) 
   for (int64_t r : R0) blocks += (r + (int64_t)(3.0 * std::sqrt((double)r)) + per_block - 1) / per_block;
   const int64_t most = (blocks + c.sms - 1) / c.sms, grid = (c.capacity + per_block - 1) / per_block;
   const bool full = most > 1 && 10 * blocks >= 9 * most * c.sms;
-  const bool spare = 10 * blocks >= 7 * most * c.sms && 10 * grid >= 9 * (most + 1) * c.sms;
+  const int64_t places = (R0.size() > 1 && (most > 1 || grid > c.sms) ? most : most + 1) * c.sms;
+  const bool spare = 10 * blocks >= 7 * most * c.sms && 10 * grid >= 9 * places;
   if (!full && !spare) return;
   c.min_smem = std::max<int>(0, (int)(SM_SMEM / (most + 1)) / 128 * 128 + 128 - BLOCK_RESERVED);
 }
@@ -854,7 +862,7 @@ static int refit_classes(Engine& E, const std::vector<int64_t>& targets) {
   PA_CUDA(cudaStreamIsCapturing(E.st, &capture));
   if (capture != cudaStreamCaptureStatusNone) return PA_OK;
   for (int r = 0; r < E.n; ++r) E.most[r] = std::max(E.most[r], target(r));
-  const bool alone = E.cls.size() == 1;
+  const bool alone = spreads_alone(E.cls);
   for (auto& c : E.cls) {
     std::vector<int64_t> R;
     int64_t sum = 0;
@@ -1024,7 +1032,7 @@ int engine_create(Engine& E, int n_runs, const pa_run_spec* specs, const pa_opts
       c.capacity += E.h[r].R_cap;
     }
     set_default_launch(c, tpb_opt, split_opt, R0);
-    spread_blocks(c, R0, E.cls.size() == 1);
+    spread_blocks(c, R0, spreads_alone(E.cls));
     for (int64_t r : R0) c.shaped += r;
     c.spread = c.shaped;
     if (split_opt > 1 && c.split != split_opt)

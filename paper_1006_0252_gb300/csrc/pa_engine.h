@@ -318,6 +318,7 @@ int setup_run(char* base, const Geometry& g, const pa_run_spec& s, int64_t cap, 
 int default_tpb(int dim, int L);
 int sm_count(int device);
 void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::vector<int64_t>& R0);
+bool spreads_alone(const std::vector<LatticeClass>& cls);
 void spread_blocks(LatticeClass& c, const std::vector<int64_t>& R0, bool alone);
 std::vector<LaunchShape> launch_shapes(const LatticeClass& c);
 bool split_supported(const LatticeClass& c, int split);

@@ -104,7 +104,7 @@ def test_shared_memory_keeps_one_block_more_out(shape, kind, size):
             held = shape(kind, size, R0, capacity=200 * R0)["min_smem"] + BLOCK_RESERVED
             assert most * held <= SM_SMEM < (most + 1) * held, (R0, sh)
         # classes of one step share the SMs
-        assert shape(kind, size, R0, alone=False)["min_smem"] == 0
+        assert shape(kind, size, R0, alone=False, capacity=200 * R0)["min_smem"] == 0
 
 
 # Eight threads a resample, so a block of 128 threads takes 16: the thread's
@@ -123,3 +123,10 @@ def test_chain_splits_leave_few_places_idle(shape, kind):
         sh = shape(kind, 32 * words, 300000)
         places = -(-words // sh["split"]) * sh["split"]
         assert places <= 1.25 * words, (words, sh)
+
+
+# Several runs: the blocks of their unused capacity lie between the others.
+def test_unused_capacity_between_runs_is_spread(shape):
+    sh = shape("pm", 16, *[500] * 7, capacity=7 * 794)
+    assert 2 * (sh["min_smem"] + BLOCK_RESERVED) <= SM_SMEM < 3 * (sh["min_smem"] + BLOCK_RESERVED)
+    assert shape("pm", 16, 3500, capacity=4156)["min_smem"] == 0
