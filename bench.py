@@ -346,6 +346,7 @@ def main():
 
     value = flips_all / (gpu_ms_max / 1000.0)
     shape = pa.pa_sweep_shape(run._h)  # (threads per block, threads per replica)
+    pair = 2 if spec.R0 * shape[1] > 900 * 152 else 1  # replicas per thread, the library's own rule
     peaks = measured_peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     alu_peak = 152 * 128 * sm_max * 1e6 / 1e12  # int32 lane ops/s, TOP/s
@@ -364,7 +365,7 @@ def main():
                    "spins": "bit-packed, 32-bit words", "l2": "flushed between timed runs (256 MB write)",
                    "parallelism": "replicas only" if ws > 1 else "single GPU"},
         "wall_s": wall,
-        "roofline": {"bound": "alu", "kernel": f"k_sweep3d<8,{shape[0]},{shape[1]}>", "achieved": achieved,
+        "roofline": {"bound": "alu", "kernel": f"k_sweep3d<8,{shape[0]},{shape[1]},{pair}>", "achieved": achieved,
                      "peak": alu_peak,
                      "unit": "TOP/s", "frac": achieved / alu_peak, "traffic": sweep_traffic(),
                      "ops_per_flip": OPS_PER_FLIP, "launch_ms": per_launch_ms,

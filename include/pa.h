@@ -240,7 +240,9 @@ int pa_sweep_shape(pa_run* run, int32_t* threads_per_block, int32_t* threads_per
  * sweeps >= 0.  Asynchronous. */
 int pa_step(pa_run* run, double beta_next, int sweeps);
 /* pa_step with an explicit population target R_beta' (Sec. 4 varies it with
- * temperature: R = 1000 below beta = 0.9 and 3000 above).  R_target >= 1. */
+ * temperature: R = 1000 below beta = 0.9 and 3000 above).  R_target >= 1.  The
+ * launch shapes follow the largest target so far: a call that raises it may
+ * wait for the stream once (also in the schedule calls). */
 int pa_step_target(pa_run* run, double beta_next, int sweeps, int64_t R_target);
 /* The next n_steps steps of the Algorithm at once: step k goes to
  * betas[k] with thetas[k] sweeps (NULL: 10 each) and population target
@@ -456,10 +458,12 @@ int pa_batch_overlap_hist(pa_batch* b, int n_pairs, const int32_t* run_a, const 
  * candidates on the batch's own populations at the current temperature (a
  * dry step of min(sweeps, 20) Metropolis sweeps, sweeps <= 0 meaning 10: pass
  * the schedule's sweeps per step, since a block's fixed cost weighs less the
- * more sweeps it runs; no state is committed): the block size, and for +-1 cubic
- * lattices the threads per replica (1, 2, 4 or 8 threads sweeping disjoint
- * ranges of whole rows; 1, 2 or 4 for Gaussian ones, whose candidates include
- * blocks of 512 and 1024 threads at L <= 10).  The bit packing of the lattice is not a candidate:
+ * more sweeps it runs; no state is committed): the block size, the threads
+ * sharing a replica's sweep (ranges of whole rows of a cubic lattice: 1, 2, 4 or 8
+ * and, where its rows divide so, 3, 5, 6, 7 or 12; ranges of words of a chain: 1, 2, 4 or
+ * 8; of a general box: powers of two up to 32) and the replicas a thread sweeps side
+ * by side (1 or 2, up to 4 in boxes).  Gaussian cubic lattices of L <= 10 and boxes include
+ * blocks of 512 and 1024 threads with threshold tables.  The bit packing of the lattice is not a candidate:
  * it is part of the random keying (a site's uniform is keyed by its word and
  * bit), so another packing would draw other random numbers.  Writes up to 8
  * (L, threads per block, threads per replica) triples (L < 0 for chains; any

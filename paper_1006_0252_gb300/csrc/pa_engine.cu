@@ -6,9 +6,10 @@
 // An Engine owns a set of annealing runs on one GPU: one device-memory slab
 // per run, the RunDev array, and the work tables that map kernel blocks to
 // (run, slot range).  Single runs (pa_run) and batches (pa_batch) are both
-// Engines; every step enqueues the same seven launches (prepare, copies,
-// scan, scatter, one sweep launch per lattice class, commit) with no host
-// synchronisation, so a batch schedule can be captured as one CUDA graph.
+// Engines; every step enqueues the same launches (prepare, copies, scan,
+// scatter, one sweep launch per lattice class, commit; small +-1 runs resample
+// in one launch, which in a schedule also commits the step before) with no
+// host synchronisation, so a batch schedule can be captured as one CUDA graph.
 #include "pa_engine.h"
 
 

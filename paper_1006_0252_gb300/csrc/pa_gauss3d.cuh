@@ -164,7 +164,7 @@ __device__ __forceinline__ void grow3d(uint32_t* __restrict__ col, const int32_t
 // couplings (four ranks per 128-bit load) and the branch-free windowed
 // decision; sites inside the window are settled by gauss_resolve under a
 // warp-uniform branch.  Rows go in pairs when the colour-c sites per word are
-// not a multiple of 4 (see row3d in pa_sweep3d.cuh).
+// not a multiple of 4, since a generator call then serves two rows.
 template <class GEO, int CS, int RPP>
 __device__ __forceinline__ void half_sweep_gauss3d(uint32_t* __restrict__ col, const int32_t* __restrict__ s_J,
                                                    const int32_t* __restrict__ s_S, const GaussHalf& gh,
@@ -314,9 +314,9 @@ __global__ void __launch_bounds__(TPB) k_sweep_gauss3d(RunDev* __restrict__ runs
   const int theta = R.theta_next;
   const uint32_t T0 = (uint32_t)R.sweeps;
   const int y0 = part * RPP;
-  // half sweeps in chunks of NH tables, ordered as in k_sweep3d: block
-  // barriers around each chunk's tables, a warp barrier between the half
-  // sweeps of a replica's P threads within a chunk
+  // half sweeps in chunks of NH tables: block barriers around each chunk's
+  // tables, a warp barrier between the half sweeps of a replica's P threads
+  // within a chunk
   const int nhalf = 2 * theta;
 #pragma unroll 1
   for (int h0 = 0; h0 < nhalf; h0 += SH::NH) {

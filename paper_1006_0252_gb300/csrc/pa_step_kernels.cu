@@ -3,16 +3,24 @@
 // overlap (Sec. 4) and weighted-average (Sec. 3) kernels.
 //
 // Step pipeline for a set of runs (all state on the device):
-//   k_prepare  one warp per run: energy histogram -> Q' over the fixed
+//   k_prepare  one block per run: energy histogram -> Q' over the fixed
 //              32-lane tree, ln Q and the staged -beta F~ (Eqs. (2), (4)),
-//              per-bin Poisson means (Eq. (1)), Metropolis thresholds.
-//   k_copies   one thread per replica: Poisson copy count (inverse CDF,
-//              means above 32 split into pieces), per-chunk sums.
+//              per-bin Poisson means (Eq. (1)), Metropolis thresholds
+//              (Gaussian runs: k_gprep_head, k_gweights, k_gprep_tail).
+//   k_copies   one block per 256 replicas: Poisson copy counts (inverse CDF,
+//              means above 32 split into pieces; long walks shared out over the
+//              block), per-chunk sums.
 //   k_scan     one block per run: exclusive scan of the chunk sums, R~',
 //              capacity / extinction check.
-//   k_scatter  one thread per replica: source slot of every new slot.
-//   k_sweep*   fused copy + sweeps + measurement (pa_sweep*.cu).
-//   k_commit   one thread per run: commit the step or leave it untouched.
+//   k_scatter  one block per 256 replicas: source slot of every new slot, the
+//              new slots taken in turn.
+//   k_resample one block per run of at most SMALL_RUN slots (+-1 couplings): the
+//              four above in one launch.
+//   k_sweep*   fused copy + sweeps + measurement (pa_sweep*.cu, pa_gauss*.cu*,
+//              pa_box*.cu*).
+//   k_commit   one thread per run: commit the step or leave it untouched.  In a
+//              schedule of small runs k_resample of the next step does this, and
+//              k_commit follows the last step only.
 #include <math.h>
 
 #include "pa_dexp.cuh"
@@ -171,7 +179,7 @@ __global__ void k_init_finish(RunDev* __restrict__ runs, const int32_t* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Step: Q, ln Q, -beta F~, Poisson tables, thresholds (one warp per run)
+// Step: Q, ln Q, -beta F~, Poisson tables, thresholds (one block per run)
 // ---------------------------------------------------------------------------
 constexpr int PREP_THREADS = 256;
 constexpr int PREP_WIN = 2048;  // bins of one shared-memory window of the Q' sum
@@ -787,7 +795,7 @@ cudaError_t launch_overlap_pairs(const RunDev* runs, const int32_t* ra, const in
 }
 
 // ---------------------------------------------------------------------------
-// Sec. 3 weighted averages: one warp per group of M runs.
+// Sec. 3 weighted averages: a warp or a block per group of M runs.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
