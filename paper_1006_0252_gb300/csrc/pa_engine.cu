@@ -611,8 +611,9 @@ void set_default_launch(LatticeClass& c, int tpb_opt, int split_opt, const std::
   if (tpb_opt && tpb_supported(c, tpb_opt) && (tpb_opt < 512 || table)) c.tpb = tpb_opt;
   else if (c.bx > 0) c.tpb = std::min(64, c.max_tpb);
   else if (table) c.tpb = 1024;
-  else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * c.sms ? 256 : 128;  // 5 threads a replica: 25 or 51 of
-                                                                               // them a block
+  // L = 10: 5 threads a replica, 25 of them or 51 a block; 12 steps, us, at 128 / 256 threads:
+  // 2000 replicas 1259 / 1478, 9000 1857 / 2198, 20000 3074 / 3016, 30000 4197 / 3460, 60000 6240 / 6256
+  else if (pm_cubic(c)) c.tpb = c.L == 10 && replicas > 51 * c.sms ? 256 : 128;
   else if (c.split > 1) c.tpb = 128;
   else c.tpb = default_tpb(c.dim, c.L);
   if (c.tpb / c.split < 4 || (c.split > 1 && c.tpb < 64)) c.split = 1;
